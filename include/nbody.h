@@ -206,9 +206,9 @@ int nbody_get_launch(nbody_ctx *ctx, int *ipt, int *jsplit, int *threads, int *t
  * particles (Newton's third law; the same terms with opposite signs, summed in
  * a different fixed order than the one-sided kernels, so results differ from
  * them by rounding only and stay deterministic).  Particles are cut into
- * blocks of 384 (FP64) or 256 (F64E).  mode = -1 (default): automatic, used
- * when n spans at least 64 blocks; 0: never; 1: whenever n spans at least 2
- * blocks.  The launch shape of nbody_set_launch does not apply to this path.
+ * blocks of 256 (FP64 with eps = 0: 384).  mode = -1 (default): automatic, used
+ * when n spans at least 64 blocks of 384 (FP64) or 256 (F64E); 0: never; 1:
+ * whenever n spans at least 2 blocks.  The launch shape of nbody_set_launch does not apply to this path.
  * Memory: the first force evaluation on this path allocates the context's
  * per-diagonal row and column buffers (2 x D x n x 32 bytes, at most 1 GiB;
  * D = 8 at n = 2^20 in FP64) and P + 2 slices of partial sums (P <= 4);

@@ -165,14 +165,15 @@ static int ensure_part(nbody_ctx *c, int S) {
 // The force kernels' output slices for this evaluation.
 static void *force_out(const nbody_ctx *c) { return c->order ? c->part_alt : c->part; }
 
-// Blocks (of sym_block_particles()) below which the automatic choice keeps
-// the one-sided kernel: with few blocks the diagonals hold too few work items
-// to fill the GPU (measured on GB300 with blocks of 512: 43.6 against 55.9
-// Gint/s at 32 blocks, N = 2^14; 68.5 against 56.6 at 64 blocks, N = 2^15).
-static const int SYM_AUTO_MIN_BLOCKS = 64;
+// Smallest n at which the automatic choice evaluates each pair once: 64 blocks
+// of 256 (F64E), and 64 blocks of 384 in FP64 whatever its block size.  With
+// few blocks the diagonals hold too few work items to fill the GPU (measured
+// on GB300 with blocks of 512: 43.6 against 55.9 Gint/s at 32 blocks, N = 2^14;
+// 68.5 against 56.6 at 64 blocks, N = 2^15).
+static int64_t sym_auto_min_n(int mode) { return mode == NBODY_F64E ? 63 * 256 + 1 : 63 * 384 + 1; }
 
 static int sym_block(const nbody_ctx *c) {
-  return c->mode == NBODY_F64E ? nb::sym_block_particles_ff() : nb::sym_block_particles();
+  return c->mode == NBODY_F64E ? nb::sym_block_particles_ff() : nb::sym_block_particles(c->eps * c->eps);
 }
 
 static int sym_blocks(const nbody_ctx *c) {
@@ -182,7 +183,7 @@ static int sym_blocks(const nbody_ctx *c) {
 
 static bool use_sym(const nbody_ctx *c) {
   if ((c->mode != NBODY_FP64 && c->mode != NBODY_F64E) || c->sym == 0) return false;
-  return c->sym == 1 ? sym_blocks(c) >= 2 : sym_blocks(c) >= SYM_AUTO_MIN_BLOCKS;
+  return c->sym == 1 ? sym_blocks(c) >= 2 : c->n >= sym_auto_min_n(c->mode);
 }
 
 // FP64 and F64E, each pair once: slices 0..P-1 of c->part = pairs inside each
@@ -198,7 +199,7 @@ static int force_sym(nbody_ctx *c, const void *posm_in, int &S) {
   // pairs inside the diagonal blocks: each block's j range in P parts (one
   // unit each, partial sums in slices 0..P-1) so that the one-sided launch has
   // at least two work items per resident block slot
-  const int ur = ff ? nb::sym_r_ff() : nb::sym_units_r();  // one-sided R covering a block
+  const int ur = ff ? nb::sym_r_ff() : nb::sym_units_r(c->eps * c->eps);  // one-sided R covering a block
   const int per_sm_1 = nb::force_max_blocks_per_sm(c->mode, nb::Shape{nb::force_block_threads(c->mode),
                                                                       ur, nb::force_tile(c->mode), 1});
   const int64_t slots_1 = (int64_t)c->num_sms * std::max(1, per_sm_1);
@@ -233,7 +234,7 @@ static int force_sym(nbody_ctx *c, const void *posm_in, int &S) {
   }
   if (!c->sym_d && nd > 0) {
     // enough work items per launch for ~32 waves, within 1 GiB of buffers
-    const int per_sm = ff ? nb::sym_blocks_per_sm_ff() : nb::sym_blocks_per_sm();
+    const int per_sm = ff ? nb::sym_blocks_per_sm_ff() : nb::sym_blocks_per_sm(c->eps * c->eps);
     const int64_t slots = (int64_t)c->num_sms * std::max(1, per_sm);
     int64_t D = (32 * slots + M - 1) / M;
     const int64_t cap = std::max<int64_t>(1, ((int64_t)1 << 30) / (64 * c->n));

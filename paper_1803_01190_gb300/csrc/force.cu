@@ -16,15 +16,19 @@
 // G and the update of the integrator.
 //
 // Four arithmetics:
-//   f64   binary64 pair arithmetic.  GB300 issues binary64 at about 1/72 of the
-//         binary32 rate, so the kernel is bound by the FP64 pipe and its cost
-//         is its count of FP64 instructions per pair: 9 (3 DADD for d,
-//         3 DFMA for |d|^2 + eps^2, 3 DFMA for the acceleration sums).  The
-//         rest runs on the otherwise idle integer and FP32 pipes: 1/r and
-//         1/r^2 within 0.52 ulp (SFU seed, exact integer residual), the
-//         products m/r and (m/r)/r^2 by a correctly rounded integer binary64
-//         multiply, and the potential sum by a correctly rounded integer
-//         binary64 add.  From 64 blocks of 384 particles the FP64 path
+//   f64   binary64.  GB300 issues binary64 at about 1/72 of the binary32
+//         rate, one FP64 instruction in the time of 32 integer ones, so the
+//         one-sided kernel sums softened pairs in 64-bit fixed point on the
+//         integer pipes (fixed.cuh), with less rounding than binary64 pair
+//         terms have.  Where that does not apply (eps = 0, masses of one tile
+//         over more than 2^6, close pairs in a wide tile) it takes the
+//         binary64 body, bound by the FP64 pipe with 9 FP64 instructions per
+//         pair (3 DADD for d, 3 DFMA for |d|^2 + eps^2, 3 DFMA for the
+//         acceleration sums); the rest of that body runs on the integer and
+//         FP32 pipes: 1/r and 1/r^2 within 0.52 ulp (SFU seed, exact integer
+//         residual), the products m/r and (m/r)/r^2 by a correctly rounded
+//         integer binary64 multiply, and the potential sum by a correctly
+//         rounded integer binary64 add.  From 64 blocks of 384 particles the FP64 path
 //         evaluates each pair once for both particles (k_force_f64_sym:
 //         12 FP64 instructions per pair, 6 per interaction).
 //   mixed binary32 pair arithmetic (packed: two j per instruction, SFU
@@ -48,6 +52,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "fixed.cuh"
 #include "nbody_internal.cuh"
 
 namespace nb {
@@ -221,19 +226,26 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float b) {
 // A kernel runs units k = first(), first() + stride(), ... < count().
 // Dense: one system of n particles; block (x, y) = i-block x of the rows
 // [i_base, i_base + rows) against j-segment y of all n; the row sums go to
-// part[y * rows + (i - i_base)] (all rows: i_base = 0, rows = n).
+// part[y * rows + (i - i_base)] (all rows: i_base = 0, rows = n).  aligned:
+// i-blocks start at multiples of per_block whatever i_base is (the binary64
+// kernel's unit depends on the particles of the whole i-block, so a row's sum
+// is the same, bit for bit, whichever rows are asked for); only the rows
+// asked for are written.
 struct DenseWork {
   int64_t n, seg, i_base, rows;
   double eps2;
   int per_block, tile;
+  bool aligned;
   __device__ __forceinline__ int64_t first() const { return 0; }
   __device__ __forceinline__ int64_t stride() const { return 1; }
   __device__ __forceinline__ int64_t count() const { return 1; }
   __device__ __forceinline__ Unit get(int64_t) const {
     Unit u;
-    const int64_t r0 = (int64_t)blockIdx.x * per_block;
+    const int64_t r0 = (int64_t)blockIdx.x * per_block - (aligned ? i_base % per_block : 0);
     u.i0 = i_base + r0;
-    u.ni = (int)min((int64_t)per_block, rows - r0);
+    u.ni = (int)min((int64_t)per_block, (aligned ? n - i_base : rows) - r0);
+    u.w0 = (int)max((int64_t)0, -r0);
+    u.w1 = (int)min((int64_t)u.ni, rows - r0);
     u.j0 = (int64_t)blockIdx.y * seg;
     u.nj = (int)min(seg, n - u.j0);
     u.out = (int64_t)blockIdx.y * rows + r0;
@@ -290,67 +302,329 @@ __device__ __forceinline__ void body_f64(const d4 &pj, double xi, double yi, dou
   acc_pos(pt, my);  // the potential sum: integer pipes
 }
 
-template <int BT, int R, int T, class W>
+// One pair of the binary64 body, out of line: (d_x, d_y, d_z) m / r^3 and m / r.
+__device__ __noinline__ d4 pair_f64(double dx, double dy, double dz, double m, double eps2) {
+  double ax = 0.0, ay = 0.0, az = 0.0;
+  uint64_t pt = 0;
+  body_f64<false>(d4{dx, dy, dz, m}, 0.0, 0.0, 0.0, eps2, ax, ay, az, pt, false);
+  return d4{ax, ay, az, __longlong_as_double((long long)pt)};
+}
+
+// ---------------------------------------------------------------- fixed point: tile scale
+// Enclosing box of a set of particles from the high words of their coordinates
+// (order-preserving signed keys), their largest mass and smallest positive
+// mass (high words); mmin = -1 marks a non-finite value or a negative mass.
+struct FxBox {
+  int lo[3], hi[3], mmax, mmin;
+};
+__device__ __forceinline__ int fx_key(int hi) { return hi ^ ((hi >> 31) & 0x7FFFFFFF); }
+__device__ __forceinline__ void fx_box_init(FxBox &b) {
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    b.lo[c] = 0x7FFFFFFF;
+    b.hi[c] = (int)0x80000000;
+  }
+  b.mmax = 0;
+  b.mmin = 0x7FFFFFFF;
+}
+__device__ __forceinline__ void fx_box_add(FxBox &b, const d4 &p) {
+  const int h[4] = {__double2hiint(p.x), __double2hiint(p.y), __double2hiint(p.z),
+                    __double2hiint(p.w)};
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    b.lo[c] = min(b.lo[c], fx_key(h[c]));
+    b.hi[c] = max(b.hi[c], fx_key(h[c]));
+  }
+  bool bad = h[3] < 0;
+#pragma unroll
+  for (int c = 0; c < 4; c++) bad |= (h[c] & 0x7FF00000) == 0x7FF00000;
+  b.mmax = max(b.mmax, h[3]);
+  b.mmin = min(b.mmin, bad ? -1 : p.w > 0.0 ? h[3] : 0x7FFFFFFF);
+}
+__device__ __forceinline__ void fx_box_warp(FxBox &b) {
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    b.lo[c] = __reduce_min_sync(0xFFFFFFFFu, b.lo[c]);
+    b.hi[c] = __reduce_max_sync(0xFFFFFFFFu, b.hi[c]);
+  }
+  b.mmax = __reduce_max_sync(0xFFFFFFFFu, b.mmax);
+  b.mmin = __reduce_min_sync(0xFFFFFFFFu, b.mmin);
+}
+__device__ __forceinline__ void fx_box_join(FxBox &b, const FxBox &o) {
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    b.lo[c] = min(b.lo[c], o.lo[c]);
+    b.hi[c] = max(b.hi[c], o.hi[c]);
+  }
+  b.mmax = max(b.mmax, o.mmax);
+  b.mmin = min(b.mmin, o.mmin);
+}
+
+// Unit exponent L and mass exponent em for the i's of box bi against the j's
+// of box bj; ok = false: the fixed-point form does not apply (non-finite
+// values, negative masses, positive masses over a range above
+// 2^FX_MASS_RANGE, extreme exponents, or eps = 0).  eps = 0 stays in
+// binary64: there every pair term is specified to the ulp of the binary64
+// operations.  wide: the masses need exponents of their own.
+struct FxScale {
+  int L, em;
+  bool ok, wide;
+};
+// em of a box's masses; false: outside the rule above
+__device__ __forceinline__ bool fx_mass_scale(const FxBox &b, int &em, bool &wide) {
+  const int ex = b.mmax >> 20;
+  em = b.mmax == 0 ? 0 : ex - 1023;
+  wide = b.mmax != 0 && (b.mmin >> 20) < ex - FX_MASS_NARROW;
+  return b.mmin >= 0 &&
+         (b.mmax == 0 || (ex > 623 && ex < 1423 && (b.mmin >> 20) >= ex - FX_MASS_RANGE));
+}
+__device__ __forceinline__ FxScale fx_scale(const FxBox &bi, const FxBox &bj, double eps2) {
+  int top = ((__double2hiint(eps2) >> 20) - 1021) >> 1;  // eps < 2^top
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    // bounds of the coordinate: the low words of the keys are unknown
+    const int l = fx_key(min(bi.lo[c], bj.lo[c])), h = fx_key(max(bi.hi[c], bj.hi[c]));
+    const double lo = __hiloint2double(l, l < 0 ? -1 : 0), hi = __hiloint2double(h, h < 0 ? 0 : -1);
+    top = max(top, (__double2hiint(hi - lo) >> 20) - 1022);  // hi - lo < 2^top
+  }
+  FxScale f;
+  f.L = top - FX_BITS;
+  const bool m = fx_mass_scale(bj, f.em, f.wide);
+  f.ok = m && eps2 > 0.0 && bi.mmin >= 0 && top > -200 && top < 200;
+  return f;
+}
+__device__ __forceinline__ double fx_exp2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+// acc + a 2^e, a the accumulator, scale = 2^(e + 32)
+__device__ __forceinline__ double fx_fold(double acc, const fx96 &a, double scale) {
+  const double v = fma((double)a.w0, 0x1p-32, fma((double)a.w2, 0x1p32, (double)a.w1));
+  return fma(v, scale, acc);
+}
+__device__ __forceinline__ void fx_coords(const d4 &p, int L, uint64_t (&X)[3]) {
+  X[0] = fx_coord((uint32_t)__double2hiint(p.x), (uint32_t)__double2loint(p.x), L);
+  X[1] = fx_coord((uint32_t)__double2hiint(p.y), (uint32_t)__double2loint(p.y), L);
+  X[2] = fx_coord((uint32_t)__double2hiint(p.z), (uint32_t)__double2loint(p.z), L);
+}
+struct FxRsqrt {
+  __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
+    return __float_as_uint(rsqrt_approx(__uint2float_rn(x)));
+  }
+};
+
+// How the masses of a tile enter (fixed.cuh): all equal, one exponent, or an
+// exponent each.
+enum FxMode { FX_EQUAL, FX_NARROW, FX_WIDE };
+
+// The fixed-point sum of RI i-particles against the tile entries [k0, k1).
+// self(r, k): the pair of particle r with itself (looked at in FX_WIDE
+// only, which the tiles that hold the block's own particles take);
+// close(r, k): adds a pair too close for the tile's unit in binary64.
+template <int RI, FxMode MODE, class Self, class Close>
+__device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, const int *tdm, int k0,
+                                        int k1, const FxEps &e2, const uint64_t (&Xi)[RI][3],
+                                        fx96 (&f)[RI][3], fx96 (&pt)[RI], Self self, Close close) {
+#pragma unroll 1
+  for (int k = k0; k < k1; k++) {
+    const uint4 a = txy[k], b = tzm[k];
+    const uint64_t Xj[3] = {((uint64_t)a.y << 32) | a.x, ((uint64_t)a.w << 32) | a.z,
+                            ((uint64_t)b.y << 32) | b.x};
+    const int dm = MODE == FX_WIDE ? tdm[k] : 0;
+#pragma unroll
+    for (int r = 0; r < RI; r++) {
+      const bool s = MODE == FX_WIDE && self(r, k);
+      FxPair p;
+      if (!fx_geometry(Xj, Xi[r], e2, FxRsqrt(), p)) {
+        if (!s) close(r, k);
+      } else if (MODE == FX_EQUAL) {
+        fx_both(p, f[r], pt[r], nullptr, nullptr);
+      } else {
+        fx_side<MODE == FX_WIDE>(p, FxMass{s ? 0u : b.w, s ? 0u : b.z, dm}, f[r], pt[r]);
+      }
+    }
+  }
+}
+
+// The binary64 force sum, bound by the FMA-heavy pipe (the wide integer
+// multiplies of fixed.cuh; 89 % busy by ncu at N = 16384), not by the FP64
+// pipe.  Measured on GB300 (force kernel alone, disk + halo of equal masses,
+// N = 65536): 131 Gint/s at R = 1, 127 at R = 2 (122 for unequal masses)
+// against 62 for the binary64 body with its 9 FP64 instructions; the relative
+// error of the accelerations against binary64 terms with pairwise sums falls
+// from 4.5e-16 to 1.9e-16 (it is the rounding of the tile sums).  R above 2
+// runs in groups of two.
+//
+// IW warps of a block share the same i-particles and split each j-tile (IW =
+// 1: BT * R i-particles per block; IW = 4, for small n: BT / 4 * R, four times
+// as many blocks and a quarter of the sequential pairs per thread).  Each tile
+// is summed in fixed point where fx_scale allows it and in binary64 otherwise;
+// pairs too close for the tile's unit go through pair_f64.  i-particles are
+// taken two at a time (RI), whatever R is.
+template <int BT, int R, int T, int IW, class W>
 __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W work,
                                                   d4 *__restrict__ part) {
+  static_assert(T == BT, "one j per thread");
+  constexpr int NW = BT / 32, RI = R < 2 ? R : 2, NG = R / RI, IT = BT / IW;
   __shared__ d4 tile[T];
+  __shared__ uint4 txy[T], tzm[T];
+  __shared__ int tdm[T];
+  __shared__ FxBox sbox[NW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int it = tid % IT, jw = tid / IT;  // i-thread, share of the j-tile
   for (int64_t uk = work.first(); uk < work.count(); uk += work.stride()) {
     const Unit u = work.get(uk);
-    const int tid = threadIdx.x;
     const int64_t j1 = u.j0 + u.nj;
     const double eps2 = u.eps2;
-    double xi[R], yi[R], zi[R], ax[R], ay[R], az[R];
-    uint64_t pt[R];  // bit patterns of the potential sums
-  #pragma unroll
-    for (int r = 0; r < R; r++) {
-      const int li = r * BT + tid;
-      const d4 p = posm[u.i0 + (li < u.ni ? li : 0)];
-      xi[r] = p.x;
-      yi[r] = p.y;
-      zi[r] = p.z;
-      ax[r] = ay[r] = az[r] = 0.0;
-      pt[r] = 0;
-    }
+    d4 acc[NG][RI];
+    FxBox bi;
+    fx_box_init(bi);
+    for (int g = 0; g < NG; g++)
+#pragma unroll
+      for (int r = 0; r < RI; r++) {
+        const int li = (g * RI + r) * IT + it;
+        fx_box_add(bi, posm[u.i0 + (li < u.ni ? li : 0)]);
+        acc[g][r] = d4{0.0, 0.0, 0.0, 0.0};
+      }
+    fx_box_warp(bi);
+    __syncthreads();
+    if (lane == 0) sbox[warp] = bi;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NW; w++) fx_box_join(bi, sbox[w]);
     for (int64_t jt = u.j0; jt < j1; jt += T) {
       const int cnt = (int)min((int64_t)T, j1 - jt);
       __syncthreads();
-      for (int k = tid; k < cnt; k += BT) tile[k] = posm[jt + k];
+      d4 pj = d4{0.0, 0.0, 0.0, 0.0};
+      FxBox bj;
+      fx_box_init(bj);
+      if (tid < cnt) {
+        pj = posm[jt + tid];
+        tile[tid] = pj;
+        fx_box_add(bj, pj);
+      }
+      fx_box_warp(bj);
+      if (lane == 0) sbox[warp] = bj;
       __syncthreads();
+#pragma unroll
+      for (int w = 0; w < NW; w++) fx_box_join(bj, sbox[w]);
+      const FxScale sc = fx_scale(bi, bj, eps2);
+      const int k0 = cnt * jw / IW, k1 = cnt * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      if (cnt == T && !diag) {
-  #pragma unroll 2
-        for (int k = 0; k < T; k++) {
-          const d4 pj = tile[k];
-  #pragma unroll
-          for (int r = 0; r < R; r++)
-            body_f64<false>(pj, xi[r], yi[r], zi[r], eps2, ax[r], ay[r], az[r], pt[r], false);
+      if (sc.ok) {
+        {
+          uint64_t X[3];
+          fx_coords(pj, sc.L, X);
+          const uint32_t mh = (uint32_t)__double2hiint(pj.w), ml = (uint32_t)__double2loint(pj.w);
+          const FxMass M = sc.wide ? fx_mass<true>(mh, ml, sc.em) : fx_mass<false>(mh, ml, sc.em);
+          txy[tid] = make_uint4((uint32_t)X[0], (uint32_t)(X[0] >> 32), (uint32_t)X[1],
+                                (uint32_t)(X[1] >> 32));
+          tzm[tid] = make_uint4((uint32_t)X[2], (uint32_t)(X[2] >> 32), M.l, M.h);
+          tdm[tid] = M.dm;
         }
-      } else if (cnt == T) {  // a full tile that holds some of this block's own i
-  #pragma unroll 2
-        for (int k = 0; k < T; k++) {
-          const d4 pj = tile[k];
-          const int64_t j = jt + k;
-  #pragma unroll
-          for (int r = 0; r < R; r++)
-            body_f64<true>(pj, xi[r], yi[r], zi[r], eps2, ax[r], ay[r], az[r], pt[r],
-                           j == u.i0 + r * BT + tid);
+        const double m0 = tile[0].w;
+        const bool equal = __syncthreads_and(
+            __double_as_longlong(pj.w) == __double_as_longlong(m0) || tid >= cnt);
+        const FxMode mode = diag || sc.wide ? FX_WIDE : equal ? FX_EQUAL : FX_NARROW;
+        const int em = mode == FX_EQUAL ? FX_EQ_EM : sc.em;
+        const FxEps e2 = fx_eps2(eps2, sc.L);
+        double fs = fx_exp2(fx_force_exp(sc.L, em) + 32), ps = fx_exp2(fx_pot_exp(sc.L, em) + 32);
+        if (mode == FX_EQUAL) {
+          fs *= m0;
+          ps *= m0;
+        }
+        for (int g = 0; g < NG; g++) {
+          uint64_t Xi[RI][3];
+          fx96 f[RI][3] = {}, pt[RI] = {};
+#pragma unroll
+          for (int r = 0; r < RI; r++) {
+            const int li = (g * RI + r) * IT + it;
+            fx_coords(posm[u.i0 + (li < u.ni ? li : 0)], sc.L, Xi[r]);
+          }
+          const int ii = (int)(u.i0 - jt) + g * RI * IT + it;  // tile entry of particle 0
+          auto self = [&](int r, int k) { return diag && k == ii + r * IT; };
+          auto close = [&](int r, int k) {
+            const int li = (g * RI + r) * IT + it;
+            const d4 pi = posm[u.i0 + (li < u.ni ? li : 0)], q = tile[k];
+            const d4 v = pair_f64(q.x - pi.x, q.y - pi.y, q.z - pi.z, q.w, eps2);
+            acc[g][r].x += v.x;
+            acc[g][r].y += v.y;
+            acc[g][r].z += v.z;
+            acc[g][r].w += v.w;
+          };
+          if (mode == FX_WIDE)
+            fx_tile<RI, FX_WIDE>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+          else if (mode == FX_EQUAL)
+            fx_tile<RI, FX_EQUAL>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+          else
+            fx_tile<RI, FX_NARROW>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+#pragma unroll
+          for (int r = 0; r < RI; r++) {
+            acc[g][r].x = fx_fold(acc[g][r].x, f[r][0], fs);
+            acc[g][r].y = fx_fold(acc[g][r].y, f[r][1], fs);
+            acc[g][r].z = fx_fold(acc[g][r].z, f[r][2], fs);
+            acc[g][r].w = fx_fold(acc[g][r].w, pt[r], ps);
+          }
         }
       } else {
-        for (int k = 0; k < cnt; k++) {
-          const d4 pj = tile[k];
-          const int64_t j = jt + k;
-  #pragma unroll
-          for (int r = 0; r < R; r++)
-            body_f64<true>(pj, xi[r], yi[r], zi[r], eps2, ax[r], ay[r], az[r], pt[r],
-                           j == u.i0 + r * BT + tid);
+        for (int g = 0; g < NG; g++) {
+          d4 pi[RI];
+          uint64_t pt[RI];  // bit patterns of the potential sums
+#pragma unroll
+          for (int r = 0; r < RI; r++) {
+            const int li = (g * RI + r) * IT + it;
+            pi[r] = posm[u.i0 + (li < u.ni ? li : 0)];
+            pt[r] = (uint64_t)__double_as_longlong(acc[g][r].w);
+          }
+          if (!diag) {
+#pragma unroll 2
+            for (int k = k0; k < k1; k++) {
+              const d4 q = tile[k];
+#pragma unroll
+              for (int r = 0; r < RI; r++)
+                body_f64<false>(q, pi[r].x, pi[r].y, pi[r].z, eps2, acc[g][r].x, acc[g][r].y,
+                                acc[g][r].z, pt[r], false);
+            }
+          } else {
+            for (int k = k0; k < k1; k++) {
+              const d4 q = tile[k];
+#pragma unroll
+              for (int r = 0; r < RI; r++)
+                body_f64<true>(q, pi[r].x, pi[r].y, pi[r].z, eps2, acc[g][r].x, acc[g][r].y,
+                               acc[g][r].z, pt[r], jt + k == u.i0 + (g * RI + r) * IT + it);
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < RI; r++) acc[g][r].w = __longlong_as_double((long long)pt[r]);
         }
       }
     }
-  #pragma unroll
-    for (int r = 0; r < R; r++) {
-      const int li = r * BT + tid;
-      if (li < u.ni)
-        part[u.out + li] = d4{ax[r], ay[r], az[r], __longlong_as_double((long long)pt[r])};
+    const int w1 = min(u.ni, u.w1);
+    if (IW == 1) {
+      for (int g = 0; g < NG; g++)
+#pragma unroll
+        for (int r = 0; r < RI; r++) {
+          const int li = (g * RI + r) * IT + it;
+          if (li >= u.w0 && li < w1) part[u.out + li] = acc[g][r];
+        }
+    } else {  // the shares of the j-tiles, added in order
+      for (int g = 0; g < NG; g++)
+#pragma unroll
+        for (int r = 0; r < RI; r++) {
+          __syncthreads();
+          tile[tid] = acc[g][r];
+          __syncthreads();
+          const int li = (g * RI + r) * IT + it;
+          if (jw == 0 && li >= u.w0 && li < w1) {
+            d4 s = tile[it];
+#pragma unroll
+            for (int w = 1; w < IW; w++) {
+              const d4 v = tile[w * IT + it];
+              s.x += v.x;
+              s.y += v.y;
+              s.z += v.z;
+              s.w += v.w;
+            }
+            part[u.out + li] = s;
+          }
+        }
     }
   }
 }
@@ -534,8 +808,234 @@ __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ pos
   }
 }
 
+// ---------------------------------------------------------------- fixed point, each pair once
+// The work items, row and column slices of k_force_f64_sym with the pair
+// arithmetic of fixed.cuh: the geometry of a pair (d, 1/r, 1/r^2: 20 of the 38
+// wide multiplies of one side) serves both particles.  Sums of a tile are
+// 96-bit integers in registers; the column sums of a chunk of 32 j travel
+// around the lanes (12 words per step).  Pairs too close for the unit, and
+// every pair of an item that fx_scale does not take, are evaluated in
+// binary64 out of line and added in binary64 (rows in registers, columns in
+// the warp's slots of colw, where a lane owns its j at each step).  Measured
+// (whole force evaluation, N = 65536): 215-219 Gint/s for equal masses, where
+// the two sides share their terms, 147 for lognormal masses, against 93 for
+// k_force_f64_sym; relative error of the accelerations 1.6e-16 against 2.6e-16.
+// Four blocks of 128 per SM (128 registers, R = 2): 202 at 166 registers and
+// three blocks, 214 at R = 1, 175 at R = 3.
+template <int BT, int R, int T, FxMode MODE>
+__device__ __forceinline__ void fx_sym_tile(const d4 *__restrict__ posm, int64_t n, int64_t i0,
+                                            double eps2, bool ok, const FxEps &e2,
+                                            const d4 *tile, const uint4 *txy, const uint4 *tzm,
+                                            const int *tdm, int cnt, const uint64_t (&Xi)[R][3],
+                                            const FxMass (&Mi)[R], d4 (&acc)[R], double fs,
+                                            double ps, double gs, double qs, d4 *colw) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  fx96 f[R][3] = {}, pt[R] = {};
+#pragma unroll 1
+  for (int c = 0; c < T; c += 32) {
+    if (c >= cnt) break;
+    fx96 g[3] = {}, gp = {};
+#pragma unroll 1
+    for (int k = 0; k < 32; k++) {
+      const int jj = c + ((lane + k) & 31);
+      const uint4 a = txy[jj], b = tzm[jj];
+      const uint64_t Xj[3] = {((uint64_t)a.y << 32) | a.x, ((uint64_t)a.w << 32) | a.z,
+                              ((uint64_t)b.y << 32) | b.x};
+      const FxMass Mj{b.w, b.z, MODE == FX_WIDE ? tdm[jj] : 0};
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        FxPair p;
+        if (ok && fx_geometry(Xj, Xi[r], e2, FxRsqrt(), p)) {
+          if (MODE == FX_EQUAL) {
+            fx_both(p, f[r], pt[r], &g, &gp);
+          } else {
+            fx_side<MODE == FX_WIDE>(p, Mj, f[r], pt[r]);
+            fx_side<MODE == FX_WIDE>(p, Mi[r], g, gp);
+          }
+        } else {
+          const int64_t i = i0 + r * BT + tid;
+          if (jj < cnt && i < n) {
+            const d4 pi = posm[i], q = tile[jj];
+            const double dx = q.x - pi.x, dy = q.y - pi.y, dz = q.z - pi.z;
+            const d4 v = pair_f64(dx, dy, dz, q.w, eps2);
+            acc[r].x += v.x;
+            acc[r].y += v.y;
+            acc[r].z += v.z;
+            acc[r].w += v.w;
+            const d4 w = pair_f64(-dx, -dy, -dz, pi.w, eps2);
+            colw[jj].x += w.x;
+            colw[jj].y += w.y;
+            colw[jj].z += w.z;
+            colw[jj].w += w.w;
+          }
+        }
+      }
+      __syncwarp();  // the slots of colw change hands
+      const int src = (lane + 1) & 31;
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        g[q].w0 = __shfl_sync(0xFFFFFFFFu, g[q].w0, src);
+        g[q].w1 = __shfl_sync(0xFFFFFFFFu, g[q].w1, src);
+        g[q].w2 = __shfl_sync(0xFFFFFFFFu, g[q].w2, src);
+      }
+      gp.w0 = __shfl_sync(0xFFFFFFFFu, gp.w0, src);
+      gp.w1 = __shfl_sync(0xFFFFFFFFu, gp.w1, src);
+      gp.w2 = __shfl_sync(0xFFFFFFFFu, gp.w2, src);
+    }
+    d4 s = colw[c + lane];
+    s.x = fx_fold(s.x, g[0], -gs);
+    s.y = fx_fold(s.y, g[1], -gs);
+    s.z = fx_fold(s.z, g[2], -gs);
+    s.w = fx_fold(s.w, gp, qs);
+    colw[c + lane] = s;
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    acc[r].x = fx_fold(acc[r].x, f[r][0], fs);
+    acc[r].y = fx_fold(acc[r].y, f[r][1], fs);
+    acc[r].z = fx_fold(acc[r].z, f[r][2], fs);
+    acc[r].w = fx_fold(acc[r].w, pt[r], ps);
+  }
+}
+
+template <int BT, int R, int T>
+__global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ posm, int64_t n,
+                                                     double eps2, int M, int d0,
+                                                     d4 *__restrict__ rows,
+                                                     d4 *__restrict__ cols) {
+  constexpr int B = BT * R, NW = BT / 32;
+  static_assert(T == BT && B % T == 0, "one column sum per thread per tile");
+  __shared__ d4 tile[T];
+  __shared__ uint4 txy[T], tzm[T];
+  __shared__ int tdm[T];
+  __shared__ d4 colw[NW][T];
+  __shared__ FxBox sbox[NW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int dl = blockIdx.x / M, I = blockIdx.x % M, d = d0 + dl;
+  const int J = (I + d) % M;
+  const int64_t i0 = (int64_t)I * B, j0 = (int64_t)J * B;
+  d4 *rowo = rows + (int64_t)dl * n;
+  d4 *colo = cols + (int64_t)dl * n;
+  if (2 * d == M && I >= M / 2) {  // the pair of blocks is the item (I - M/2, I)
+    for (int k = tid; k < B; k += BT) {
+      if (i0 + k < n) rowo[i0 + k] = d4{0.0, 0.0, 0.0, 0.0};
+      if (j0 + k < n) colo[j0 + k] = d4{0.0, 0.0, 0.0, 0.0};
+    }
+    return;
+  }
+  // particles beyond n stand at the block's first one, without mass
+  d4 acc[R];
+  FxBox bi;
+  fx_box_init(bi);
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int64_t i = i0 + r * BT + tid;
+    fx_box_add(bi, posm[i < n ? i : i0]);
+    acc[r] = d4{0.0, 0.0, 0.0, 0.0};
+  }
+  fx_box_warp(bi);
+  if (lane == 0) sbox[warp] = bi;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NW; w++) fx_box_join(bi, sbox[w]);
+  int emi;
+  bool widei;
+  const bool oki = fx_mass_scale(bi, emi, widei);
+  const double mi0 = posm[i0].w;
+  bool equali = i0 + B <= n;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int64_t i = i0 + r * BT + tid;
+    equali = equali && __double_as_longlong(posm[i < n ? i : i0].w) == __double_as_longlong(mi0);
+  }
+  for (int t0 = 0; t0 < B && j0 + t0 < n; t0 += T) {
+    const int64_t jt = j0 + t0;
+    const int cnt = (int)min((int64_t)T, n - jt);
+    __syncthreads();
+    d4 pj = posm[jt + (tid < cnt ? tid : 0)];
+    FxBox bj;
+    fx_box_init(bj);
+    fx_box_add(bj, pj);
+    tile[tid] = pj;
+    if (tid >= cnt) pj.w = 0.0;
+    fx_box_warp(bj);
+    if (lane == 0) sbox[warp] = bj;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NW; w++) fx_box_join(bj, sbox[w]);
+    FxScale sc = fx_scale(bi, bj, eps2);
+    const bool ok = sc.ok && oki, wide = sc.wide || widei;
+    if (!ok) sc.L = sc.em = emi = 0;  // the integer sums stay zero
+    {
+      uint64_t X[3];
+      fx_coords(pj, sc.L, X);
+      const uint32_t mh = (uint32_t)__double2hiint(pj.w), ml = (uint32_t)__double2loint(pj.w);
+      const FxMass m = wide ? fx_mass<true>(mh, ml, sc.em) : fx_mass<false>(mh, ml, sc.em);
+      txy[tid] = make_uint4((uint32_t)X[0], (uint32_t)(X[0] >> 32), (uint32_t)X[1],
+                            (uint32_t)(X[1] >> 32));
+      tzm[tid] = make_uint4((uint32_t)X[2], (uint32_t)(X[2] >> 32), m.l, m.h);
+      tdm[tid] = m.dm;
+    }
+#pragma unroll
+    for (int w = 0; w < NW; w++) colw[w][tid] = d4{0.0, 0.0, 0.0, 0.0};
+    const double mj0 = tile[0].w;
+    const bool equal = __syncthreads_and(
+        equali && tid < cnt && __double_as_longlong(pj.w) == __double_as_longlong(mj0));
+    const FxMode mode = wide || !ok ? FX_WIDE : equal ? FX_EQUAL : FX_NARROW;
+    const FxEps e2 = fx_eps2(eps2, sc.L);
+    const int emr = mode == FX_EQUAL ? FX_EQ_EM : sc.em, emc = mode == FX_EQUAL ? FX_EQ_EM : emi;
+    double fs = fx_exp2(fx_force_exp(sc.L, emr) + 32), ps = fx_exp2(fx_pot_exp(sc.L, emr) + 32);
+    double gs = fx_exp2(fx_force_exp(sc.L, emc) + 32), qs = fx_exp2(fx_pot_exp(sc.L, emc) + 32);
+    if (mode == FX_EQUAL) {
+      fs *= mj0;
+      ps *= mj0;
+      gs *= mi0;
+      qs *= mi0;
+    }
+    uint64_t Xi[R][3];
+    FxMass Mi[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const int64_t i = i0 + r * BT + tid;
+      const d4 p = posm[i < n ? i : i0];
+      fx_coords(p, sc.L, Xi[r]);
+      const double m = i < n ? p.w : 0.0;
+      const uint32_t mh = (uint32_t)__double2hiint(m), ml = (uint32_t)__double2loint(m);
+      Mi[r] = wide ? fx_mass<true>(mh, ml, emi) : fx_mass<false>(mh, ml, emi);
+    }
+    if (mode == FX_WIDE)
+      fx_sym_tile<BT, R, T, FX_WIDE>(posm, n, i0, eps2, ok, e2, tile, txy, tzm, tdm, cnt, Xi, Mi,
+                                     acc, fs, ps, gs, qs, colw[warp]);
+    else if (mode == FX_EQUAL)
+      fx_sym_tile<BT, R, T, FX_EQUAL>(posm, n, i0, eps2, true, e2, tile, txy, tzm, tdm, cnt, Xi,
+                                      Mi, acc, fs, ps, gs, qs, colw[warp]);
+    else
+      fx_sym_tile<BT, R, T, FX_NARROW>(posm, n, i0, eps2, true, e2, tile, txy, tzm, tdm, cnt, Xi,
+                                       Mi, acc, fs, ps, gs, qs, colw[warp]);
+    __syncthreads();
+    {
+      d4 s = colw[0][tid];
+#pragma unroll
+      for (int w = 1; w < NW; w++) {
+        const d4 v = colw[w][tid];
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+      }
+      if (jt + tid < n) colo[jt + tid] = s;
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const int64_t i = i0 + r * BT + tid;
+    if (i < n) rowo[i] = acc[r];
+  }
+}
+
 // acc_rows[i] (+)= rows[0][i] + ... + rows[D-1][i], the same for the columns,
-// in diagonal order.
+// in diagonal order, in groups of eight (one after another the roundings of a
+// sum over hundreds of diagonals would exceed those of the pair sums).
 __global__ void k_sym_combine(const d4 *__restrict__ rows, const d4 *__restrict__ cols, int D,
                               int64_t n, d4 *__restrict__ acc_rows, d4 *__restrict__ acc_cols,
                               int first) {
@@ -543,16 +1043,27 @@ __global__ void k_sym_combine(const d4 *__restrict__ rows, const d4 *__restrict_
        i += (int64_t)gridDim.x * blockDim.x) {
     d4 a = first ? d4{0.0, 0.0, 0.0, 0.0} : acc_rows[i];
     d4 b = first ? d4{0.0, 0.0, 0.0, 0.0} : acc_cols[i];
-    for (int k = 0; k < D; k++) {
-      const d4 u = rows[(int64_t)k * n + i], v = cols[(int64_t)k * n + i];
-      a.x += u.x;
-      a.y += u.y;
-      a.z += u.z;
-      a.w += u.w;
-      b.x += v.x;
-      b.y += v.y;
-      b.z += v.z;
-      b.w += v.w;
+    for (int k0 = 0; k0 < D; k0 += 8) {
+      d4 c = {0.0, 0.0, 0.0, 0.0}, e = {0.0, 0.0, 0.0, 0.0};
+      for (int k = k0; k < min(k0 + 8, D); k++) {
+        const d4 u = rows[(int64_t)k * n + i], v = cols[(int64_t)k * n + i];
+        c.x += u.x;
+        c.y += u.y;
+        c.z += u.z;
+        c.w += u.w;
+        e.x += v.x;
+        e.y += v.y;
+        e.z += v.z;
+        e.w += v.w;
+      }
+      a.x += c.x;
+      a.y += c.y;
+      a.z += c.z;
+      a.w += c.w;
+      b.x += e.x;
+      b.y += e.y;
+      b.z += e.z;
+      b.w += e.w;
     }
     acc_rows[i] = a;
     acc_cols[i] = b;
@@ -1321,7 +1832,7 @@ bool shape_supported(int mode, const Shape &sh) {
 template <int R>
 static const void *kernel_for(int mode) {
   switch (mode) {
-    case NBODY_FP64: return (const void *)k_force_f64<BT_F64, R, T_F64, DenseWork>;
+    case NBODY_FP64: return (const void *)k_force_f64<BT_F64, R, T_F64, 1, DenseWork>;
     case NBODY_MIXED: return (const void *)k_force_mixed<BT_F32, R, T_F32, DenseWork>;
     case NBODY_F64E: return (const void *)k_force_f64e<BT_FF, (R < 4 ? R : 4), T_FF, DenseWork>;
     default: return (const void *)k_force_f32<BT_F32, R, T_F32, DenseWork>;
@@ -1349,7 +1860,7 @@ template <int R, class W>
 static void launch_rw(int mode, const void *posm, const float4 *fpos, const float4 *anchor,
                       const W &w, dim3 grid, void *part, cudaStream_t st) {
   if (mode == NBODY_FP64) {
-    k_force_f64<BT_F64, R, T_F64, W><<<grid, BT_F64, 0, st>>>((const d4 *)posm, w, (d4 *)part);
+    k_force_f64<BT_F64, R, T_F64, 1, W><<<grid, BT_F64, 0, st>>>((const d4 *)posm, w, (d4 *)part);
   } else if (mode == NBODY_MIXED) {
     k_force_mixed<BT_F32, R, T_F32, W><<<grid, BT_F32, 0, st>>>((const d4 *)posm, fpos, anchor, w,
                                                                 (d4 *)part);
@@ -1385,24 +1896,34 @@ static cudaError_t launch_w(int mode, int r, const void *posm, const float4 *fpo
 // pipes, k-loop not unrolled: R = 3 96.1, R = 2 96.3, R = 1 95.3 (unrolled twice:
 // R = 2 92.2).
 constexpr int SYM_BT = 128, SYM_R = 3, SYM_T = 128;
+// softened systems: fixed point
+constexpr int FXS_R = 2;
 
-int sym_block_particles() { return SYM_BT * SYM_R; }
-int sym_r() { return SYM_R; }
+static bool fx_sym(double eps2) { return eps2 > 0.0; }
+int sym_block_particles(double eps2) { return SYM_BT * (fx_sym(eps2) ? FXS_R : SYM_R); }
 // the one-sided kernel's R for the pairs inside the diagonal blocks: the
 // smallest supported R whose BT*R covers a block
-int sym_units_r() { return SYM_R <= 1 ? 1 : SYM_R <= 2 ? 2 : SYM_R <= 4 ? 4 : 8; }
+int sym_units_r(double eps2) {
+  const int r = fx_sym(eps2) ? FXS_R : SYM_R;
+  return r <= 1 ? 1 : r <= 2 ? 2 : r <= 4 ? 4 : 8;
+}
 
-int sym_blocks_per_sm() {
+int sym_blocks_per_sm(double eps2) {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force_f64_sym<SYM_BT, SYM_R, SYM_T>,
-                                                    SYM_BT, 0) != cudaSuccess)
-    return 0;
+  const void *k = fx_sym(eps2) ? (const void *)k_force_fx_sym<SYM_BT, FXS_R, SYM_T>
+                               : (const void *)k_force_f64_sym<SYM_BT, SYM_R, SYM_T>;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, SYM_BT, 0) != cudaSuccess) return 0;
   return nb;
 }
 
 cudaError_t launch_force_f64_sym(const d4 *posm, int64_t n, double eps2, int M, int d0, int D,
                                  d4 *rows, d4 *cols, cudaStream_t st) {
-  k_force_f64_sym<SYM_BT, SYM_R, SYM_T><<<D * M, SYM_BT, 0, st>>>(posm, n, eps2, M, d0, rows, cols);
+  if (fx_sym(eps2))
+    k_force_fx_sym<SYM_BT, FXS_R, SYM_T><<<D * M, SYM_BT, 0, st>>>(posm, n, eps2, M, d0, rows,
+                                                                   cols);
+  else
+    k_force_f64_sym<SYM_BT, SYM_R, SYM_T><<<D * M, SYM_BT, 0, st>>>(posm, n, eps2, M, d0, rows,
+                                                                    cols);
   return cudaGetLastError();
 }
 
@@ -1440,7 +1961,8 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   if (!shape_supported(mode, sh) || in.n < 1 || rows < 1 || in.i0 < 0 || in.i0 + rows > in.n)
     return cudaErrorInvalidValue;
   const int64_t per_block = (int64_t)sh.bt * sh.r;
-  const int64_t gx = (rows + per_block - 1) / per_block;
+  const bool aligned = mode == NBODY_FP64;
+  const int64_t gx = ((aligned ? in.i0 % per_block : 0) + rows + per_block - 1) / per_block;
   if (gx > 0x7fffffff) return cudaErrorInvalidValue;
   DenseWork w;
   w.n = in.n;
@@ -1450,6 +1972,7 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   w.eps2 = in.eps2;
   w.per_block = (int)per_block;
   w.tile = sh.t;
+  w.aligned = aligned;
   return launch_w(mode, sh.r, in.posm, in.fpos, in.anchor, w, dim3((unsigned)gx, (unsigned)sh.s),
                   in.part, st);
 }

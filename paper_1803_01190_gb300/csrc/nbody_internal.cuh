@@ -54,6 +54,7 @@ struct Unit {
   int64_t i0, j0, out, anchor;
   double eps2;
   int32_t ni, nj;
+  int32_t w0 = 0, w1 = 0x7FFFFFFF;  // FP64: only i0 + [w0, w1) is written
 };
 
 // One MIXED prep block: the tile [j0, j0+cnt) with anchor index `anchor`.
@@ -94,16 +95,16 @@ int force_tile(int mode);
 cudaError_t launch_mixed_prep(const d4 *posm, int64_t n, int tile, float4 *fpos, float4 *anchor,
                               cudaStream_t st, bool ff = false);
 int force_max_blocks_per_sm(int mode, const Shape &sh);
-// FP64, each pair once (Newton's third law): blocks of sym_block_particles()
-// particles (the one-sided kernel with R = sym_units_r() runs the pairs inside
+// FP64, each pair once (Newton's third law): blocks of
+// sym_block_particles(eps^2) particles (softened: fixed point, 256; eps = 0:
+// binary64, 384; the one-sided kernel with R = sym_units_r() runs the pairs inside
 // each block); launch D diagonals d0 .. d0+D-1 of the M x M block pairs, row
 // sums of diagonal d0+k into rows[k*n ..], column sums into cols[k*n ..];
 // launch_sym_combine adds them (in diagonal order) into acc_rows / acc_cols
 // (overwriting them when first).
-int sym_block_particles();
-int sym_r();
-int sym_units_r();
-int sym_blocks_per_sm();
+int sym_block_particles(double eps2);
+int sym_units_r(double eps2);
+int sym_blocks_per_sm(double eps2);
 cudaError_t launch_force_f64_sym(const d4 *posm, int64_t n, double eps2, int M, int d0, int D,
                                  d4 *rows, d4 *cols, cudaStream_t st);
 cudaError_t launch_sym_combine(const d4 *rows, const d4 *cols, int D, int64_t n, d4 *acc_rows,

@@ -1,0 +1,100 @@
+// Host check of the fixed-point pair arithmetic (csrc/fixed.cuh): random pairs
+// over its whole range (extents 2^-30 to 2^30, distances down to the close-pair
+// limit, offsets up to 2^15 extents, masses over the mass rule) against
+// extended precision.  Prints the largest errors in units of their bounds.
+//   force: 2^-55 (largest / mass) + 4 u / r;  potential: 2^-57 (largest / mass) + 4 u / r
+// where u is the unit of the coordinates (each rounded by at most u / 2, plus
+// the 16-bit products of the low words: below 2^-52 r at r = 2^51 u).  With an
+// exponent of its own a mass is as exact as the largest, down to the last place
+// of the sums (2^-57 of the largest mass's force at the tile's extent).
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <random>
+
+#include "../paper_1803_01190_gb300/csrc/fixed.cuh"
+
+using namespace nb;
+typedef long double ld;
+
+static uint32_t hi(double x) { uint64_t b; memcpy(&b, &x, 8); return (uint32_t)(b >> 32); }
+static uint32_t lo(double x) { uint64_t b; memcpy(&b, &x, 8); return (uint32_t)b; }
+static ld value(const fx96 &a, int e) {
+  return ldexpl((ld)a.w2, e + 64) + ldexpl((ld)a.w1, e + 32) + ldexpl((ld)a.w0, e);
+}
+
+int main() {
+  std::mt19937_64 g(5);
+  auto U = [&] { return (double)(g() >> 11) * 0x1p-53; };
+  double worst_f = 0, worst_p = 0, bias = 0;
+  long used = 0, plain = 0, close = 0, wrong = 0;
+  for (long t = 0; t < 600000; t++) {
+    const double E = std::exp2(-30 + 60 * U());
+    int e;
+    frexp(E, &e);
+    const int L = e - FX_BITS;
+    const double eps = E * std::exp2(-20 + 20 * U()) * 0.99;
+    const double off = (t & 1) ? 0.0 : E * std::exp2(20 * U() - 5) * (U() - 0.5);
+    const double span = E * std::exp2(-14 * U());
+    double xi[3], xj[3];
+    uint64_t Xi[3], Xj[3];
+    for (int c = 0; c < 3; c++) {
+      xi[c] = off + 0.3 * E * (U() - 0.5);
+      xj[c] = xi[c] + 0.99 * span * (U() - 0.5);
+      Xi[c] = fx_coord(hi(xi[c]), lo(xi[c]), L);
+      Xj[c] = fx_coord(hi(xj[c]), lo(xj[c]), L);
+    }
+    const double mmax = std::exp2(-20 + 40 * U());
+    const int em = ilogb(mmax);
+    const bool wide = t % 5 == 0, equal = t % 5 == 1;
+    const int range = wide ? FX_MASS_RANGE : FX_MASS_NARROW;
+    const double m = equal ? 1.0 : t % 3 ? mmax * std::exp2(-range * U()) : mmax;
+    if (!equal && ilogb(m) < em - range) continue;
+    const FxMass M = equal ? FxMass{0, 0, 0} : wide ? fx_mass<true>(hi(m), lo(m), em) : fx_mass<false>(hi(m), lo(m), em);
+    const FxEps e2 = fx_eps2(eps * eps, L);
+    const float off_seed = 1.0f + (float)((2 * U() - 1) * 0x1p-22);  // the SFU's error
+    FxPair p;
+    const bool ok = fx_geometry(Xj, Xi, e2, [&](uint32_t x) {
+      const float y = (float)(1.0 / std::sqrt((double)(float)x)) * off_seed;
+      uint32_t b;
+      memcpy(&b, &y, 4);
+      return b;
+    }, p);
+    ld d[3], r2 = (ld)(eps * eps);
+    for (int c = 0; c < 3; c++) {
+      d[c] = (ld)xj[c] - (ld)xi[c];
+      r2 += d[c] * d[c];
+    }
+    const ld r = sqrtl(r2), ur = ldexpl(1, L) / r;
+    if (!ok) {
+      close++;
+      if (ur < ldexpl(0.999L, -51)) wrong++;
+      continue;
+    }
+    if (ur > ldexpl(1.001L, -51)) wrong++;
+    fx96 f[3] = {}, pot = {};
+    if (equal)
+      fx_both(p, f, pot, nullptr, nullptr);
+    else if (wide)
+      fx_side<true>(p, M, f, pot);
+    else
+      fx_side<false>(p, M, f, pot);
+const ld ratio = equal ? 1 : (ld)mmax / m;
+    const int e_m = equal ? FX_EQ_EM : em;
+    // with its own exponent: the place of the last bit of the 96-bit sums
+    const ld light_f = wide ? 1 + ldexpl(ratio, -2) : ratio;
+    const ld light_p = wide ? 1 + ldexpl(ratio, -12) : ratio;
+    const ld rel = value(pot, fx_pot_exp(L, e_m)) * r / m - 1;
+    ld err = 0;
+    for (int c = 0; c < 3; c++) {
+      const ld x = value(f[c], fx_force_exp(L, e_m)) * r2 / m - d[c] / r;
+      err += x * x;
+    }
+    worst_f = std::fmax(worst_f, (double)(sqrtl(err) / (ldexpl(light_f, -55) + 4 * ur)));
+    worst_p = std::fmax(worst_p, (double)(fabsl(rel) / (ldexpl(light_p, -57) + 4 * ur)));
+    if (!wide) bias += (double)rel, plain++;
+    used++;
+  }
+  printf("%ld %ld %ld %.4f %.4f %.3e\n", used, close, wrong, worst_f, worst_p, bias / plain);
+  return 0;
+}

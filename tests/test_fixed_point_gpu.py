@@ -1,0 +1,107 @@
+"""The fixed-point pair sums of the binary64 mode (softened systems), at the edges of their rules.
+
+The reference is the FP64 oracle.  A tile that the fixed-point form does not
+take, and pairs too close for its unit, run in binary64, so every case has to
+meet the same gate: |da| <= 1e-12 |a| + 4 u sqrt(N) S (tests/gates.py), and
+potentials to 1e-12.
+"""
+import numpy as np
+import pytest
+
+import nbody_ics
+import oracle
+from gates import fp64_accel_gate
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nb():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    import paper_1803_01190_gb300 as m
+    return m
+
+
+def _case(kind, n):
+    pos, _, mass = nbody_ics.plummer(n, 20180300 + n)
+    eps = 0.01
+    if kind == "offset":  # coordinates far larger than the differences
+        pos = pos + np.array([3.0e6, -7.0e5, 1.0])
+    elif kind == "scaled":  # units of 1e-40 and 1e30
+        pos, eps, mass = pos * 1e-40, eps * 1e-40, mass * 1e30
+    elif kind == "close":  # half the particles within 1e-5 of another, one escaper
+        pos[n // 2:n // 2 * 2] = pos[:n // 2] + 1e-5 * np.random.default_rng(1).standard_normal((n // 2, 3))
+        pos[-1] = [4.0e3, 0.0, 0.0]
+        eps = 1e-6
+    elif kind == "masses":  # over the mass rule in some tiles, zeros, within it in others
+        rng = np.random.default_rng(2)
+        mass = mass * np.exp(0.5 * rng.standard_normal(n))
+        mass[: n // 3] *= np.exp2(rng.uniform(-30, 30, n // 3))
+        mass[n // 2:n // 2 + 40] = 0.0
+    elif kind == "coincident":
+        pos[1::2] = pos[::2][: len(pos[1::2])]
+    elif kind == "wide eps":
+        eps = 300.0
+    return pos, mass, eps
+
+
+KINDS = ["plain", "offset", "scaled", "close", "masses", "coincident", "wide eps"]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n", [2, 127, 129, 1000, 2305])
+@pytest.mark.parametrize("ipt", [1, 2, 8])
+def test_one_sided(nb, kind, n, ipt):
+    pos, mass, eps = _case(kind, n)
+    with nb.Simulation(n, "fp64", eps=eps) as sim:
+        sim.set_symmetric(0)
+        sim.set_launch(ipt, 0)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, eps, acc, pot)
+
+
+# blocks of 256: n = 257, 512 (M = 2), 700 (M = 3), 2305 (M = 10, tail of one)
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n", [257, 512, 700, 2305])
+def test_each_pair_once(nb, kind, n):
+    pos, mass, eps = _case(kind, n)
+    with nb.Simulation(n, "fp64", eps=eps) as sim:
+        sim.set_symmetric(1)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, eps, acc, pot)
+
+
+def _check(pos, mass, eps, acc, pot):
+    oa, op, smag = oracle.accel(pos, mass, eps)
+    ok, err, amag = fp64_accel_gate(acc, oa, smag, len(mass))
+    assert ok.all(), float((err / np.maximum(amag, 1e-300)).max())
+    assert np.all(np.abs(pot - op) <= 1e-12 * np.abs(op))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("where", ["pos", "mass"])
+def test_non_finite_input_gives_non_finite_output(nb, bad, where):
+    pos, mass, eps = _case("plain", 300)
+    (pos if where == "pos" else mass[:, None])[17, 0] = bad
+    with nb.Simulation(300, "fp64", eps=eps) as sim:
+        acc, pot = sim.accel(pos, mass)
+    others = np.delete(np.arange(300), 17)
+    if np.isnan(bad) or where == "mass":
+        assert not np.isfinite(acc[others]).any() and not np.isfinite(pot[others]).any()
+    else:  # at an infinite distance: no force, by inf * 0
+        assert not np.isfinite(acc[others, 0]).any()
+
+
+def test_negative_mass(nb):
+    pos, mass, eps = _case("plain", 300)
+    mass[5] = -mass[5]
+    with nb.Simulation(300, "fp64", eps=eps) as sim:
+        acc, pot = sim.accel(pos, mass)
+    a1, p1, _ = oracle.accel(pos, np.maximum(mass, 0.0), eps)
+    a2, p2, _ = oracle.accel(pos, np.maximum(-mass, 0.0), eps)
+    assert np.abs(acc - (a1 - a2)).max() <= 1e-12 * np.abs(a1).max()
+    assert np.abs(pot - (p1 - p2)).max() <= 1e-12 * np.abs(p1).max()
