@@ -35,11 +35,18 @@ N_FULL = 2 ** 20
 EPS, DT = 0.02, 5e-4
 # Work each force kernel issues on the pipe that bounds it, per interaction
 # (counted from the kernels' source, confirmed by ncu instruction counts):
-# FP64 pipe instructions of the binary64 paths: 9 one-sided (3 DADD, 3 DFMA for
-# |d|^2 + eps^2, 3 DFMA for the acceleration sums; the potential sum is an
+# FP64 pipe instructions of the binary64 pair body: 9 one-sided (3 DADD, 3 DFMA
+# for |d|^2 + eps^2, 3 DFMA for the acceleration sums; the potential sum is an
 # integer add); 12 per pair evaluated once for both particles (both potential
-# sums integer adds), i.e. 6 per interaction.
+# sums integer adds), i.e. 6 per interaction.  Softened systems, this workload
+# among them, are summed in 64-bit fixed point on the integer pipes instead
+# (csrc/fixed.cuh): the counts then say what the binary64 body would need, and
+# the pipe that binds is the FMA-heavy one.
 FP64_INSTR_PER_INTERACTION = {False: 9, True: 6}
+# FMA-heavy pipe cycles per warp and interaction of the fixed-point kernels,
+# equal masses, by ncu (sm__pipe_fmaheavy_cycles_active at N = 16384): each
+# pair once, 273 per pair.
+FX_HEAVY_CYCLES_PER_INTERACTION = {True: 136.5}
 # FP32 FMA-pipe lane operations: mixed 13 (3 differences, 3 FMAs for
 # |d|^2 + eps^2, m y, y^2, m y^3, 3 FMAs and 1 add into the sums; two j per
 # packed instruction); F64E float-float 162 one-sided, 112 per interaction
@@ -52,15 +59,15 @@ F64E_LANEOPS_PER_INTERACTION = {False: 162, True: 112}
 # DRAM traffic of one FP64 force launch at N = 2^20 (dram__bytes_read.sum +
 # dram__bytes_write.sum from one full-size ncu capture; see the k_force_f64 DRAM
 # profile summary).  It is reported only while the kernel's source is the one
-# that was captured: `src_sha` hashes rsqrt_recip_sig, mul_sig, body_f64 and
-# k_force_f64.
+# that was captured (`src_sha`: the kernels that read and write the slices; the
+# one-sided capture is of an earlier form and no longer reported).
 TRAFFIC = {"k_force_f64": {"bytes": 47.05e6 + 62.96e6, "n": 2 ** 20, "src_sha": "01dc06074becbf43"},
-           # each pair once, blocks of 384: per force evaluation 1 one-sided launch on the
-           # 2731 diagonal blocks + 1365 block diagonals in launches of 8 (pair kernel and
-           # combine); bytes of the first launch of each kernel in one full-size capture,
-           # the pair and combine launches scaled by 1365 / 8
-           "k_force_f64_sym": {"bytes": 34.00e6 + 1365 / 8 * (679.80e6 + 589.80e6), "n": 2 ** 20,
-                               "src_sha": "39fcfb6aac42cd11"}}
+           # each pair once, fixed point, blocks of 256: per force evaluation 1 one-sided
+           # launch on the 4096 diagonal blocks + 2048 block diagonals in launches of 5 (pair
+           # kernel and combine); bytes of the first launch of each kernel in one full-size
+           # capture, the pair and combine launches scaled by 2048 / 5
+           "k_force_f64_sym": {"bytes": 34.01e6 + 2048 / 5 * (433.28e6 + 384.12e6), "n": 2 ** 20,
+                               "src_sha": "29bfce536ae80db9"}}
 
 
 def _kernel_src_sha(names):
@@ -83,13 +90,7 @@ def _kernel_src_sha(names):
 def traffic_f64(n, sym=False):
     if sym:
         t = TRAFFIC["k_force_f64_sym"]
-        sha = _kernel_src_sha(["__device__ __forceinline__ void rsqrt_recip_sig(",
-                               "__device__ __forceinline__ uint64_t mul_sig(",
-                               "__device__ __forceinline__ uint64_t add_pos_bits(",
-                               "__device__ __forceinline__ void acc_pos(",
-                               "__device__ __forceinline__ void scale_pair(",
-                               "__device__ __forceinline__ void body_f64_sym(",
-                               "__global__ void __launch_bounds__(BT) k_force_f64_sym(",
+        sha = _kernel_src_sha(["__global__ void __launch_bounds__(BT, 4) k_force_fx_sym(",
                                "__global__ void k_sym_combine("])
         return t["bytes"] if (sha == t["src_sha"] and n == t["n"]) else None
     t = TRAFFIC["k_force_f64"]
@@ -456,14 +457,24 @@ def run_gpu(args):
 
 
 def roofline_fp64(n, sym, force_ms, step_ms, pipes):
-    """The binary64 force path is bound by the FP64 pipe: achieved = its FP64
-    instructions per interaction x N^2 / the force evaluation's CUDA-event
-    time; peak = the DFMA issue rate measured in the same run."""
+    """The binary64 force path against the FP64 pipe: achieved = the FP64
+    instructions per interaction of the binary64 pair body x N^2 / the force
+    evaluation's CUDA-event time; peak = the DFMA issue rate measured in the
+    same run.  The fixed-point kernels do not issue them, so the fraction may
+    exceed 1: `integer_pipe` is the pipe that binds those."""
     inter = float(n) * n
     ipi = FP64_INSTR_PER_INTERACTION[sym]
     achieved = inter * ipi / (force_ms * 1e-3) / 1e9
     conv = inter * FLOP_PER_INTERACTION / (force_ms * 1e-3) / 1e12
-    return {"bound": "alu", "pipe": "fp64", "kernel": "k_force_f64_sym" if sym else "k_force_f64",
+    heavy = FX_HEAVY_CYCLES_PER_INTERACTION.get(sym)
+    heavy_peak = 4 * pipes["sms"] * pipes["sm_mhz"] / 1e3
+    heavy_achieved = heavy and inter / 32 * heavy / (force_ms * 1e-3) / 1e9
+    return {"bound": "alu", "pipe": "fp64", "kernel": "k_force_fx_sym" if sym else "k_force_f64",
+            "integer_pipe": heavy and {
+                "pipe": "fma heavy", "cycles_per_warp_interaction": heavy, "achieved": heavy_achieved,
+                "peak": heavy_peak, "unit": "G pipe cycles/s", "frac": heavy_achieved / heavy_peak,
+                "note": "fixed-point pair sums: 32 x 32 -> 64 products of 4 cycles a warp; peak = "
+                        "4 sub-partitions x SMs x the SM clock of this run"},
             "achieved": achieved, "peak": pipes["dfma_ginstr_s"], "unit": "G FP64-pipe instr/s",
             "frac": achieved / pipes["dfma_ginstr_s"],
             "peak_source": (f"measured in this run: nbody_measure_pipes DFMA issue rate "
@@ -472,8 +483,8 @@ def roofline_fp64(n, sym, force_ms, step_ms, pipes):
             "instr_per_interaction": ipi,
             "traffic": traffic_f64(n, sym),
             "traffic_note": ("DRAM bytes per force evaluation from one full-size ncu capture: mostly the "
-                             "per-diagonal row/column slices of the each-pair-once schedule, O(N^2/384), far "
-                             "above the O(N) algorithmic bytes but ~0.3% of HBM bandwidth over the evaluation"
+                             "per-diagonal row/column slices of the each-pair-once schedule, O(N^2/256), far "
+                             "above the O(N) algorithmic bytes but ~1% of HBM bandwidth over the evaluation"
                              if sym else
                              "DRAM bytes per force evaluation from one full-size ncu capture; the O(N) "
                              "algorithmic bytes (32 B in + partial sums out per particle) mostly stay in L2"),

@@ -234,8 +234,8 @@ int nbody_get_symmetric(const nbody_ctx *ctx, int *mode, int *active);
  * NBODY_FP64 (which accepts either: the order changes only its summation
  * order).  NBODY_FP32 keeps input order (the paper's SP).
  * Memory: the first force evaluation with the spatial order allocates about
- * 70 + 32 S bytes per particle (keys, indices, permutation, sort scratch and
- * sorted copies of the positions and of the S partial-sum slices).
+ * 70 bytes per particle (keys, indices, permutation, sort scratch and a
+ * sorted copy of the positions).
  * Errors: EINVAL (NULL context, unknown order, NBODY_ORDER_SPATIAL in FP32).
  */
 #define NBODY_ORDER_INPUT   0

@@ -54,14 +54,14 @@ struct nbody_ctx {
   void *sym_buf = nullptr;
   int sym_d = 0;
   // particle order of the force sum: 0 = input order, 1 = spatial (Morton)
-  // order; order scratch, sorted-to-input permutation, sorted positions and
-  // the sorted partial sums (alt_slices slices of n)
+  // order; order scratch, sorted-to-input permutation, sorted positions.  The
+  // partial sums are in the order of the force sum; sums_perm is the
+  // permutation of the last evaluation (NULL: input order)
   int order = 0;
   void *ord_scratch = nullptr;
   int32_t *perm = nullptr;
   d4 *sposm = nullptr;
-  void *part_alt = nullptr;
-  int alt_slices = 0;
+  const int32_t *sums_perm = nullptr;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pool;  // all created events
   size_t ev_used = 0;                                          // pairs recorded since last read
 };
@@ -113,20 +113,34 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
   sh = nb::Shape();
   sh.bt = nb::force_block_threads(c->mode);
   sh.t = nb::force_tile(c->mode);
-  // measured on GB300: FP64 is FP64-pipe bound at any R; the packed FP32 and
-  // float-float kernels keep enough warps resident only at R = 2
-  int r = r_req ? r_req : (c->mode == NBODY_FP64 ? 4 : 2);
+  // measured on GB300: the FP64 kernel runs alike at R = 1 and 2 (131 and 127
+  // Gint/s at N = 65536); the packed FP32 and float-float kernels keep enough
+  // warps resident only at R = 2
+  int r = r_req ? r_req : (c->mode == NBODY_FP64 ? 1 : 2);
   if (c->mode == NBODY_F64E && r > 4) r = 4;
   while (!r_req && r > 1 && (int64_t)sh.bt * r * c->num_sms > c->n) r >>= 1;
   sh.r = r;
-  const int64_t bx = (c->n + (int64_t)sh.bt * r - 1) / ((int64_t)sh.bt * r);
+  // small n: with one i-particle per thread and one tile per block there are
+  // still fewer warps than hide the latency of a pair; split the tiles over
+  // the warps of a block instead
+  if (!r_req && !s_req && c->n < nb::force_split_max_n(c->mode)) {
+    sh.r = r = 1;
+    sh.iw = nb::force_split(c->mode);
+  }
+  const int64_t bx = (c->n + sh.per_block() - 1) / sh.per_block();
   const int64_t smax = (c->n + sh.t - 1) / sh.t;
   int64_t s = s_req;
   if (!s) {
     int occ = nb::force_max_blocks_per_sm(c->mode, sh);
     if (occ < 1) occ = 1;
-    const int64_t target = 8LL * c->num_sms * occ;
-    s = (target + bx - 1) / bx;
+    // eight waves of resident blocks; where segments stay 16 tiles or longer,
+    // up to 32, so that the last wave weighs less (measured, Gint/s: MIXED
+    // N = 131072 at 8, 16 and 24 segments 2449, 2549, 2557; 300000 at 4, 8, 32:
+    // 2462, 2543, 2568; 2^20 at 2, 4, 16: 2550, 2556, 2562; one-sided FP64 65536
+    // at 8, 16, 32: 128, 131, 132)
+    const int64_t slots = (int64_t)c->num_sms * occ;
+    s = std::max<int64_t>((8 * slots + bx - 1) / bx,
+                          std::min<int64_t>((32 * slots + bx - 1) / bx, smax / 16));
   }
   if (s > smax) s = smax;
   if (s > 64) s = 64;
@@ -142,28 +156,17 @@ static int64_t seg_len(const nbody_ctx *c, int &S) {
   return seg;
 }
 
-static int ensure_slices(nbody_ctx *c, void **buf, int *have, int S) {
-  if (S <= *have) return NBODY_OK;
-  if (*buf) cudaFree(*buf);
-  *buf = nullptr;
-  *have = 0;
-  if (cudaMalloc(buf, (size_t)S * c->n * part_r4(c)) != cudaSuccess)
+// S slices of partial sums in c->part.
+static int ensure_part(nbody_ctx *c, int S) {
+  if (S <= c->part_slices) return NBODY_OK;
+  if (c->part) cudaFree(c->part);
+  c->part = nullptr;
+  c->part_slices = 0;
+  if (cudaMalloc(&c->part, (size_t)S * c->n * part_r4(c)) != cudaSuccess)
     return fail(NBODY_ENOMEM, "j-segment partial buffer");
-  *have = S;
+  c->part_slices = S;
   return NBODY_OK;
 }
-
-// S slices of partial sums in c->part and, with the spatial order, as many in
-// c->part_alt (the force kernels write there; the slices are then moved to
-// input order in c->part).
-static int ensure_part(nbody_ctx *c, int S) {
-  int rc = ensure_slices(c, &c->part, &c->part_slices, S);
-  if (!rc && c->order) rc = ensure_slices(c, &c->part_alt, &c->alt_slices, S);
-  return rc;
-}
-
-// The force kernels' output slices for this evaluation.
-static void *force_out(const nbody_ctx *c) { return c->order ? c->part_alt : c->part; }
 
 // Smallest n at which the automatic choice evaluates each pair once: 64 blocks
 // of 256 (F64E), and 64 blocks of 384 in FP64 whatever its block size.  With
@@ -208,7 +211,7 @@ static int force_sym(nbody_ctx *c, const void *posm_in, int &S) {
   while (P < want && P < (ff ? 2 : 4)) P *= 2;
   int rc = ensure_part(c, P + 2);
   if (rc) return rc;
-  void *out = force_out(c);  // only after ensure_part, which may (re)allocate it
+  void *out = c->part;  // only after ensure_part, which may (re)allocate it
   if (c->sym_units_m != M * P) {
     if (c->sym_units) cudaFree(c->sym_units);
     c->sym_units = nullptr;
@@ -283,24 +286,22 @@ static int ensure_order(nbody_ctx *c) {
 
 static int force_sums(nbody_ctx *c, const void *posm_in, int &S);
 
-// Raw force sums of the positions in posm_in into c->part (input order);
-// returns the number of partial slices written through S.  With the spatial
-// order the particles are sorted along a Morton curve first, the force
-// kernels run on the sorted copy, and their slices are scattered back.
+// Raw force sums of the positions in posm_in into c->part; returns the number
+// of partial slices written through S.  With the spatial order the particles
+// are sorted along a Morton curve first and the force kernels run on the
+// sorted copy; the epilogues read the sums through the permutation.
 static int force(nbody_ctx *c, const void *posm_in, int &S) {
+  c->sums_perm = nullptr;
   if (!c->order) return force_sums(c, posm_in, S);
   int rc = ensure_order(c);
   if (rc) return rc;
   CK(nb::launch_spatial_order((const d4 *)posm_in, c->n, c->ord_scratch, c->perm, c->sposm, c->st));
   c->launches += 4;
-  rc = force_sums(c, c->sposm, S);
-  if (rc) return rc;
-  CK(nb::launch_unpermute((const d4 *)c->part_alt, c->perm, S, c->n, (d4 *)c->part, c->st));
-  c->launches++;
-  return NBODY_OK;
+  c->sums_perm = c->perm;
+  return force_sums(c, c->sposm, S);
 }
 
-// The force kernels on posm_in, partial slices into force_out(c).
+// The force kernels on posm_in, partial slices into c->part.
 static int force_sums(nbody_ctx *c, const void *posm_in, int &S) {
   std::pair<cudaEvent_t, cudaEvent_t> *ev = nullptr;
   if (c->prof) {
@@ -334,7 +335,7 @@ static int force_sums(nbody_ctx *c, const void *posm_in, int &S) {
   in.n = c->n;
   in.eps2 = c->eps * c->eps;
   in.seg = seg;
-  in.part = force_out(c);
+  in.part = c->part;
   nb::Shape sh = c->shape;
   sh.s = S;
   if (ev) CK(cudaEventRecord(ev->first, c->st));
@@ -350,6 +351,7 @@ static nb::EpiIn epi(const nbody_ctx *c, int S) {
   e.S = S;
   e.part = c->part;
   e.G = c->G;
+  e.perm = c->sums_perm;
   return e;
 }
 
@@ -380,7 +382,7 @@ static void free_all(nbody_ctx *c) {
   void *ptrs[] = {c->posm[0], c->posm[1], c->vel, c->vbar, c->acc, c->part, c->rk_vs, c->rk_sr,
                   c->rk_sv, c->tmp_posm, c->tmp_acc, c->fpos, c->anchor, c->diag_blocks,
                   c->diag_out, c->d_flag, c->stage, c->sym_units, c->sym_buf,
-                  c->ord_scratch, c->perm, c->sposm, c->part_alt};
+                  c->ord_scratch, c->perm, c->sposm};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (c->h_diag) cudaFreeHost(c->h_diag);
@@ -634,6 +636,7 @@ int nbody_accel_rows(nbody_ctx *c, int64_t i0, int64_t ni, const double *pos, co
   CK(nb::launch_force(c->mode, in, sh, c->st));
   nb::EpiIn e = epi(c, S);
   e.n = ni;
+  e.perm = nullptr;
   CK(nb::launch_store_acc(c->mode, e, c->tmp_acc, c->st));
   c->launches += 2;
   return copy_acc_out(c, c->tmp_acc, acc, pot, on_device, ni);

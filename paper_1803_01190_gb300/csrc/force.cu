@@ -266,6 +266,28 @@ struct TableWork {
   __device__ __forceinline__ Unit get(int64_t k) const { return units[k]; }
 };
 
+// Writes the sums v of i-particle li (< ni).  IW > 1: the IW threads that share
+// it (thread `it` of IT, share jw) add theirs in order first.
+template <int IW, class V>
+__device__ __forceinline__ void store_shares(V *out, int li, int ni, V v, V *red, int it, int IT,
+                                             int jw) {
+  if (IW > 1) {
+    __syncthreads();
+    red[threadIdx.x] = v;
+    __syncthreads();
+    if (jw != 0) return;
+#pragma unroll
+    for (int w = 1; w < IW; w++) {
+      const V o = red[w * IT + it];
+      v.x += o.x;
+      v.y += o.y;
+      v.z += o.z;
+      v.w += o.w;
+    }
+  }
+  if (li < ni) out[li] = v;
+}
+
 // ---------------------------------------------------------------- binary64
 template <bool MASK>
 __device__ __forceinline__ void body_f64(const d4 &pj, double xi, double yi, double zi,
@@ -317,7 +339,6 @@ __device__ __noinline__ d4 pair_f64(double dx, double dy, double dz, double m, d
 struct FxBox {
   int lo[3], hi[3], mmax, mmin;
 };
-__device__ __forceinline__ int fx_key(int hi) { return hi ^ ((hi >> 31) & 0x7FFFFFFF); }
 __device__ __forceinline__ void fx_box_init(FxBox &b) {
 #pragma unroll
   for (int c = 0; c < 3; c++) {
@@ -468,7 +489,8 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
   __shared__ int tdm[T];
   __shared__ FxBox sbox[NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int it = tid % IT, jw = tid / IT;  // i-thread, share of the j-tile
+  // i-thread, share of the j-tile
+  const int it = IW == 1 ? tid : tid % IT, jw = IW == 1 ? 0 : tid / IT;
   for (int64_t uk = work.first(); uk < work.count(); uk += work.stride()) {
     const Unit u = work.get(uk);
     const int64_t j1 = u.j0 + u.nj;
@@ -1172,6 +1194,33 @@ __device__ __forceinline__ double f2d_exact(float f) {
   return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+// x = h + l in floats: h to nearest, l = the rest rounded to 24 bits.  The
+// conversions run on the FP64 pipe (64 cycles a warp each: the three
+// coordinates of an i-particle cost as much as 22 mixed pairs), so they are
+// integer moves in the range where both halves are normal floats.
+__device__ __forceinline__ void split_ff(double x, float &h, float &l) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7FFu;
+  if (ex - 960u < 180u) {  // 2^-63 <= |x| < 2^117
+    const unsigned mag = (hi & 0x7FFFFFFFu) - 0x38000000u;
+    const unsigned rlo = lo + 0x10000000u;  // round the upper 24 bits to nearest
+    const unsigned rhi = mag + (rlo < lo);
+    const unsigned sign = hi & 0x80000000u;
+    h = __uint_as_float(__funnelshift_l(rlo, rhi, 3) | sign);
+    const int rest = (int)(lo << 3) >> 3;  // signed 29 bits below them
+    const float scale = __uint_as_float(((ex - 948u) << 23) | sign);  // 2^(ex - 1075)
+    l = __int2float_rn(rest) * scale;
+  } else {
+    h = __double2float_rn(x);
+    l = __double2float_rn(x - (double)h);
+  }
+}
+// h + l in binary64 (non-finite halves by conversion, which keeps them so)
+__device__ __forceinline__ double join_ff(float h, float l) {
+  const bool finite = fabsf(h) < INFINITY && fabsf(l) < INFINITY;
+  return finite ? f2d_exact(h) + f2d_exact(l) : (double)h + (double)l;
+}
+
 // One tile entry: j = 2k, 2k+1 as H = (xh0, xh1, yh0, yh1), H2 = (zh0, zh1, mh0, mh1),
 // L, L2 the matching low parts.  (nxh, nxl, ...) are the negated float-float
 // i coordinates in both halves; the four float-float accumulators get the
@@ -1278,15 +1327,19 @@ __device__ __forceinline__ void load_pairs_ff(const float4 *__restrict__ src, in
 // F64E force: i coordinates re-centred on each j-tile's anchor in float-float
 // (from the particle's own float-float and the anchor's), pair terms and
 // per-tile partial sums in float-float, folded into binary64 once per tile.
-template <int BT, int R, int T, class W>
+template <int BT, int R, int T, int IW, class W>
 __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
                                                    const float4 *__restrict__ jff,
                                                    const float4 *__restrict__ anchor, W work,
                                                    d4 *__restrict__ part) {
+  constexpr int IT = BT / IW;
   __shared__ float4 tH[T / 2], tH2[T / 2], tL[T / 2], tL2[T / 2];
+  __shared__ d4 red[IW > 1 ? BT : 1];
   for (int64_t uk = work.first(); uk < work.count(); uk += work.stride()) {
     const Unit u = work.get(uk);
     const int tid = threadIdx.x;
+    // i-thread, share of the j-tile
+  const int it = IW == 1 ? tid : tid % IT, jw = IW == 1 ? 0 : tid / IT;
     const int64_t j1 = u.j0 + u.nj;
     const float e2hs = (float)u.eps2;
     const float e2ls = (float)(u.eps2 - (double)e2hs);
@@ -1295,13 +1348,12 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
     double acc[R][4];
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int li = r * BT + tid;
+      const int li = r * IT + it;
       const d4 p = posm[u.i0 + (li < u.ni ? li : 0)];
       const double c3[3] = {p.x, p.y, p.z};
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        xh[r][c] = __double2float_rn(c3[c]);
-        xl[r][c] = __double2float_rn(c3[c] - (double)xh[r][c]);
+        split_ff(c3[c], xh[r][c], xl[r][c]);
       }
 #pragma unroll
       for (int c = 0; c < 4; c++) acc[r][c] = 0.0;
@@ -1331,9 +1383,10 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
         for (int c = 0; c < 4; c++) ah[r][c] = al[r][c] = f2(0.0f, 0.0f);
       }
       const int np = (cnt + 1) / 2;
+      const int k0 = np * jw / IW, k1 = np * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
       if (cnt == T && !diag) {
-        for (int k = 0; k < T / 2; k++) {
+        for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
           const float4 H = tH[k], H2 = tH2[k], L = tL[k], L2 = tL2[k];
 #pragma unroll
           for (int r = 0; r < R; r++)
@@ -1341,12 +1394,12 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
                            nl[r][2], e2h, e2l, ah[r], al[r], false, false);
         }
       } else {
-        for (int k = 0; k < np; k++) {
+        for (int k = k0; k < k1; k++) {
           const float4 H = tH[k], H2 = tH2[k], L = tL[k], L2 = tL2[k];
           const int64_t j = jt + 2 * k;
 #pragma unroll
           for (int r = 0; r < R; r++) {
-            const int64_t i = u.i0 + r * BT + tid;
+            const int64_t i = u.i0 + r * IT + it;
             body_ff<true>(H, H2, L, L2, nh[r][0], nl[r][0], nh[r][1], nl[r][1], nh[r][2],
                           nl[r][2], e2h, e2l, ah[r], al[r], j == i, j + 1 == i);
           }
@@ -1365,8 +1418,9 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
     }
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int li = r * BT + tid;
-      if (li < u.ni) part[u.out + li] = d4{acc[r][0], acc[r][1], acc[r][2], acc[r][3]};
+      const int li = r * IT + it;
+      const d4 v = {acc[r][0], acc[r][1], acc[r][2], acc[r][3]};
+      store_shares<IW>(part + u.out, li, u.ni, v, red, it, IT, jw);
     }
   }
 }
@@ -1503,8 +1557,8 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
     const double c3[3] = {pi.x, pi.y, pi.z};
 #pragma unroll
     for (int c = 0; c < 3; c++) {  // -(x_i - c_J) as float-float
-      const float xh = __double2float_rn(c3[c]);
-      const float xl = __double2float_rn(c3[c] - (double)xh);
+      float xh, xl;
+      split_ff(c3[c], xh, xl);
       float s, e;
       two_sum1(xh, -chv[c], s, e);
       const float t = __fadd_rn(__fsub_rn(xl, clv[c]), e);
@@ -1514,8 +1568,8 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
       nh[r][c] = f2(-h, -h);
       nl[r][c] = f2(-l, -l);
     }
-    const float m_h = __double2float_rn(pi.w);
-    const float m_l = __double2float_rn(pi.w - (double)m_h);
+    float m_h, m_l;
+    split_ff(pi.w, m_h, m_l);
     mh[r] = f2(m_h, m_h);
     ml[r] = f2(m_l, m_l);
 #pragma unroll
@@ -1596,12 +1650,9 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
     for (int r = 0; r < R; r++) {
       const int li = r * BT + tid;
       const d4 p = posm[u.i0 + (li < u.ni ? li : 0)];
-      xh[r] = __double2float_rn(p.x);
-      yh[r] = __double2float_rn(p.y);
-      zh[r] = __double2float_rn(p.z);
-      xl[r] = __double2float_rn(p.x - (double)xh[r]);
-      yl[r] = __double2float_rn(p.y - (double)yh[r]);
-      zl[r] = __double2float_rn(p.z - (double)zh[r]);
+      split_ff(p.x, xh[r], xl[r]);
+      split_ff(p.y, yh[r], yl[r]);
+      split_ff(p.z, zh[r], zl[r]);
       axh[r] = axl[r] = ayh[r] = ayl[r] = azh[r] = azl[r] = pth[r] = ptl[r] = 0.0f;
     }
     for (int64_t jt = u.j0; jt < j1; jt += T) {
@@ -1630,7 +1681,8 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
       const int np = (cnt + 1) / 2;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
       if (cnt == T && !diag) {
-#pragma unroll 2
+// unroll 2 / 4 measured at N = 131072: R = 1 2446 / 2406 Gint/s, R = 2 2500 / 2517
+#pragma unroll(R == 1 ? 2 : 4)
         for (int k = 0; k < T / 2; k++) {
           const float4 A = tA[k], B = tB[k];
 #pragma unroll
@@ -1639,6 +1691,7 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
                                    false, false);
         }
       } else {
+#pragma unroll(R == 1 ? 2 : 1)
         for (int k = 0; k < np; k++) {
           const float4 A = tA[k], B = tB[k];
           const int64_t j = jt + 2 * k;
@@ -1662,8 +1715,8 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
     for (int r = 0; r < R; r++) {
       const int li = r * BT + tid;
       if (li < u.ni)
-        part[u.out + li] = d4{(double)axh[r] + (double)axl[r], (double)ayh[r] + (double)ayl[r],
-                              (double)azh[r] + (double)azl[r], (double)pth[r] + (double)ptl[r]};
+        part[u.out + li] = d4{join_ff(axh[r], axl[r]), join_ff(ayh[r], ayl[r]),
+                              join_ff(azh[r], azl[r]), join_ff(pth[r], ptl[r])};
     }
   }
 }
@@ -1675,7 +1728,11 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
 // stays near the centre of the particle distribution even when a few members
 // sit far out in a halo (a bounding-box centre would be pulled out there and
 // cost every coordinate relative to it several digits).  It is found with a
-// bitonic sort of each coordinate in shared memory (tile = block = 256).
+// bitonic sort of the high words as integers, the three coordinates together
+// (tile = block = 256; lane shuffles below strides of 32), and a count among
+// the members that share the median's high word.  6.5 us at N = 2048; sorting
+// the binary64 values in shared memory, one coordinate after the other, took
+// about 15: its comparisons ran on the FP64 pipe and every stage had a barrier.
 struct DensePrep {
   int64_t n;
   int tile;
@@ -1700,7 +1757,10 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
                                                    float4 *__restrict__ fpos,
                                                    float4 *__restrict__ anchor) {
   static_assert((BT & (BT - 1)) == 0, "bitonic sort needs a power-of-two block");
-  __shared__ double v[BT];
+  __shared__ int v[2][3][BT];
+  __shared__ int mid[3], first[3], same[3];
+  __shared__ unsigned low[3][BT];
+  __shared__ double med[3];
   const PrepUnit pu = work.get();
   const int64_t t = pu.anchor;
   const int64_t j0 = pu.j0;
@@ -1708,27 +1768,67 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
   const int tid = threadIdx.x;
   d4 p = {0, 0, 0, 0};
   if (tid < cnt) p = posm[j0 + tid];
-  double c[3];
-  for (int q = 0; q < 3; q++) {
-    __syncthreads();
-    v[tid] = tid < cnt ? (q == 0 ? p.x : q == 1 ? p.y : p.z) : 1e308;
-    __syncthreads();
-    for (int k = 2; k <= BT; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        const int o = tid ^ j;
-        if (o > tid) {
-          const double a = v[tid], b = v[o];
-          const bool up = (tid & k) == 0;
-          if ((a > b) == up) {
-            v[tid] = b;
-            v[o] = a;
-          }
-        }
+  int key[3] = {0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF};
+  if (tid < cnt) {
+    key[0] = fx_key(__double2hiint(p.x));
+    key[1] = fx_key(__double2hiint(p.y));
+    key[2] = fx_key(__double2hiint(p.z));
+  }
+  int buf = 0;
+  for (int k = 2; k <= BT; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const bool low = ((tid & j) == 0) == ((tid & k) == 0);  // keeps the smaller one
+      if (j >= 32) {
+#pragma unroll
+        for (int q = 0; q < 3; q++) v[buf][q][tid] = key[q];
         __syncthreads();
       }
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        const int o = j >= 32 ? v[buf][q][tid ^ j] : __shfl_xor_sync(0xFFFFFFFFu, key[q], j);
+        key[q] = low ? min(key[q], o) : max(key[q], o);
+      }
+      if (j >= 32) buf ^= 1;  // the next exchange writes the other buffer
     }
-    c[q] = v[(cnt - 1) / 2];
   }
+  // key[q] is now the tid-th smallest high word; of the members with the
+  // median's, in any order, the one of rank (cnt - 1) / 2 - first is the median
+  const int rank = (cnt - 1) / 2;
+  if (tid == rank) {
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      mid[q] = key[q];
+      first[q] = rank;
+      same[q] = 0;
+    }
+  }
+  __syncthreads();
+  const double x[3] = {p.x, p.y, p.z};
+  bool member[3];
+  unsigned lo[3];
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    if (tid < rank && key[q] == mid[q]) atomicMin(&first[q], tid);
+    member[q] = tid < cnt && fx_key(__double2hiint(x[q])) == mid[q];
+    // the low words ordered as the values (reversed below zero)
+    lo[q] = (unsigned)__double2loint(x[q]) ^ (mid[q] < 0 ? 0xFFFFFFFFu : 0u);
+    if (member[q]) low[q][atomicAdd(&same[q], 1)] = lo[q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    if (member[q]) {  // almost always one member
+      const int want = rank - first[q];
+      int below = 0, equal = 0;
+      for (int o = 0; o < same[q]; o++) {
+        below += low[q][o] < lo[q];
+        equal += low[q][o] == lo[q];
+      }
+      if (below <= want && want < below + equal) med[q] = x[q];  // equal values write alike
+    }
+  }
+  __syncthreads();
+  const double c[3] = {med[0], med[1], med[2]};
   if (tid < cnt) {
     const double dx = p.x - c[0], dy = p.y - c[1], dz = p.z - c[2];
     const float hx = __double2float_rn(dx), hy = __double2float_rn(dy), hz = __double2float_rn(dz),
@@ -1753,19 +1853,23 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
 }
 
 // ---------------------------------------------------------------- binary32 (paper's SP)
-template <int BT, int R, int T, class W>
+template <int BT, int R, int T, int IW, class W>
 __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ posm, W work,
                                                   float4 *__restrict__ part) {
+  constexpr int IT = BT / IW;
   __shared__ float4 tA[T / 2], tB[T / 2];
+  __shared__ float4 red[IW > 1 ? BT : 1];
   for (int64_t uk = work.first(); uk < work.count(); uk += work.stride()) {
     const Unit u = work.get(uk);
     const int tid = threadIdx.x;
+    // i-thread, share of the j-tile
+  const int it = IW == 1 ? tid : tid % IT, jw = IW == 1 ? 0 : tid / IT;
     const int64_t j1 = u.j0 + u.nj;
     const float2 e2 = f2((float)u.eps2, (float)u.eps2);
     float2 nx[R], ny[R], nz[R], ax[R], ay[R], az[R], pt[R];
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int li = r * BT + tid;
+      const int li = r * IT + it;
       const float4 p = posm[u.i0 + (li < u.ni ? li : 0)];
       nx[r] = f2(-p.x, -p.x);
       ny[r] = f2(-p.y, -p.y);
@@ -1778,10 +1882,11 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
       load_pairs<BT, T>(posm, jt, cnt, tA, tB);
       __syncthreads();
       const int np = (cnt + 1) / 2;
+      const int k0 = np * jw / IW, k1 = np * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
       if (cnt == T && !diag) {
 #pragma unroll 2
-        for (int k = 0; k < T / 2; k++) {
+        for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
           const float4 A = tA[k], B = tB[k];
 #pragma unroll
           for (int r = 0; r < R; r++)
@@ -1789,12 +1894,12 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
                                     false, false);
         }
       } else {
-        for (int k = 0; k < np; k++) {
+        for (int k = k0; k < k1; k++) {
           const float4 A = tA[k], B = tB[k];
           const int64_t j = jt + 2 * k;
 #pragma unroll
           for (int r = 0; r < R; r++) {
-            const int64_t i = u.i0 + r * BT + tid;
+            const int64_t i = u.i0 + r * IT + it;
             body_pair<true, false>(A, B, nx[r], ny[r], nz[r], e2, ax[r], ay[r], az[r], pt[r],
                                    j == i, j + 1 == i);
           }
@@ -1803,10 +1908,10 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
     }
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int li = r * BT + tid;
-      if (li < u.ni)
-        part[u.out + li] = make_float4(__fadd_rn(ax[r].x, ax[r].y), __fadd_rn(ay[r].x, ay[r].y),
-                                       __fadd_rn(az[r].x, az[r].y), __fadd_rn(pt[r].x, pt[r].y));
+      const int li = r * IT + it;
+      const float4 v = make_float4(__fadd_rn(ax[r].x, ax[r].y), __fadd_rn(ay[r].x, ay[r].y),
+                                   __fadd_rn(az[r].x, az[r].y), __fadd_rn(pt[r].x, pt[r].y));
+      store_shares<IW>(part + u.out, li, u.ni, v, red, it, IT, jw);
     }
   }
 }
@@ -1820,12 +1925,26 @@ constexpr int BT_FF = 128, T_FF = 256;
 int force_block_threads(int mode) {
   return mode == NBODY_FP64 ? BT_F64 : mode == NBODY_F64E ? BT_FF : BT_F32;
 }
+// Warps of a block that share i-particles at small n: all of them.
+constexpr int IW_F64 = BT_F64 / 32, IW_F32 = BT_F32 / 32, IW_FF = BT_FF / 32;
+int force_split(int mode) {
+  return mode == NBODY_FP64 ? IW_F64 : mode == NBODY_F64E ? IW_FF : mode == NBODY_FP32 ? IW_F32 : 1;
+}
+// Measured on GB300 (force kernel, split against one i-particle per thread, us):
+// FP64 N = 1000 23 / 57, 3000 88 / 111, 4096 147 / 162, 6000 299 / 308; F64E 1000
+// 14 / 35, 4096 88 / 100, 6000 174 / 187; FP32 3000 12.0 / 14.9, 5000 20.9 / 22.5,
+// 6000 26.5 / 26.6.  MIXED is not split: a pair costs it so little that what a
+// thread does once per i-particle weighs more (4096: 39 / 18).
+int64_t force_split_max_n(int mode) {
+  return mode == NBODY_MIXED ? 0 : mode == NBODY_FP32 ? 6144 : 8192;
+}
 int force_tile(int mode) { return mode == NBODY_FP64 ? T_F64 : mode == NBODY_F64E ? T_FF : T_F32; }
 
 bool shape_supported(int mode, const Shape &sh) {
   if (sh.r != 1 && sh.r != 2 && sh.r != 4 && sh.r != 8) return false;
   if (mode == NBODY_F64E && sh.r == 8) return false;
   if (sh.s < 1 || sh.s > 65535) return false;
+  if (sh.iw != 1 && (sh.iw != force_split(mode) || sh.r != 1)) return false;
   return sh.bt == force_block_threads(mode) && sh.t == force_tile(mode);
 }
 
@@ -1834,8 +1953,8 @@ static const void *kernel_for(int mode) {
   switch (mode) {
     case NBODY_FP64: return (const void *)k_force_f64<BT_F64, R, T_F64, 1, DenseWork>;
     case NBODY_MIXED: return (const void *)k_force_mixed<BT_F32, R, T_F32, DenseWork>;
-    case NBODY_F64E: return (const void *)k_force_f64e<BT_FF, (R < 4 ? R : 4), T_FF, DenseWork>;
-    default: return (const void *)k_force_f32<BT_F32, R, T_F32, DenseWork>;
+    case NBODY_F64E: return (const void *)k_force_f64e<BT_FF, (R < 4 ? R : 4), T_FF, 1, DenseWork>;
+    default: return (const void *)k_force_f32<BT_F32, R, T_F32, 1, DenseWork>;
   }
 }
 
@@ -1856,21 +1975,22 @@ int force_max_blocks_per_sm(int mode, const Shape &sh) {
   return nb;
 }
 
-template <int R, class W>
+template <int R, bool SPLIT, class W>
 static void launch_rw(int mode, const void *posm, const float4 *fpos, const float4 *anchor,
                       const W &w, dim3 grid, void *part, cudaStream_t st) {
   if (mode == NBODY_FP64) {
-    k_force_f64<BT_F64, R, T_F64, 1, W><<<grid, BT_F64, 0, st>>>((const d4 *)posm, w, (d4 *)part);
+    k_force_f64<BT_F64, R, T_F64, SPLIT ? IW_F64 : 1, W>
+        <<<grid, BT_F64, 0, st>>>((const d4 *)posm, w, (d4 *)part);
   } else if (mode == NBODY_MIXED) {
-    k_force_mixed<BT_F32, R, T_F32, W><<<grid, BT_F32, 0, st>>>((const d4 *)posm, fpos, anchor, w,
-                                                                (d4 *)part);
+    k_force_mixed<BT_F32, R, T_F32, W>
+        <<<grid, BT_F32, 0, st>>>((const d4 *)posm, fpos, anchor, w, (d4 *)part);
   } else if (mode == NBODY_F64E) {
     constexpr int RF = R < 4 ? R : 4;
-    k_force_f64e<BT_FF, RF, T_FF, W><<<grid, BT_FF, 0, st>>>((const d4 *)posm, fpos, anchor, w,
-                                                             (d4 *)part);
+    k_force_f64e<BT_FF, RF, T_FF, SPLIT ? IW_FF : 1, W>
+        <<<grid, BT_FF, 0, st>>>((const d4 *)posm, fpos, anchor, w, (d4 *)part);
   } else {
-    k_force_f32<BT_F32, R, T_F32, W><<<grid, BT_F32, 0, st>>>((const float4 *)posm, w,
-                                                              (float4 *)part);
+    k_force_f32<BT_F32, R, T_F32, SPLIT ? IW_F32 : 1, W>
+        <<<grid, BT_F32, 0, st>>>((const float4 *)posm, w, (float4 *)part);
   }
 }
 
@@ -1879,10 +1999,10 @@ static cudaError_t launch_w(int mode, int r, const void *posm, const float4 *fpo
                             const float4 *anchor, const W &w, dim3 grid, void *part,
                             cudaStream_t st) {
   switch (r) {
-    case 1: launch_rw<1>(mode, posm, fpos, anchor, w, grid, part, st); break;
-    case 2: launch_rw<2>(mode, posm, fpos, anchor, w, grid, part, st); break;
-    case 4: launch_rw<4>(mode, posm, fpos, anchor, w, grid, part, st); break;
-    case 8: launch_rw<8>(mode, posm, fpos, anchor, w, grid, part, st); break;
+    case 1: launch_rw<1, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
+    case 2: launch_rw<2, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
+    case 4: launch_rw<4, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
+    case 8: launch_rw<8, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -1960,7 +2080,7 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   const int64_t rows = in.rows < 0 ? in.n : in.rows;
   if (!shape_supported(mode, sh) || in.n < 1 || rows < 1 || in.i0 < 0 || in.i0 + rows > in.n)
     return cudaErrorInvalidValue;
-  const int64_t per_block = (int64_t)sh.bt * sh.r;
+  const int64_t per_block = sh.per_block();
   const bool aligned = mode == NBODY_FP64;
   const int64_t gx = ((aligned ? in.i0 % per_block : 0) + rows + per_block - 1) / per_block;
   if (gx > 0x7fffffff) return cudaErrorInvalidValue;
@@ -1973,8 +2093,12 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   w.per_block = (int)per_block;
   w.tile = sh.t;
   w.aligned = aligned;
-  return launch_w(mode, sh.r, in.posm, in.fpos, in.anchor, w, dim3((unsigned)gx, (unsigned)sh.s),
-                  in.part, st);
+  const dim3 grid((unsigned)gx, (unsigned)sh.s);
+  if (sh.iw > 1) {
+    launch_rw<1, true>(mode, in.posm, in.fpos, in.anchor, w, grid, in.part, st);
+    return cudaGetLastError();
+  }
+  return launch_w(mode, sh.r, in.posm, in.fpos, in.anchor, w, grid, in.part, st);
 }
 
 cudaError_t launch_force_units(int mode, const void *posm, const float4 *fpos,

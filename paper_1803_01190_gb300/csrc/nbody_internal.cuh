@@ -24,6 +24,9 @@ struct __align__(32) d4 {
   double x, y, z, w;
 };
 
+// High word of a binary64 as a signed integer of the same order (its own inverse).
+__device__ __forceinline__ int fx_key(int hi) { return hi ^ ((hi >> 31) & 0x7FFFFFFF); }
+
 template <typename real>
 struct vec4;
 template <>
@@ -38,12 +41,16 @@ template <typename real>
 using real4 = typename vec4<real>::type;
 
 // Force-kernel shape.  BT threads per block, R i-particles per thread, T
-// j-particles per shared-memory tile; grid = (ceil(n / (BT*R)), S).
+// j-particles per shared-memory tile; iw = 1: grid = (ceil(n / (BT*R)), S).  iw
+// = force_split(mode) (small n, R = 1): the warps of a block share BT / iw
+// i-particles and split each tile.
 struct Shape {
   int bt = 128;
   int r = 4;
   int t = 128;
   int s = 1;
+  int iw = 1;
+  int per_block() const { return bt / iw * r; }
 };
 
 // One thread block's share of a force evaluation: i-particles [i0, i0+ni)
@@ -90,6 +97,8 @@ cudaError_t launch_force_units(int mode, const void *posm, const float4 *fpos,
 cudaError_t launch_mixed_prep_units(const d4 *posm, const PrepUnit *units, int64_t nunits,
                                     float4 *fpos, float4 *anchor, cudaStream_t st, bool ff = false);
 int force_block_threads(int mode);
+int force_split(int mode);
+int64_t force_split_max_n(int mode);  // below this n the split is the better shape
 int force_tile(int mode);
 // ff: write float-float re-centred coordinates (F64E, two float4 per particle)
 cudaError_t launch_mixed_prep(const d4 *posm, int64_t n, int tile, float4 *fpos, float4 *anchor,
@@ -126,6 +135,7 @@ struct EpiIn {
   int S;
   const void *part;  // S * n raw sums (real4 for FP64/FP32; d4 for MIXED)
   double G;
+  const int32_t *perm = nullptr;  // input index of the sums' k-th particle (NULL: k)
 };
 cudaError_t launch_pack(int mode, const double *pos, const double *vel, const double *mass,
                         int64_t n, void *posm, void *velv, int *flag, cudaStream_t st);
@@ -149,14 +159,10 @@ int diag_blocks(int64_t n);
 
 // Spatial (Morton) order of the particles (order.cu).  launch_spatial_order
 // writes perm (sorted position -> input index) and sposm[s] = posm[perm[s]],
-// using `scratch` of order_scratch_bytes(n); launch_unpermute scatters S
-// slices of sorted partial sums back to input order: part[k n + perm[s]] =
-// sorted[k n + s].
+// using `scratch` of order_scratch_bytes(n).  Its kernel launches: at most 4.
 size_t order_scratch_bytes(int64_t n);
 cudaError_t launch_spatial_order(const d4 *posm, int64_t n, void *scratch, int32_t *perm,
                                  d4 *sposm, cudaStream_t st);
-cudaError_t launch_unpermute(const d4 *sorted, const int32_t *perm, int S, int64_t n, d4 *part,
-                             cudaStream_t st);
 
 // Records the detail that nbody_last_error() returns on this thread and
 // returns `code` (api.cu); every entry point reports its failures through it.

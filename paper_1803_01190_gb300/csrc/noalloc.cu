@@ -145,9 +145,9 @@ extern "C" int nbody_accel_f64_static(int64_t n, const double *pos, const double
   nb::Shape sh;
   sh.bt = nb::force_block_threads(NBODY_FP64);
   sh.t = nb::force_tile(NBODY_FP64);
-  sh.r = 4;
-  while (sh.r > 1 && (int64_t)sh.bt * sh.r * sms > n) sh.r >>= 1;
-  const int64_t bx = (n + (int64_t)sh.bt * sh.r - 1) / ((int64_t)sh.bt * sh.r);
+  sh.r = 1;
+  if (n < nb::force_split_max_n(NBODY_FP64)) sh.iw = nb::force_split(NBODY_FP64);
+  const int64_t bx = (n + sh.per_block() - 1) / sh.per_block();
   int occ = nb::force_max_blocks_per_sm(NBODY_FP64, sh);
   if (occ < 1) occ = 1;
   int64_t s = (8LL * sms * occ + bx - 1) / bx;
