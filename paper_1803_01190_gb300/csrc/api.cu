@@ -113,12 +113,19 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
   sh = nb::Shape();
   sh.bt = nb::force_block_threads(c->mode);
   sh.t = nb::force_tile(c->mode);
-  // measured on GB300: the FP64 kernel runs alike at R = 1 and 2 (131 and 127
-  // Gint/s at N = 65536); the packed FP32 and float-float kernels keep enough
-  // warps resident only at R = 2
-  int r = r_req ? r_req : (c->mode == NBODY_FP64 ? 1 : 2);
+  // measured on GB300 (Gint/s): FP64 R = 1, 2 at N = 65536 131, 127; MIXED R = 1,
+  // 2 at 16384 2247, 2253, at 12000 2067, 1919, at 65536 2548, 2601, at 131072
+  // 2605, 2735; FP32 R = 1, 2, 4 at 8192 1806, 1632, 1577, at 16384 2348, 2381,
+  // 2390, at 131072 2656, 2733, 2856; F64E keeps enough warps resident only at
+  // R = 2 and below one block per SM at R = 1
+  int r = r_req;
+  if (!r) switch (c->mode) {
+      case NBODY_FP64: r = 1; break;
+      case NBODY_MIXED: r = c->n < 16384 ? 1 : 2; break;
+      case NBODY_FP32: r = c->n < 16384 ? 1 : 4; break;
+      default: r = (int64_t)sh.bt * 2 * c->num_sms > c->n ? 1 : 2;
+    }
   if (c->mode == NBODY_F64E && r > 4) r = 4;
-  while (!r_req && r > 1 && (int64_t)sh.bt * r * c->num_sms > c->n) r >>= 1;
   sh.r = r;
   // small n: with one i-particle per thread and one tile per block there are
   // still fewer warps than hide the latency of a pair; split the tiles over

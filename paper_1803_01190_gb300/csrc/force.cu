@@ -222,6 +222,13 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float b) {
   lo = __fadd_rn(lo, err);
 }
 
+// a += s m, the product with its rounding error (m = 1: exactly a += s).
+__device__ __forceinline__ void fold_tile(float &hi, float &lo, float s, float m) {
+  const float p = __fmul_rn(s, m);
+  two_sum_acc(hi, lo, p);
+  lo = __fadd_rn(lo, __fmaf_rn(s, m, -p));
+}
+
 // ---------------------------------------------------------------- work descriptors
 // A kernel runs units k = first(), first() + stride(), ... < count().
 // Dense: one system of n particles; block (x, y) = i-block x of the rows
@@ -1105,7 +1112,11 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 // on the disk + halo and uniform-sphere workloads, the step changed the RMS force
 // error of the mixed kernel by less than 0.2 % (coordinate rounding and
 // accumulation dominate) while costing 26 % of its throughput.
-template <bool MASK, bool REFINE>
+// EQUAL leaves the mass out: the sums are those of 1/r^3 and 1/r, multiplied by
+// the tile's one mass when they are folded: 12 lane operations instead of 13.
+// Measured at N = 131072: MIXED 2735 Gint/s against 2545, FP32 (R = 2) 2731
+// against 2620.
+template <bool MASK, bool REFINE, bool EQUAL = false>
 __device__ __forceinline__ void body_pair(const float4 &A, const float4 &B, float2 nx, float2 ny,
                                           float2 nz, float2 e2, float2 &ax, float2 &ay,
                                           float2 &az, float2 &pt, bool self0, bool self1) {
@@ -1129,7 +1140,7 @@ __device__ __forceinline__ void body_pair(const float4 &A, const float4 &B, floa
     const float2 e = __ffma2_rn(__fmul2_rn(r2, y), y, f2(-1.0f, -1.0f));
     y = __ffma2_rn(__fmul2_rn(y, f2(-0.5f, -0.5f)), e, y);
   }
-  const float2 my = __fmul2_rn(m, y);
+  const float2 my = EQUAL ? y : __fmul2_rn(m, y);
   const float2 f = __fmul2_rn(my, __fmul2_rn(y, y));
   ax = __ffma2_rn(dx, f, ax);
   ay = __ffma2_rn(dy, f, ay);
@@ -1632,7 +1643,8 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
 
 // ---------------------------------------------------------------- mixed
 // fpos[j] = (x_j - c_t, y_j - c_t, z_j - c_t, m_j) in binary32, c_t the anchor of
-// j's tile; anchor[2t] = float hi part of c_t, anchor[2t+1] = float lo part.
+// j's tile; anchor[2t] = float hi part of c_t, anchor[2t+1] = float lo part;
+// anchor[2t].w = the mass of a full tile of equal masses, or 0.
 template <int BT, int R, int T, class W>
 __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
                                                     const float4 *__restrict__ fpos,
@@ -1680,7 +1692,17 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
       }
       const int np = (cnt + 1) / 2;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      if (cnt == T && !diag) {
+      const bool equal = ch.w != 0.0f;
+      if (cnt == T && !diag && equal) {
+#pragma unroll(R == 1 ? 2 : 4)
+        for (int k = 0; k < T / 2; k++) {
+          const float4 A = tA[k], B = tB[k];
+#pragma unroll
+          for (int r = 0; r < R; r++)
+            body_pair<false, false, true>(A, B, nx[r], ny[r], nz[r], e2, sx[r], sy[r], sz[r],
+                                         sp[r], false, false);
+        }
+      } else if (cnt == T && !diag) {
 // unroll 2 / 4 measured at N = 131072: R = 1 2446 / 2406 Gint/s, R = 2 2500 / 2517
 #pragma unroll(R == 1 ? 2 : 4)
         for (int k = 0; k < T / 2; k++) {
@@ -1703,12 +1725,13 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
           }
         }
       }
+      const float m = cnt == T && !diag && equal ? ch.w : 1.0f;
 #pragma unroll
       for (int r = 0; r < R; r++) {
-        two_sum_acc(axh[r], axl[r], __fadd_rn(sx[r].x, sx[r].y));
-        two_sum_acc(ayh[r], ayl[r], __fadd_rn(sy[r].x, sy[r].y));
-        two_sum_acc(azh[r], azl[r], __fadd_rn(sz[r].x, sz[r].y));
-        two_sum_acc(pth[r], ptl[r], __fadd_rn(sp[r].x, sp[r].y));
+        fold_tile(axh[r], axl[r], __fadd_rn(sx[r].x, sx[r].y), m);
+        fold_tile(ayh[r], ayl[r], __fadd_rn(sy[r].x, sy[r].y), m);
+        fold_tile(azh[r], azl[r], __fadd_rn(sz[r].x, sz[r].y), m);
+        fold_tile(pth[r], ptl[r], __fadd_rn(sp[r].x, sp[r].y), m);
       }
     }
 #pragma unroll
@@ -1842,10 +1865,12 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
       fpos[j0 + tid] = make_float4(hx, hy, hz, hm);
     }
   }
+  const bool equal = __syncthreads_and(
+      tid < cnt && __double_as_longlong(p.w) == __double_as_longlong(posm[j0].w));
   if (tid == 0) {
     const float hx = __double2float_rn(c[0]), hy = __double2float_rn(c[1]),
                 hz = __double2float_rn(c[2]);
-    anchor[2 * t] = make_float4(hx, hy, hz, 0.0f);
+    anchor[2 * t] = make_float4(hx, hy, hz, equal ? __double2float_rn(p.w) : 0.0f);
     anchor[2 * t + 1] = make_float4(__double2float_rn(c[0] - (double)hx),
                                     __double2float_rn(c[1] - (double)hy),
                                     __double2float_rn(c[2] - (double)hz), 0.0f);
@@ -1880,10 +1905,33 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
       const int cnt = (int)min((int64_t)T, j1 - jt);
       __syncthreads();
       load_pairs<BT, T>(posm, jt, cnt, tA, tB);
-      __syncthreads();
+      const float m = posm[jt].w;
+      const bool equal = __syncthreads_and(tid < cnt && posm[jt + min(tid, cnt - 1)].w == m);
       const int np = (cnt + 1) / 2;
       const int k0 = np * jw / IW, k1 = np * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
+      if (cnt == T && !diag && equal) {
+        float2 sx[R], sy[R], sz[R], sp[R];
+#pragma unroll
+        for (int r = 0; r < R; r++) sx[r] = sy[r] = sz[r] = sp[r] = f2(0.0f, 0.0f);
+#pragma unroll 2
+        for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
+          const float4 A = tA[k], B = tB[k];
+#pragma unroll
+          for (int r = 0; r < R; r++)
+            body_pair<false, false, true>(A, B, nx[r], ny[r], nz[r], e2, sx[r], sy[r], sz[r],
+                                         sp[r], false, false);
+        }
+        const float2 m2 = f2(m, m);
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+          ax[r] = __ffma2_rn(sx[r], m2, ax[r]);
+          ay[r] = __ffma2_rn(sy[r], m2, ay[r]);
+          az[r] = __ffma2_rn(sz[r], m2, az[r]);
+          pt[r] = __ffma2_rn(sp[r], m2, pt[r]);
+        }
+        continue;
+      }
       if (cnt == T && !diag) {
 #pragma unroll 2
         for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
