@@ -41,7 +41,8 @@
 //   f64e  binary64-class accuracy on the binary32 pipes: float-float (about 48
 //         significant bits) pair arithmetic on coordinates re-centred per
 //         j-tile, float-float tile partials folded into binary64 per tile.
-//         About 160 binary32 instructions per pair, but on pipes 64 times
+//         About 134 to 146 binary32 operations per pair (84 to 96 per
+//         interaction when each pair is evaluated once), but on pipes 64 times
 //         faster than GB300's FP64 pipe.  From 64 blocks of 256 particles it
 //         evaluates each pair once for both particles (k_force_f64e_sym).
 //   f32   binary32 throughout (packed pairs, SFU reciprocal square root) with
@@ -233,24 +234,24 @@ __device__ __forceinline__ void fold_tile(float &hi, float &lo, float s, float m
 // A kernel runs units k = first(), first() + stride(), ... < count().
 // Dense: one system of n particles; block (x, y) = i-block x of the rows
 // [i_base, i_base + rows) against j-segment y of all n; the row sums go to
-// part[y * rows + (i - i_base)] (all rows: i_base = 0, rows = n).  aligned:
-// i-blocks start at multiples of per_block whatever i_base is (the binary64
-// kernel's unit depends on the particles of the whole i-block, so a row's sum
-// is the same, bit for bit, whichever rows are asked for); only the rows
-// asked for are written.
+// part[y * rows + (i - i_base)] (all rows: i_base = 0, rows = n).  i-blocks
+// start at multiples of per_block whatever i_base is: how a tile is summed
+// depends on the whole i-block (the unit of the fixed-point sums; whether the
+// tile holds some of the block's own particles), so a row's sum is the same,
+// bit for bit, whichever rows are asked for.  Only the rows asked for are
+// written.
 struct DenseWork {
   int64_t n, seg, i_base, rows;
   double eps2;
   int per_block, tile;
-  bool aligned;
   __device__ __forceinline__ int64_t first() const { return 0; }
   __device__ __forceinline__ int64_t stride() const { return 1; }
   __device__ __forceinline__ int64_t count() const { return 1; }
   __device__ __forceinline__ Unit get(int64_t) const {
     Unit u;
-    const int64_t r0 = (int64_t)blockIdx.x * per_block - (aligned ? i_base % per_block : 0);
+    const int64_t r0 = (int64_t)blockIdx.x * per_block - i_base % per_block;
     u.i0 = i_base + r0;
-    u.ni = (int)min((int64_t)per_block, (aligned ? n - i_base : rows) - r0);
+    u.ni = (int)min((int64_t)per_block, n - i_base - r0);
     u.w0 = (int)max((int64_t)0, -r0);
     u.w1 = (int)min((int64_t)u.ni, rows - r0);
     u.j0 = (int64_t)blockIdx.y * seg;
@@ -273,11 +274,11 @@ struct TableWork {
   __device__ __forceinline__ Unit get(int64_t k) const { return units[k]; }
 };
 
-// Writes the sums v of i-particle li (< ni).  IW > 1: the IW threads that share
+// Writes the sums v of i-particle li of the unit u.  IW > 1: the IW threads that share
 // it (thread `it` of IT, share jw) add theirs in order first.
 template <int IW, class V>
-__device__ __forceinline__ void store_shares(V *out, int li, int ni, V v, V *red, int it, int IT,
-                                             int jw) {
+__device__ __forceinline__ void store_shares(V *part, const Unit &u, int li, V v, V *red, int it,
+                                             int IT, int jw) {
   if (IW > 1) {
     __syncthreads();
     red[threadIdx.x] = v;
@@ -292,7 +293,7 @@ __device__ __forceinline__ void store_shares(V *out, int li, int ni, V v, V *red
       v.w += o.w;
     }
   }
-  if (li < ni) out[li] = v;
+  if (li >= u.w0 && li < min(u.ni, u.w1)) part[u.out + li] = v;
 }
 
 // ---------------------------------------------------------------- binary64
@@ -1232,88 +1233,112 @@ __device__ __forceinline__ double join_ff(float h, float l) {
   return finite ? f2d_exact(h) + f2d_exact(l) : (double)h + (double)l;
 }
 
-// One tile entry: j = 2k, 2k+1 as H = (xh0, xh1, yh0, yh1), H2 = (zh0, zh1, mh0, mh1),
-// L, L2 the matching low parts.  (nxh, nxl, ...) are the negated float-float
-// i coordinates in both halves; the four float-float accumulators get the
-// terms m_j d_ij / w_ij (x, y, z) and m_j / sqrt(d^2 + eps^2).
+// A pair's geometry: d, y = 1/r and q = 1/r^2 as float-float, for one tile entry
+// (j = 2k, 2k+1 as H = (xh0, xh1, yh0, yh1), H2 = (zh0, zh1, mh0, mh1), L, L2 the
+// matching low parts) and the negated float-float i coordinates (nxh, ...) in
+// both halves.
+//   d = (jh - ih) + (jl - il): TwoSum of the high parts, then Fast2Sum with the
+//     low ones.  Fast2Sum(s, t) is exact here although |t| may exceed |s| after
+//     cancellation: s is then a multiple of the smaller ulp of jh and ih, t is
+//     below two of it, so s is a multiple of ulp(t), which is all it needs.
+//   y = r2^{-1/2}: SFU seed y0, residual e = 1 - r2 y0^2 in float-float,
+//     y = y0 (1 + e/2 + 3 e^2 / 8) = y0 + y0 e (1/2 + 3e/8).
+struct FfPair {
+  float2 dh[3], dl[3], y0, yl, q, ql, r2h, r2l;
+};
 template <bool MASK>
-__device__ __forceinline__ void body_ff(const float4 &H, const float4 &H2, const float4 &L,
-                                        const float4 &L2, float2 nxh, float2 nxl, float2 nyh,
-                                        float2 nyl, float2 nzh, float2 nzl, float2 e2h, float2 e2l,
-                                        float2 (&ah)[4], float2 (&al)[4], bool self0, bool self1) {
-  float2 dh[3], dl[3];
-  {
-    const float2 jh[3] = {f2(H.x, H.y), f2(H.z, H.w), f2(H2.x, H2.y)};
-    const float2 jl[3] = {f2(L.x, L.y), f2(L.z, L.w), f2(L2.x, L2.y)};
-    const float2 ih[3] = {nxh, nyh, nzh}, il[3] = {nxl, nyl, nzl};
-#pragma unroll
-    for (int c = 0; c < 3; c++) {  // d = (jh + jl) - (ih + il), renormalised
-      float2 s, e;
-      two_sum2(jh[c], ih[c], s, e);
-      const float2 t = __fadd2_rn(__fadd2_rn(jl[c], il[c]), e);
-      two_sum2(s, t, dh[c], dl[c]);
-    }
-  }
-  // r2 = |d|^2 + eps^2
-  float2 p[3], pe[3];
+__device__ __forceinline__ void ff_geometry(const float4 &H, const float4 &H2, const float4 &L,
+                                            const float4 &L2, const float2 (&nh)[3],
+                                            const float2 (&nl)[3], float2 e2h, float2 e2l,
+                                            bool self0, bool self1, FfPair &g) {
+  const float2 jh[3] = {f2(H.x, H.y), f2(H.z, H.w), f2(H2.x, H2.y)};
+  const float2 jl[3] = {f2(L.x, L.y), f2(L.z, L.w), f2(L2.x, L2.y)};
+  float2 p[3], pe[3], cross;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    two_prod2(dh[c], dh[c], p[c], pe[c]);
-    pe[c] = __ffma2_rn(__fadd2_rn(dh[c], dh[c]), dl[c], pe[c]);
+    float2 s, e;
+    two_sum2(jh[c], nh[c], s, e);
+    const float2 t = __fadd2_rn(__fadd2_rn(jl[c], nl[c]), e);
+    fast_two_sum2(s, t, g.dh[c], g.dl[c]);
+    two_prod2(g.dh[c], g.dh[c], p[c], pe[c]);
+    cross = c == 0 ? __fmul2_rn(g.dh[c], g.dl[c]) : __ffma2_rn(g.dh[c], g.dl[c], cross);
   }
+  // r2 = |d|^2 + eps^2
   float2 s1, e1, s2, e2, s3, e3;
   two_sum2(p[0], p[1], s1, e1);
   two_sum2(s1, p[2], s2, e2);
   two_sum2(s2, e2h, s3, e3);
-  const float2 lo = __fadd2_rn(__fadd2_rn(__fadd2_rn(pe[0], pe[1]), __fadd2_rn(pe[2], e2l)),
-                               __fadd2_rn(__fadd2_rn(e1, e2), e3));
+  const float2 lo =
+      __ffma2_rn(cross, f2(2.0f, 2.0f),
+                 __fadd2_rn(__fadd2_rn(__fadd2_rn(pe[0], pe[1]), __fadd2_rn(pe[2], e2l)),
+                            __fadd2_rn(__fadd2_rn(e1, e2), e3)));
   float2 r2h, r2l;
   fast_two_sum2(s3, lo, r2h, r2l);
-  float2 mh = f2(H2.z, H2.w), ml = f2(L2.z, L2.w);
   if (MASK) {
-    if (self0) {
-      r2h.x = 1.0f;
-      r2l.x = 0.0f;
-      mh.x = ml.x = 0.0f;
-    }
-    if (self1) {
-      r2h.y = 1.0f;
-      r2l.y = 0.0f;
-      mh.y = ml.y = 0.0f;
-    }
+    if (self0) r2h.x = 1.0f, r2l.x = 0.0f;
+    if (self1) r2h.y = 1.0f, r2l.y = 0.0f;
   }
-  // y = r2^{-1/2}: SFU seed y0, residual e = 1 - r2 y0^2 in float-float,
-  // y = y0 (1 + e/2 + 3 e^2 / 8) = y0 + y0 e (1/2 + 3e/8)
   const float2 y0 = f2(rsqrt_approx(r2h.x), rsqrt_approx(r2h.y));
   float2 th, tl, u, ue;
   two_prod2(y0, y0, th, tl);
   two_prod2(r2h, th, u, ue);
-  const float2 cross = __ffma2_rn(r2h, tl, __fmul2_rn(r2l, th));
-  const float2 e = fsub2(fsub2(fsub2(f2(1.0f, 1.0f), u), ue), cross);
-  const float2 yl = __fmul2_rn(__fmul2_rn(y0, e), __ffma2_rn(e, f2(0.375f, 0.375f), f2(0.5f, 0.5f)));
-  // q = y^2, a = m y, b = a q = m y^3
-  float2 q, qe, a, ae, b, be;
-  two_prod2(y0, y0, q, qe);
-  const float2 ql = __ffma2_rn(__fadd2_rn(y0, y0), yl, qe);
-  two_prod2(mh, y0, a, ae);
-  const float2 al_ = __ffma2_rn(mh, yl, __ffma2_rn(ml, y0, ae));
-  two_prod2(a, q, b, be);
-  const float2 bl = __ffma2_rn(a, ql, __ffma2_rn(al_, q, be));
-  // accumulate d b (three components) and a
+  const float2 e = fsub2(fsub2(f2(1.0f, 1.0f), u), __ffma2_rn(r2h, tl, __ffma2_rn(r2l, th, ue)));
+  g.y0 = y0;
+  g.yl = __fmul2_rn(__fmul2_rn(y0, e), __ffma2_rn(e, f2(0.375f, 0.375f), f2(0.5f, 0.5f)));
+  g.q = th;
+  g.ql = __ffma2_rn(__fadd2_rn(y0, y0), g.yl, tl);
+}
+
+// The four terms of one side, d b (three components) and a, with a = m y and
+// b = a q; EQUAL: without the mass, the same for both sides.
+struct FfTerms {
+  float2 h[4], l[4];
+};
+template <bool EQUAL>
+__device__ __forceinline__ void ff_terms(const FfPair &g, float2 mh, float2 ml, FfTerms &t) {
+  float2 a = g.y0, al = g.yl, ae, b, be;
+  if (!EQUAL) {
+    two_prod2(mh, g.y0, a, ae);
+    al = __ffma2_rn(mh, g.yl, __ffma2_rn(ml, g.y0, ae));
+  }
+  two_prod2(a, g.q, b, be);
+  const float2 bl = __ffma2_rn(a, g.ql, __ffma2_rn(al, g.q, be));
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    float2 ce;
+    two_prod2(g.dh[c], b, t.h[c], ce);
+    t.l[c] = __ffma2_rn(g.dh[c], bl, __ffma2_rn(g.dl[c], b, ce));
+  }
+  t.h[3] = a;
+  t.l[3] = al;
+}
+
+// (h, l) += t: the high parts by TwoSum, the rest into the low part.  The sums
+// are renormalised (ff_renorm) every few terms, not after each, which saves 3
+// of 11 operations a term: the low part then grows to a few ulps of the high
+// one.  Every 4 terms for the accelerations, whose error is that of the
+// coordinates; every 2 for the potentials, whose error is that of the sum.
+// Measured each pair once, N = 65536, equal masses (Gint/s, relative error of
+// the potentials): every term 375, 7.0e-16; all every 2: 400, 7.1e-16; all every
+// 4: 411, 7.4e-16; every 8: 410, 8.0e-16; 303, 6.9e-16 before this and the shared
+// terms; unequal masses 355 every 4.
+__device__ __forceinline__ void ff_add(const FfTerms &t, float2 (&h)[4], float2 (&l)[4]) {
 #pragma unroll
   for (int c = 0; c < 4; c++) {
-    float2 th2, tl2;
-    if (c < 3) {
-      float2 ce;
-      two_prod2(dh[c], b, th2, ce);
-      tl2 = __ffma2_rn(dh[c], bl, __ffma2_rn(dl[c], b, ce));
-    } else {
-      th2 = a;
-      tl2 = al_;
-    }
     float2 s, es;
-    two_sum2(ah[c], th2, s, es);
-    fast_two_sum2(s, __fadd2_rn(al[c], __fadd2_rn(es, tl2)), ah[c], al[c]);
+    two_sum2(h[c], t.h[c], s, es);
+    h[c] = s;
+    l[c] = __fadd2_rn(l[c], __fadd2_rn(es, t.l[c]));
+  }
+}
+template <int C0 = 0>
+__device__ __forceinline__ void ff_renorm(float2 (&h)[4], float2 (&l)[4]) {
+#pragma unroll
+  for (int c = C0; c < 4; c++) {
+    float2 s, e;
+    fast_two_sum2(h[c], l[c], s, e);
+    h[c] = s;
+    l[c] = e;
   }
 }
 
@@ -1332,6 +1357,36 @@ __device__ __forceinline__ void load_pairs_ff(const float4 *__restrict__ src, in
     tH2[k] = make_float4(ah.z, bh.z, ah.w, bh.w);
     tL[k] = make_float4(alo.x, blo.x, alo.y, blo.y);
     tL2[k] = make_float4(alo.z, blo.z, alo.w, blo.w);
+  }
+}
+
+// Terms between renormalisations of the acceleration sums.
+constexpr int FF_STEPS = 4;
+
+template <int R, bool EQUAL>
+__device__ __forceinline__ void ff_tile(const float4 *tH, const float4 *tH2, const float4 *tL,
+                                        const float4 *tL2, int k0, int k1,
+                                        const float2 (&nh)[R][3], const float2 (&nl)[R][3],
+                                        float2 e2h, float2 e2l, float2 (&ah)[R][4],
+                                        float2 (&al)[R][4]) {
+#pragma unroll 1
+  for (int k = k0; k < k1; k += FF_STEPS) {
+#pragma unroll
+    for (int q = 0; q < FF_STEPS; q++) {
+      const float4 H = tH[k + q], H2 = tH2[k + q], L = tL[k + q], L2 = tL2[k + q];
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        FfPair g;
+        FfTerms t;
+        ff_geometry<false>(H, H2, L, L2, nh[r], nl[r], e2h, e2l, false, false, g);
+        ff_terms<EQUAL>(g, f2(H2.z, H2.w), f2(L2.z, L2.w), t);
+        ff_add(t, ah[r], al[r]);
+        if (q == FF_STEPS - 1)
+          ff_renorm(ah[r], al[r]);
+        else if (q % 2 == 1)
+          ff_renorm<3>(ah[r], al[r]);
+      }
+    }
   }
 }
 
@@ -1396,14 +1451,12 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
       const int np = (cnt + 1) / 2;
       const int k0 = np * jw / IW, k1 = np * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      if (cnt == T && !diag) {
-        for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
-          const float4 H = tH[k], H2 = tH2[k], L = tL[k], L2 = tL2[k];
-#pragma unroll
-          for (int r = 0; r < R; r++)
-            body_ff<false>(H, H2, L, L2, nh[r][0], nl[r][0], nh[r][1], nl[r][1], nh[r][2],
-                           nl[r][2], e2h, e2l, ah[r], al[r], false, false);
-        }
+      const bool full = cnt == T && !diag, equal = full && ch.w != 0.0f;
+      if (full) {  // k1 - k0 is a multiple of FF_STEPS
+        if (equal)
+          ff_tile<R, true>(tH, tH2, tL, tL2, k0, k1, nh, nl, e2h, e2l, ah, al);
+        else
+          ff_tile<R, false>(tH, tH2, tL, tL2, k0, k1, nh, nl, e2h, e2l, ah, al);
       } else {
         for (int k = k0; k < k1; k++) {
           const float4 H = tH[k], H2 = tH2[k], L = tL[k], L2 = tL2[k];
@@ -1411,11 +1464,18 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
 #pragma unroll
           for (int r = 0; r < R; r++) {
             const int64_t i = u.i0 + r * IT + it;
-            body_ff<true>(H, H2, L, L2, nh[r][0], nl[r][0], nh[r][1], nl[r][1], nh[r][2],
-                          nl[r][2], e2h, e2l, ah[r], al[r], j == i, j + 1 == i);
+            const bool self0 = diag && j == i, self1 = diag && j + 1 == i;
+            FfPair g;
+            FfTerms t;
+            ff_geometry<true>(H, H2, L, L2, nh[r], nl[r], e2h, e2l, self0, self1, g);
+            ff_terms<false>(g, f2(self0 ? 0.0f : H2.z, self1 ? 0.0f : H2.w),
+                            f2(self0 ? 0.0f : L2.z, self1 ? 0.0f : L2.w), t);
+            ff_add(t, ah[r], al[r]);
+            ff_renorm(ah[r], al[r]);
           }
         }
       }
+      const double m = equal ? posm[jt].w : 1.0;
       // fold the tile: even + odd lanes in float-float, then into binary64
 #pragma unroll
       for (int r = 0; r < R; r++)
@@ -1424,97 +1484,83 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
           float s, e;
           two_sum1(ah[r][c].x, ah[r][c].y, s, e);
           const float l = __fadd_rn(__fadd_rn(al[r][c].x, al[r][c].y), e);
-          acc[r][c] += f2d_exact(s) + f2d_exact(l);
+          acc[r][c] = fma(f2d_exact(s) + f2d_exact(l), m, acc[r][c]);
         }
     }
 #pragma unroll
     for (int r = 0; r < R; r++) {
       const int li = r * IT + it;
       const d4 v = {acc[r][0], acc[r][1], acc[r][2], acc[r][3]};
-      store_shares<IW>(part + u.out, li, u.ni, v, red, it, IT, jw);
+      store_shares<IW>(part, work.get(uk), li, v, red, it, IT, jw);
     }
   }
 }
 
 // ---------------------------------------------------------------- float-float, each pair once
-// The F64E pair body evaluated once for both particles (Newton's third law):
-// the difference, |d|^2 + eps^2, y = 1/r and q = y^2 are shared; the i side
-// gets m_j y and m_j y q, the j side m_i y and m_i y q with -d.  Two
-// j-particles per packed instruction (one tile entry); the j side's four
-// float-float sums for an entry are (gh, gl).
-__device__ __forceinline__ void body_ff_sym(const float4 &H, const float4 &H2, const float4 &L,
-                                            const float4 &L2, float2 nxh, float2 nxl,
-                                            float2 nyh, float2 nyl, float2 nzh, float2 nzl,
-                                            float2 mih, float2 mil, float2 e2h, float2 e2l,
-                                            float2 (&ah)[4], float2 (&al)[4], float2 (&gh)[4],
-                                            float2 (&gl)[4]) {
-  float2 dh[3], dl[3];
-  {
-    const float2 jh[3] = {f2(H.x, H.y), f2(H.z, H.w), f2(H2.x, H2.y)};
-    const float2 jl[3] = {f2(L.x, L.y), f2(L.z, L.w), f2(L2.x, L2.y)};
-    const float2 ih[3] = {nxh, nyh, nzh}, il[3] = {nxl, nyl, nzl};
-#pragma unroll
-    for (int c = 0; c < 3; c++) {  // d = (jh + jl) - (ih + il), renormalised
-      float2 s, e;
-      two_sum2(jh[c], ih[c], s, e);
-      const float2 t = __fadd2_rn(__fadd2_rn(jl[c], il[c]), e);
-      two_sum2(s, t, dh[c], dl[c]);
-    }
-  }
-  float2 p[3], pe[3];
-#pragma unroll
-  for (int c = 0; c < 3; c++) {
-    two_prod2(dh[c], dh[c], p[c], pe[c]);
-    pe[c] = __ffma2_rn(__fadd2_rn(dh[c], dh[c]), dl[c], pe[c]);
-  }
-  float2 s1, e1, s2, e2, s3, e3;
-  two_sum2(p[0], p[1], s1, e1);
-  two_sum2(s1, p[2], s2, e2);
-  two_sum2(s2, e2h, s3, e3);
-  const float2 lo = __fadd2_rn(__fadd2_rn(__fadd2_rn(pe[0], pe[1]), __fadd2_rn(pe[2], e2l)),
-                               __fadd2_rn(__fadd2_rn(e1, e2), e3));
-  float2 r2h, r2l;
-  fast_two_sum2(s3, lo, r2h, r2l);
-  const float2 y0 = f2(rsqrt_approx(r2h.x), rsqrt_approx(r2h.y));
-  float2 th, tl, u, ue;
-  two_prod2(y0, y0, th, tl);
-  two_prod2(r2h, th, u, ue);
-  const float2 cross = __ffma2_rn(r2h, tl, __fmul2_rn(r2l, th));
-  const float2 e = fsub2(fsub2(fsub2(f2(1.0f, 1.0f), u), ue), cross);
-  const float2 yl = __fmul2_rn(__fmul2_rn(y0, e), __ffma2_rn(e, f2(0.375f, 0.375f), f2(0.5f, 0.5f)));
-  float2 q, qe;
-  two_prod2(y0, y0, q, qe);
-  const float2 ql = __ffma2_rn(__fadd2_rn(y0, y0), yl, qe);
-  // one side: a = m y, b = a q, sums += (sgn d b, a)
-  auto side = [&](float2 mh, float2 ml, bool neg, float2(&sh)[4], float2(&sl)[4]) {
-    float2 a, ae, b, be;
-    two_prod2(mh, y0, a, ae);
-    const float2 al_ = __ffma2_rn(mh, yl, __ffma2_rn(ml, y0, ae));
-    two_prod2(a, q, b, be);
-    const float2 bl = __ffma2_rn(a, ql, __ffma2_rn(al_, q, be));
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      float2 th2, tl2;
-      if (c < 3) {
-        const float2 dhc = neg ? neg2(dh[c]) : dh[c], dlc = neg ? neg2(dl[c]) : dl[c];
-        float2 ce;
-        two_prod2(dhc, b, th2, ce);
-        tl2 = __ffma2_rn(dhc, bl, __ffma2_rn(dlc, b, ce));
-      } else {
-        th2 = a;
-        tl2 = al_;
-      }
-      float2 s, es;
-      two_sum2(sh[c], th2, s, es);
-      fast_two_sum2(s, __fadd2_rn(sl[c], __fadd2_rn(es, tl2)), sh[c], sl[c]);
-    }
-  };
-  side(f2(H2.z, H2.w), f2(L2.z, L2.w), false, ah, al);
-  side(mih, mil, true, gh, gl);
-}
-
+// The F64E pair evaluated once for both particles (Newton's third law): the
+// geometry (d, |d|^2 + eps^2, 1/r, 1/r^2) is shared; the i side gets the terms
+// with m_j, the j side those with m_i and -d (the sign is applied to the column
+// sums at the end).  Equal masses in both blocks share the terms as well.  Two
+// j-particles per packed instruction (one tile entry).
 __device__ __forceinline__ float2 shfl2(float2 v, int src) {
   return f2(__shfl_sync(0xFFFFFFFFu, v.x, src), __shfl_sync(0xFFFFFFFFu, v.y, src));
+}
+
+// The column block's NE entries against the R i-particles of each thread: row
+// sums in (ah, al), the warp's column sums into colw (binary64).
+template <int R, int NE, int T, bool EQUAL>
+__device__ __forceinline__ void ff_sym_tile(const float4 *tH, const float4 *tH2, const float4 *tL,
+                                            const float4 *tL2, const float2 (&nh)[R][3],
+                                            const float2 (&nl)[R][3], const float2 (&mh)[R],
+                                            const float2 (&ml)[R], float2 e2h, float2 e2l,
+                                            float2 (&ah)[R][4], float2 (&al)[R][4],
+                                            double (*colw)[T]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int c0 = 0; c0 < NE; c0 += 32) {
+    float2 gh[4], gl[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) gh[c] = gl[c] = f2(0.0f, 0.0f);
+#pragma unroll 1
+    for (int k = 0; k < 32; k += FF_STEPS) {
+#pragma unroll
+      for (int s = 0; s < FF_STEPS; s++) {
+        const int ent = c0 + ((lane + k + s) & 31);
+        const float4 H = tH[ent], H2 = tH2[ent], L = tL[ent], L2 = tL2[ent];
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+          FfPair g;
+          FfTerms t;
+          ff_geometry<false>(H, H2, L, L2, nh[r], nl[r], e2h, e2l, false, false, g);
+          ff_terms<EQUAL>(g, f2(H2.z, H2.w), f2(L2.z, L2.w), t);
+          ff_add(t, ah[r], al[r]);
+          if (!EQUAL) ff_terms<false>(g, mh[r], ml[r], t);
+          ff_add(t, gh, gl);
+        }
+        if (s == FF_STEPS - 1) {
+          ff_renorm(gh, gl);
+#pragma unroll
+          for (int r = 0; r < R; r++) ff_renorm(ah[r], al[r]);
+        } else if (s % 2 == 1) {
+          ff_renorm<3>(gh, gl);
+#pragma unroll
+          for (int r = 0; r < R; r++) ff_renorm<3>(ah[r], al[r]);
+        }
+        const int src = (lane + 1) & 31;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          gh[c] = shfl2(gh[c], src);
+          gl[c] = shfl2(gl[c], src);
+        }
+      }
+    }
+    // lane holds entry c0 + lane (j = 2 (c0 + lane) and 2 (c0 + lane) + 1)
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      colw[c][2 * (c0 + lane)] = f2d_exact(gh[c].x) + f2d_exact(gl[c].x);
+      colw[c][2 * (c0 + lane) + 1] = f2d_exact(gh[c].y) + f2d_exact(gl[c].y);
+    }
+  }
 }
 
 // Work item (d, I) of the block-diagonal schedule of k_force_f64_sym with
@@ -1587,34 +1633,13 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
     for (int c = 0; c < 4; c++) ah[r][c] = al[r][c] = f2(0.0f, 0.0f);
   }
   __syncthreads();
-#pragma unroll 1
-  for (int c0 = 0; c0 < NE; c0 += 32) {
-    float2 gh[4], gl[4];
-#pragma unroll
-    for (int c = 0; c < 4; c++) gh[c] = gl[c] = f2(0.0f, 0.0f);
-#pragma unroll 1
-    for (int k = 0; k < 32; k++) {
-      const int ent = c0 + ((lane + k) & 31);
-      const float4 H = tH[ent], H2 = tH2[ent], L = tL[ent], L2 = tL2[ent];
-#pragma unroll
-      for (int r = 0; r < R; r++)
-        body_ff_sym(H, H2, L, L2, nh[r][0], nl[r][0], nh[r][1], nl[r][1], nh[r][2], nl[r][2],
-                    mh[r], ml[r], e2h, e2l, ah[r], al[r], gh, gl);
-      const int src = (lane + 1) & 31;
-#pragma unroll
-      for (int c = 0; c < 4; c++) {
-        gh[c] = shfl2(gh[c], src);
-        gl[c] = shfl2(gl[c], src);
-      }
-    }
-    // lane holds entry c0 + lane (j = 2 (c0 + lane) and 2 (c0 + lane) + 1)
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      colw[warp][c][2 * (c0 + lane)] = f2d_exact(gh[c].x) + f2d_exact(gl[c].x);
-      colw[warp][c][2 * (c0 + lane) + 1] = f2d_exact(gh[c].y) + f2d_exact(gl[c].y);
-    }
-  }
+  const bool equal = ch.w != 0.0f && anchor[2 * I].w != 0.0f;
+  if (equal)
+    ff_sym_tile<R, NE, T, true>(tH, tH2, tL, tL2, nh, nl, mh, ml, e2h, e2l, ah, al, colw[warp]);
+  else
+    ff_sym_tile<R, NE, T, false>(tH, tH2, tL, tL2, nh, nl, mh, ml, e2h, e2l, ah, al, colw[warp]);
   __syncthreads();
+  const double mj = equal ? posm[j0].w : 1.0, mi = equal ? posm[i0].w : 1.0;
   for (int k = tid; k < T; k += BT) {
     double v[4];
 #pragma unroll
@@ -1623,7 +1648,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
 #pragma unroll
       for (int w = 1; w < NW; w++) v[c] += colw[w][c][k];
     }
-    if (j0 + k < n) colo[j0 + k] = d4{v[0], v[1], v[2], v[3]};
+    if (j0 + k < n) colo[j0 + k] = d4{-v[0] * mi, -v[1] * mi, -v[2] * mi, v[3] * mi};
   }
   // rows: fold even + odd lanes in float-float, then into binary64
 #pragma unroll
@@ -1635,7 +1660,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
       float s, e;
       two_sum1(ah[r][c].x, ah[r][c].y, s, e);
       const float l = __fadd_rn(__fadd_rn(al[r][c].x, al[r][c].y), e);
-      v[c] = f2d_exact(s) + f2d_exact(l);
+      v[c] = (f2d_exact(s) + f2d_exact(l)) * mj;
     }
     if (i < n) rowo[i] = d4{v[0], v[1], v[2], v[3]};
   }
@@ -1737,8 +1762,9 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
 #pragma unroll
     for (int r = 0; r < R; r++) {
       const int li = r * BT + tid;
-      if (li < u.ni)
-        part[u.out + li] = d4{join_ff(axh[r], axl[r]), join_ff(ayh[r], ayl[r]),
+      const Unit w = work.get(uk);  // again: not kept in registers over the pair loop
+      if (li >= w.w0 && li < min(w.ni, w.w1))
+        part[w.out + li] = d4{join_ff(axh[r], axl[r]), join_ff(ayh[r], ayl[r]),
                               join_ff(azh[r], azl[r]), join_ff(pth[r], ptl[r])};
     }
   }
@@ -1959,7 +1985,7 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
       const int li = r * IT + it;
       const float4 v = make_float4(__fadd_rn(ax[r].x, ax[r].y), __fadd_rn(ay[r].x, ay[r].y),
                                    __fadd_rn(az[r].x, az[r].y), __fadd_rn(pt[r].x, pt[r].y));
-      store_shares<IW>(part + u.out, li, u.ni, v, red, it, IT, jw);
+      store_shares<IW>(part, work.get(uk), li, v, red, it, IT, jw);
     }
   }
 }
@@ -2129,8 +2155,7 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   if (!shape_supported(mode, sh) || in.n < 1 || rows < 1 || in.i0 < 0 || in.i0 + rows > in.n)
     return cudaErrorInvalidValue;
   const int64_t per_block = sh.per_block();
-  const bool aligned = mode == NBODY_FP64;
-  const int64_t gx = ((aligned ? in.i0 % per_block : 0) + rows + per_block - 1) / per_block;
+  const int64_t gx = (in.i0 % per_block + rows + per_block - 1) / per_block;
   if (gx > 0x7fffffff) return cudaErrorInvalidValue;
   DenseWork w;
   w.n = in.n;
@@ -2140,7 +2165,6 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   w.eps2 = in.eps2;
   w.per_block = (int)per_block;
   w.tile = sh.t;
-  w.aligned = aligned;
   const dim3 grid((unsigned)gx, (unsigned)sh.s);
   if (sh.iw > 1) {
     launch_rw<1, true>(mode, in.posm, in.fpos, in.anchor, w, grid, in.part, st);

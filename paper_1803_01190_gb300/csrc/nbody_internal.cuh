@@ -61,7 +61,7 @@ struct Unit {
   int64_t i0, j0, out, anchor;
   double eps2;
   int32_t ni, nj;
-  int32_t w0 = 0, w1 = 0x7FFFFFFF;  // FP64: only i0 + [w0, w1) is written
+  int32_t w0 = 0, w1 = 0x7FFFFFFF;  // only i0 + [w0, w1) is written
 };
 
 // One MIXED prep block: the tile [j0, j0+cnt) with anchor index `anchor`.

@@ -82,6 +82,23 @@ def _check(pos, mass, eps, acc, pot):
     assert np.all(np.abs(pot - op) <= 1e-12 * np.abs(op))
 
 
+@pytest.mark.parametrize("mode", ["fp64", "f64e", "mixed", "fp32"])
+@pytest.mark.parametrize("n", [1500, 20003])
+def test_rows_of_equal_masses(nb, mode, n):
+    """Row blocks that start inside i-blocks, with tiles of equal masses: bit for bit
+    the rows of one evaluation, whichever rows share a block."""
+    pos, _, mass = nbody_ics.plummer(n, 20180400)
+    with nb.Simulation(n, mode, eps=0.02) as sim:
+        if mode in ("fp64", "f64e"):
+            sim.set_symmetric(0)
+        if mode != "fp32":
+            sim.set_order("input")
+        acc, pot = sim.accel(pos, mass)
+        for i0, ni in ((0, 1), (1, n - 1), (333, 700), (n - 77, 77)):
+            a, p = sim.accel_rows(i0, ni, pos, mass)
+            assert np.array_equal(a, acc[i0:i0 + ni]) and np.array_equal(p, pot[i0:i0 + ni])
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 @pytest.mark.parametrize("where", ["pos", "mass"])
 def test_non_finite_input_gives_non_finite_output(nb, bad, where):
