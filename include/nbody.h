@@ -352,11 +352,11 @@ int nbody_batch_slot_info(nbody_batch *b, int slot, int64_t *n, int *mode, int64
  * is split into at most 16 segments).  Changes rounding order only. */
 int nbody_batch_set_launch(nbody_batch *b, int mode, int ipt, int64_t seg);
 
-/* FP64 force launches of this pool run as a persistent grid of at most
- * blocks_per_sm thread blocks per SM (default 2; 0 = one block per work unit).
- * FP64 work keeps the FP64 pipe busy with few warps; capping its residency
- * leaves the rest of each SM to FP32-bound work of other streams (for
- * instance a MIXED pool ticking at the same time). */
+/* Cap on the FP64 force launches of this pool: blocks_per_sm > 0 runs them as
+ * a persistent grid of at most that many thread blocks per SM, which leaves
+ * the rest of each SM to work of other streams (for instance a MIXED pool
+ * ticking at the same time); 0 (the default) runs one block per work unit.
+ * Results do not depend on it. */
 int nbody_batch_set_fp64_residency(nbody_batch *b, int blocks_per_sm);
 
 /* Per-tick CUDA-event timing (see nbody_batch_profile_read). */

@@ -159,9 +159,12 @@ struct nbody_batch {
   // host state
   std::vector<SimHost> sims;
   std::map<int64_t, int64_t> free_ranges;  // offset -> length
-  int r_mode[3] = {2, 2, 2};                 // R per kernel class (FP64, MIXED, F64E)
-  int fp64_per_sm = 2;                       // resident FP64 force blocks per SM (persistent grid)
-  int64_t seg_mode[3] = {4096, 8192, 4096};  // target j-segment length per class
+  // R and target j-segment length per kernel class (FP64, MIXED, F64E).  FP64
+  // measured on twelve simulations of 1000 to 27000 particles (ms a tick, one
+  // block per unit): R = 2, 4096: 8.9; R = 1, 4096: 8.3; R = 1, 2048: 7.6
+  int r_mode[3] = {1, 2, 2};
+  int fp64_per_sm = 0;  // most resident FP64 force blocks per SM (0: one block per unit)
+  int64_t seg_mode[3] = {2048, 8192, 4096};
   // profiling
   std::vector<cudaEvent_t> evs;  // 8 per tick: tick start/end, then start/end per class
   size_t ev_used = 0;
@@ -583,9 +586,12 @@ static int batch_step_impl(nbody_batch *b, int64_t nticks) {
     }
     if (b->n64) {
       if (b->prof) BCK(cudaEventRecord(e[2], b->st));
-      // FP64 blocks are long and need few warps to keep the FP64 pipe busy: a
-      // persistent grid of fp64_per_sm blocks per SM leaves the rest of each
-      // SM to FP32-bound work running on other streams (another pool's ticks)
+      // One block per unit by default: the fixed-point pair sums need the warps
+      // of a full SM to hide their latency, and blocks of one unit end soon
+      // enough for another pool's ticks on a stream of higher priority to get
+      // their SMs.  Measured with the serving mix (12 s, FP64 and MIXED pools):
+      // 967 Gint/s, FP64 tick p50 106 ms, MIXED 21 ms; a persistent grid of 2
+      // blocks per SM 824, 109, 14; of 4, 721, 86, 27.
       BCK(nb::launch_force_units(NBODY_FP64, b->F, nullptr, nullptr, b->d_units[tb], b->n64,
                                  b->r_mode[0], b->part, (int64_t)b->fp64_per_sm * b->sms, b->st));
       if (b->prof) BCK(cudaEventRecord(e[3], b->st));
