@@ -33,7 +33,7 @@ struct nbody_ctx {
   void *part = nullptr;
   int part_slices = 0;
   void *rk_vs = nullptr, *rk_sr = nullptr, *rk_sv = nullptr;
-  void *tmp_posm = nullptr, *tmp_acc = nullptr;
+  void *tmp_posm = nullptr;
   float4 *fpos = nullptr, *anchor = nullptr;
   double *diag_blocks = nullptr, *diag_out = nullptr, *h_diag = nullptr;
   int *d_flag = nullptr, *h_flag = nullptr;
@@ -114,14 +114,14 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
   sh.bt = nb::force_block_threads(c->mode);
   sh.t = nb::force_tile(c->mode);
   // measured on GB300 (Gint/s): FP64 R = 1, 2 at N = 65536 131, 127; MIXED R = 1,
-  // 2 at 16384 2247, 2253, at 12000 2067, 1919, at 65536 2548, 2601, at 131072
-  // 2605, 2735; FP32 R = 1, 2, 4 at 8192 1806, 1632, 1577, at 16384 2348, 2381,
+  // 2 at 12000 2067, 1919, at 32768 2485, 2474, at 65536 2548, 2601, at 131072
+  // 2605, 2735 (unequal masses at 16387: 5 % slower at R = 2); FP32 R = 1, 2, 4 at 8192 1806, 1632, 1577, at 16384 2348, 2381,
   // 2390, at 131072 2656, 2733, 2856; F64E keeps enough warps resident only at
   // R = 2 and below one block per SM at R = 1
   int r = r_req;
   if (!r) switch (c->mode) {
       case NBODY_FP64: r = 1; break;
-      case NBODY_MIXED: r = c->n < 16384 ? 1 : 2; break;
+      case NBODY_MIXED: r = c->n < 40000 ? 1 : 2; break;
       case NBODY_FP32: r = c->n < 16384 ? 1 : 4; break;
       default: r = (int64_t)sh.bt * 2 * c->num_sms > c->n ? 1 : 2;
     }
@@ -387,7 +387,7 @@ static void free_all(nbody_ctx *c) {
   }
   c->ev_pool.clear();
   void *ptrs[] = {c->posm[0], c->posm[1], c->vel, c->vbar, c->acc, c->part, c->rk_vs, c->rk_sr,
-                  c->rk_sv, c->tmp_posm, c->tmp_acc, c->fpos, c->anchor, c->diag_blocks,
+                  c->rk_sv, c->tmp_posm, c->fpos, c->anchor, c->diag_blocks,
                   c->diag_out, c->d_flag, c->stage, c->sym_units, c->sym_buf,
                   c->ord_scratch, c->perm, c->sposm};
   for (void *p : ptrs)
@@ -565,20 +565,26 @@ int nbody_get_state(nbody_ctx *c, double *pos, double *vel, double *t, int64_t *
   return sync(c);
 }
 
-static int copy_acc_out(nbody_ctx *c, const void *accbuf, double *acc, double *pot, int on_device,
-                        int64_t count = -1) {
-  const size_t n = (size_t)(count < 0 ? c->n : count);
-  if (on_device) {
-    CK(nb::launch_unpack_acc(c->mode, accbuf, (int64_t)n, acc, pot, c->st));
-    c->launches++;
-  } else {
+// Accelerations and potentials out: those stored in accbuf, or (accbuf NULL) the
+// sums e of the evaluation just queued.
+static int copy_acc_out(nbody_ctx *c, const void *accbuf, const nb::EpiIn &e, double *acc,
+                        double *pot, int on_device) {
+  const size_t n = (size_t)e.n;
+  double *da = acc, *dq = pot;
+  if (!on_device) {
     int rc = ensure_stage(c);
     if (rc) return rc;
-    CK(nb::launch_unpack_acc(c->mode, accbuf, (int64_t)n, acc ? c->stage : nullptr,
-                             pot ? c->stage + 3 * n : nullptr, c->st));
-    c->launches++;
-    if (acc) CK(cudaMemcpyAsync(acc, c->stage, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, c->st));
-    if (pot) CK(cudaMemcpyAsync(pot, c->stage + 3 * n, n * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+    da = acc ? c->stage : nullptr;
+    dq = pot ? c->stage + 3 * n : nullptr;
+  }
+  if (accbuf)
+    CK(nb::launch_unpack_acc(c->mode, accbuf, e.n, da, dq, c->st));
+  else
+    CK(nb::launch_acc_out(c->mode, e, da, dq, c->st));
+  c->launches++;
+  if (!on_device) {
+    if (acc) CK(cudaMemcpyAsync(acc, da, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+    if (pot) CK(cudaMemcpyAsync(pot, dq, n * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   }
   return sync(c);
 }
@@ -587,20 +593,15 @@ int nbody_accel(nbody_ctx *c, const double *pos, const double *mass, double *acc
                 int on_device) {
   if (!c || !pos || !mass || !acc) return fail(NBODY_EINVAL, "NULL argument");
   CK(cudaSetDevice(c->device));
-  if (!c->tmp_posm) {
-    if (cudaMalloc(&c->tmp_posm, (size_t)c->n * r4(c)) != cudaSuccess ||
-        cudaMalloc(&c->tmp_acc, (size_t)c->n * r4(c)) != cudaSuccess)
-      return fail(NBODY_ENOMEM, "accel buffers");
-  }
+  if (!c->tmp_posm && cudaMalloc(&c->tmp_posm, (size_t)c->n * r4(c)) != cudaSuccess)
+    return fail(NBODY_ENOMEM, "accel buffers");
   nvtxRangePushA("nbody_accel");
   int rc = load_arrays(c, pos, nullptr, mass, on_device, c->tmp_posm, nullptr, false);
   int S = 0;
   if (!rc) rc = force(c, c->tmp_posm, S);
   nvtxRangePop();
   if (rc) return rc;
-  CK(nb::launch_store_acc(c->mode, epi(c, S), c->tmp_acc, c->st));
-  c->launches++;
-  return copy_acc_out(c, c->tmp_acc, acc, pot, on_device);
+  return copy_acc_out(c, nullptr, epi(c, S), acc, pot, on_device);
 }
 
 int nbody_accel_rows(nbody_ctx *c, int64_t i0, int64_t ni, const double *pos, const double *mass,
@@ -608,11 +609,8 @@ int nbody_accel_rows(nbody_ctx *c, int64_t i0, int64_t ni, const double *pos, co
   if (!c || !pos || !mass || !acc) return fail(NBODY_EINVAL, "NULL argument");
   if (i0 < 0 || ni < 1 || i0 > c->n - ni) return fail(NBODY_EINVAL, "rows outside [0, n)");
   CK(cudaSetDevice(c->device));
-  if (!c->tmp_posm) {
-    if (cudaMalloc(&c->tmp_posm, (size_t)c->n * r4(c)) != cudaSuccess ||
-        cudaMalloc(&c->tmp_acc, (size_t)c->n * r4(c)) != cudaSuccess)
-      return fail(NBODY_ENOMEM, "accel buffers");
-  }
+  if (!c->tmp_posm && cudaMalloc(&c->tmp_posm, (size_t)c->n * r4(c)) != cudaSuccess)
+    return fail(NBODY_ENOMEM, "accel buffers");
   nvtxRangePushA("nbody_accel_rows");
   int rc = load_arrays(c, pos, nullptr, mass, on_device, c->tmp_posm, nullptr, false);
   int S = 0;
@@ -644,9 +642,8 @@ int nbody_accel_rows(nbody_ctx *c, int64_t i0, int64_t ni, const double *pos, co
   nb::EpiIn e = epi(c, S);
   e.n = ni;
   e.perm = nullptr;
-  CK(nb::launch_store_acc(c->mode, e, c->tmp_acc, c->st));
-  c->launches += 2;
-  return copy_acc_out(c, c->tmp_acc, acc, pot, on_device, ni);
+  c->launches++;
+  return copy_acc_out(c, nullptr, e, acc, pot, on_device);
 }
 
 int nbody_get_accel(nbody_ctx *c, double *acc, double *pot, int on_device) {
@@ -656,7 +653,7 @@ int nbody_get_accel(nbody_ctx *c, double *acc, double *pot, int on_device) {
   int rc = ensure_acc(c);
   if (rc) return rc;
   if (!acc && !pot) return sync(c);
-  return copy_acc_out(c, c->acc, acc, pot, on_device);
+  return copy_acc_out(c, c->acc, epi(c, 0), acc, pot, on_device);
 }
 
 // nsteps steps of size dt, each a sequence of nh KDK steps (Eq. 5-7) of sizes

@@ -169,8 +169,10 @@ struct FxPair {
   int s, sp;             // right shifts of the force and potential terms
 };
 
-// false: the pair is closer than 2^51 units (nothing else is set).
-template <class RSQRT>
+// false: the pair is closer than 2^51 units (EARLY: nothing else is set;
+// otherwise 1/r and 1/r^2 are 0, so that its terms add nothing, and no branch
+// keeps the pairs of several calls from being interleaved).
+template <bool EARLY = true, class RSQRT>
 FX_HD bool fx_geometry(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3], const FxEps &e2,
                        RSQRT rsqrt, FxPair &p) {
   uint64_t S2 = e2.hi;
@@ -190,11 +192,12 @@ FX_HD bool fx_geometry(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3], const F
   const int64_t Mid = S1 + (int64_t)(q >> 1);
   const uint64_t T = S2 + (uint64_t)(Mid >> 31);
   const uint32_t th = (uint32_t)(T >> 32), tl = (uint32_t)T, t0 = (uint32_t)Mid << 1;
-  if (th < 64u) return false;
+  const bool far = th >= 64u;
+  if (EARLY && !far) return false;
 #ifdef __CUDA_ARCH__
   const int h = __clz(th) >> 1;
 #else
-  const int h = __builtin_clz(th) >> 1;
+  const int h = __builtin_clz(th | 1) >> 1;
 #endif
   const uint32_t xh = fx_shl(tl, th, 2 * h), xl = fx_shl(t0, tl, 2 * h);
   const uint32_t S0 = rsqrt(xh) - 0x37000000u;  // 2^23 / sqrt(x), an integer
@@ -209,7 +212,8 @@ FX_HD bool fx_geometry(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3], const F
   const int64_t E1 = fx_mads(fx_mulhi(E27, E27), -192, E);  // -(e + 3 e^2/4) 2^78
   const int64_t V =
       fx_mads((int32_t)S0, (int32_t)(E1 >> 32), (int64_t)fx_umulhi(S0, (uint32_t)E1));
-  const uint64_t R = ((uint64_t)(S0 << 7) << 32) - (uint64_t)(V >> 8);
+  uint64_t R = ((uint64_t)(S0 << 7) << 32) - (uint64_t)(V >> 8);
+  if (!EARLY && !far) R = 0;
   const uint32_t Rh = (uint32_t)(R >> 32), Rl = (uint32_t)R;
   p.Rh = Rh;
   p.Rl = Rl;
@@ -219,7 +223,7 @@ FX_HD bool fx_geometry(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3], const F
   p.Ql = (uint32_t)R2 << 1;
   p.s = 36 - 3 * h;
   p.sp = 23 - h;
-  return true;
+  return far;
 }
 
 // a += w >> s for the 96-bit w (WIDE: s < 96, else s < 32)

@@ -440,36 +440,68 @@ struct FxRsqrt {
 };
 
 // How the masses of a tile enter (fixed.cuh): all equal, one exponent, or an
-// exponent each.
-enum FxMode { FX_EQUAL, FX_NARROW, FX_WIDE };
+// exponent each.  FX_SELF is FX_NARROW for a tile that may hold the block's own
+// particles (FX_WIDE looks for them too).
+enum FxMode { FX_EQUAL, FX_NARROW, FX_SELF, FX_WIDE };
+struct FxEarly {
+  static constexpr bool value = true;
+};
+struct FxLate {
+  static constexpr bool value = false;
+};
 
 // The fixed-point sum of RI i-particles against the tile entries [k0, k1).
-// self(r, k): the pair of particle r with itself (looked at in FX_WIDE
-// only, which the tiles that hold the block's own particles take);
+// self(r, k): the pair of particle r with itself (looked at in FX_SELF and
+// FX_WIDE);
 // close(r, k): adds a pair too close for the tile's unit in binary64.
-template <int RI, FxMode MODE, class Self, class Close>
+// U tile entries are taken at a time, interleaved (U = 2 in the split shape, for
+// the few warps of a small system, whose time is the latency of a pair: N =
+// 1000 21.3 us against 23.2, 4096 139 against 149; U = 4 21.1 and 145).
+template <int RI, int U, FxMode MODE, class Self, class Close>
 __device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, const int *tdm, int k0,
                                         int k1, const FxEps &e2, const uint64_t (&Xi)[RI][3],
                                         fx96 (&f)[RI][3], fx96 (&pt)[RI], Self self, Close close) {
-#pragma unroll 1
-  for (int k = k0; k < k1; k++) {
+  auto pair = [&](int k, int r, auto early) {
     const uint4 a = txy[k], b = tzm[k];
     const uint64_t Xj[3] = {((uint64_t)a.y << 32) | a.x, ((uint64_t)a.w << 32) | a.z,
                             ((uint64_t)b.y << 32) | b.x};
     const int dm = MODE == FX_WIDE ? tdm[k] : 0;
-#pragma unroll
-    for (int r = 0; r < RI; r++) {
-      const bool s = MODE == FX_WIDE && self(r, k);
-      FxPair p;
-      if (!fx_geometry(Xj, Xi[r], e2, FxRsqrt(), p)) {
-        if (!s) close(r, k);
-      } else if (MODE == FX_EQUAL) {
+    const bool s = (MODE == FX_WIDE || MODE == FX_SELF) && self(r, k);
+    FxPair p;
+    const bool far = fx_geometry<decltype(early)::value>(Xj, Xi[r], e2, FxRsqrt(), p);
+    if (!decltype(early)::value || far) {
+      if (MODE == FX_EQUAL)
         fx_both(p, f[r], pt[r], nullptr, nullptr);
-      } else {
+      else
         fx_side<MODE == FX_WIDE>(p, FxMass{s ? 0u : b.w, s ? 0u : b.z, dm}, f[r], pt[r]);
-      }
+    }
+    return far || s;
+  };
+  int k = k0;
+  if (U > 1) {
+#pragma unroll 1
+    for (; k + U <= k1; k += U) {
+      bool done[U][RI], all = true;
+#pragma unroll
+      for (int u = 0; u < U; u++)
+#pragma unroll
+        for (int r = 0; r < RI; r++) {
+          done[u][r] = pair(k + u, r, FxLate());
+          all &= done[u][r];
+        }
+      if (!all)
+#pragma unroll
+        for (int u = 0; u < U; u++)
+#pragma unroll
+          for (int r = 0; r < RI; r++)
+            if (!done[u][r]) close(r, k + u);
     }
   }
+#pragma unroll 1
+  for (; k < k1; k++)
+#pragma unroll
+    for (int r = 0; r < RI; r++)
+      if (!pair(k, r, FxEarly())) close(r, k);
 }
 
 // The binary64 force sum, bound by the FMA-heavy pipe (the wide integer
@@ -552,7 +584,13 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
         const double m0 = tile[0].w;
         const bool equal = __syncthreads_and(
             __double_as_longlong(pj.w) == __double_as_longlong(m0) || tid >= cnt);
-        const FxMode mode = diag || sc.wide ? FX_WIDE : equal ? FX_EQUAL : FX_NARROW;
+        // FX_SELF in the split shape alone, where such tiles are a large share
+        // (N = 4096: 139 us against 147); elsewhere one more form of the loop
+        // made the others slower (N = 20011: 3.54 ms against 3.35)
+        const FxMode mode = sc.wide || (diag && IW == 1) ? FX_WIDE
+                            : diag                       ? FX_SELF
+                            : equal                      ? FX_EQUAL
+                                                         : FX_NARROW;
         const int em = mode == FX_EQUAL ? FX_EQ_EM : sc.em;
         const FxEps e2 = fx_eps2(eps2, sc.L);
         double fs = fx_exp2(fx_force_exp(sc.L, em) + 32), ps = fx_exp2(fx_pot_exp(sc.L, em) + 32);
@@ -580,11 +618,13 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
             acc[g][r].w += v.w;
           };
           if (mode == FX_WIDE)
-            fx_tile<RI, FX_WIDE>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+            fx_tile<RI, IW == 1 ? 1 : 2, FX_WIDE>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+          else if (IW > 1 && mode == FX_SELF)
+            fx_tile<RI, IW == 1 ? 1 : 2, FX_SELF>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
           else if (mode == FX_EQUAL)
-            fx_tile<RI, FX_EQUAL>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+            fx_tile<RI, IW == 1 ? 1 : 2, FX_EQUAL>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
           else
-            fx_tile<RI, FX_NARROW>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
+            fx_tile<RI, IW == 1 ? 1 : 2, FX_NARROW>(txy, tzm, tdm, k0, k1, e2, Xi, f, pt, self, close);
 #pragma unroll
           for (int r = 0; r < RI; r++) {
             acc[g][r].x = fx_fold(acc[g][r].x, f[r][0], fs);

@@ -142,6 +142,8 @@ cudaError_t launch_pack(int mode, const double *pos, const double *vel, const do
 cudaError_t launch_unpack_state(int mode, const void *posm, const void *velv, int64_t n,
                                 double *pos, double *vel, cudaStream_t st);
 cudaError_t launch_store_acc(int mode, const EpiIn &e, void *acc, cudaStream_t st);
+// store_acc and unpack_acc in one: acc3 (n x 3), pot (n), either may be NULL
+cudaError_t launch_acc_out(int mode, const EpiIn &e, double *acc3, double *pot, cudaStream_t st);
 cudaError_t launch_unpack_acc(int mode, const void *acc, int64_t n, double *acc3, double *pot,
                               cudaStream_t st);
 cudaError_t launch_kdk_predict(int mode, int64_t n, double dt, const void *posm_cur,

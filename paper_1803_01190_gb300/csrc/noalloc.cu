@@ -37,7 +37,7 @@ namespace {
 
 constexpr int64_t kMaxN = NBODY_STATIC_MAX_N;
 constexpr size_t kScratchBytes = (size_t)NBODY_STATIC_SCRATCH_BYTES;
-static_assert(kScratchBytes >= (size_t)kMaxN * sizeof(nb::d4) * 3, "scratch too small");
+static_assert(kScratchBytes >= (size_t)kMaxN * sizeof(nb::d4) * 2, "scratch too small");
 
 // The scratch itself.  In host code this name is only a stand-in: its device
 // address comes from cudaGetSymbolAddress below.
@@ -136,11 +136,10 @@ extern "C" int nbody_accel_f64_static(int64_t n, const double *pos, const double
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)cuda_stream;
 
-  // scratch layout: [packed positions n][summed accelerations n][S partial slices of n]
+  // scratch layout: [packed positions n][S partial slices of n]
   nb::d4 *posm = (nb::d4 *)base;
-  nb::d4 *accd = posm + n;
-  nb::d4 *part = accd + n;
-  const int64_t slots = (int64_t)(kScratchBytes / sizeof(nb::d4)) / n - 2;
+  nb::d4 *part = posm + n;
+  const int64_t slots = (int64_t)(kScratchBytes / sizeof(nb::d4)) / n - 1;
 
   nb::Shape sh;
   sh.bt = nb::force_block_threads(NBODY_FP64);
@@ -177,9 +176,7 @@ extern "C" int nbody_accel_f64_static(int64_t n, const double *pos, const double
   e.S = sh.s;
   e.part = part;
   e.G = G;
-  ce = nb::launch_store_acc(NBODY_FP64, e, accd, st);
+  ce = nb::launch_acc_out(NBODY_FP64, e, acc, pot, st);
   if (ce != cudaSuccess) return fail(NBODY_ECUDA, "sum launch", ce);
-  ce = nb::launch_unpack_acc(NBODY_FP64, accd, n, acc, pot, st);
-  if (ce != cudaSuccess) return fail(NBODY_ECUDA, "unpack launch", ce);
   return NBODY_OK;
 }

@@ -110,6 +110,25 @@ __global__ void k_store_acc(const P *__restrict__ part, const int32_t *__restric
     acc[perm ? perm[k] : k] = gather_acc<real, P>(part, S, n, k, G);
 }
 
+// The sums of one evaluation straight into the caller's layout (either output
+// may be NULL).
+template <typename real, typename P>
+__global__ void k_acc_out(const P *__restrict__ part, const int32_t *__restrict__ perm, int S,
+                          int64_t n, real G, double *__restrict__ acc3,
+                          double *__restrict__ pot) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = perm ? perm[k] : k;
+    const real4<real> a = gather_acc<real, P>(part, S, n, k, G);
+    if (acc3) {
+      acc3[3 * i] = a.x;
+      acc3[3 * i + 1] = a.y;
+      acc3[3 * i + 2] = a.z;
+    }
+    if (pot) pot[i] = a.w;
+  }
+}
+
 template <typename real>
 __global__ void k_unpack_acc(const real4<real> *__restrict__ acc, int64_t n,
                              double *__restrict__ acc3, double *__restrict__ pot) {
@@ -351,6 +370,16 @@ cudaError_t launch_store_acc(int mode, const EpiIn &e, void *acc, cudaStream_t s
   else
     k_store_acc<double, d4><<<grid_for(e.n), block_for(e.n), 0, st>>>((const d4 *)e.part, e.perm, e.S, e.n, e.G,
                                                            (d4 *)acc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_acc_out(int mode, const EpiIn &e, double *acc3, double *pot, cudaStream_t st) {
+  if (mode == NBODY_FP32)
+    k_acc_out<float, float4><<<grid_for(e.n), block_for(e.n), 0, st>>>(
+        (const float4 *)e.part, e.perm, e.S, e.n, (float)e.G, acc3, pot);
+  else
+    k_acc_out<double, d4><<<grid_for(e.n), block_for(e.n), 0, st>>>((const d4 *)e.part, e.perm, e.S,
+                                                                    e.n, e.G, acc3, pot);
   return cudaGetLastError();
 }
 
