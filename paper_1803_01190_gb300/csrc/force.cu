@@ -468,12 +468,12 @@ __device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, cons
     const int dm = MODE == FX_WIDE ? tdm[k] : 0;
     const bool s = (MODE == FX_WIDE || MODE == FX_SELF) && self(r, k);
     FxPair p;
-    const bool far = fx_geometry<decltype(early)::value>(Xj, Xi[r], e2, FxRsqrt(), p);
+    const bool far = fx_geometry<false, decltype(early)::value>(Xj, Xi[r], e2, FxRsqrt(), p);
     if (!decltype(early)::value || far) {
       if (MODE == FX_EQUAL)
-        fx_both(p, f[r], pt[r], nullptr, nullptr);
+        fx_both<false>(p, f[r], pt[r], nullptr, nullptr);
       else
-        fx_side<MODE == FX_WIDE>(p, FxMass{s ? 0u : b.w, s ? 0u : b.z, dm}, f[r], pt[r]);
+        fx_side<false, MODE == FX_WIDE>(p, FxMass{s ? 0u : b.w, s ? 0u : b.z, dm}, f[r], pt[r]);
     }
     return far || s;
   };
@@ -915,12 +915,12 @@ __device__ __forceinline__ void fx_sym_tile(const d4 *__restrict__ posm, int64_t
 #pragma unroll
       for (int r = 0; r < R; r++) {
         FxPair p;
-        if (ok && fx_geometry(Xj, Xi[r], e2, FxRsqrt(), p)) {
+        if (ok && fx_geometry<true>(Xj, Xi[r], e2, FxRsqrt(), p)) {
           if (MODE == FX_EQUAL) {
-            fx_both(p, f[r], pt[r], &g, &gp);
+            fx_both<true>(p, f[r], pt[r], &g, &gp);
           } else {
-            fx_side<MODE == FX_WIDE>(p, Mj, f[r], pt[r]);
-            fx_side<MODE == FX_WIDE>(p, Mi[r], g, gp);
+            fx_side<true, MODE == FX_WIDE>(p, Mj, f[r], pt[r]);
+            fx_side<true, MODE == FX_WIDE>(p, Mi[r], g, gp);
           }
         } else {
           const int64_t i = i0 + r * BT + tid;

@@ -54,7 +54,7 @@ int main() {
     const FxEps e2 = fx_eps2(eps * eps, L);
     const float off_seed = 1.0f + (float)((2 * U() - 1) * 0x1p-22);  // the SFU's error
     FxPair p;
-    const bool ok = fx_geometry(Xj, Xi, e2, [&](uint32_t x) {
+    const bool ok = fx_geometry<false>(Xj, Xi, e2, [&](uint32_t x) {
       const float y = (float)(1.0 / std::sqrt((double)(float)x)) * off_seed;
       uint32_t b;
       memcpy(&b, &y, 4);
@@ -74,11 +74,11 @@ int main() {
     if (ur > ldexpl(1.001L, -51)) wrong++;
     fx96 f[3] = {}, pot = {};
     if (equal)
-      fx_both(p, f, pot, nullptr, nullptr);
+      fx_both<false>(p, f, pot, nullptr, nullptr);
     else if (wide)
-      fx_side<true>(p, M, f, pot);
+      fx_side<false, true>(p, M, f, pot);
     else
-      fx_side<false>(p, M, f, pot);
+      fx_side<false, false>(p, M, f, pot);
 const ld ratio = equal ? 1 : (ld)mmax / m;
     const int e_m = equal ? FX_EQ_EM : em;
     // with its own exponent: the place of the last bit of the 96-bit sums
