@@ -343,7 +343,8 @@ __device__ __noinline__ d4 pair_f64(double dx, double dy, double dz, double m, d
 // ---------------------------------------------------------------- fixed point: tile scale
 // Enclosing box of a set of particles from the high words of their coordinates
 // (order-preserving signed keys), their largest mass and smallest positive
-// mass (high words); mmin = -1 marks a non-finite value or a negative mass.
+// mass (high words); mmin = -1 marks a non-finite value or a negative or
+// subnormal mass.
 struct FxBox {
   int lo[3], hi[3], mmax, mmin;
 };
@@ -364,7 +365,7 @@ __device__ __forceinline__ void fx_box_add(FxBox &b, const d4 &p) {
     b.lo[c] = min(b.lo[c], fx_key(h[c]));
     b.hi[c] = max(b.hi[c], fx_key(h[c]));
   }
-  bool bad = h[3] < 0;
+  bool bad = h[3] < 0 || (h[3] < 0x00100000 && p.w > 0.0);
 #pragma unroll
   for (int c = 0; c < 4; c++) bad |= (h[c] & 0x7FF00000) == 0x7FF00000;
   b.mmax = max(b.mmax, h[3]);

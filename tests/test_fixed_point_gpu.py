@@ -113,6 +113,21 @@ def test_non_finite_input_gives_non_finite_output(nb, bad, where):
         assert not np.isfinite(acc[others, 0]).any()
 
 
+def test_subnormal_masses(nb):
+    # below the fixed-point form's masses: binary64, whose subnormal results are exact to
+    # a few units of 2^-1074
+    pos, mass, _ = _case("plain", 300)
+    mass = np.full(300, 3.0e-310)
+    for sym in (0, 1):
+        with nb.Simulation(300, "fp64", eps=0.5) as sim:
+            sim.set_symmetric(sym)
+            acc, pot = sim.accel(pos, mass)
+        oa, op, _ = oracle.accel(pos, mass, 0.5)
+        assert np.abs(acc).max() > 1e-309
+        assert np.abs(acc - oa).max() <= 300 * 2.0 ** -1073
+        assert np.abs(pot - op).max() <= 300 * 2.0 ** -1073
+
+
 def test_negative_mass(nb):
     pos, mass, eps = _case("plain", 300)
     mass[5] = -mass[5]
