@@ -41,22 +41,35 @@ __device__ __forceinline__ real4<real> mk4(real x, real y, real z, real w) {
   return v;
 }
 
-// Sum of the S j-segment partials of the i-th particle of the sums in segment order, with G and
-// the sign of the potential applied: returns (a_x, a_y, a_z, pot).
-template <typename real, typename P>
-__device__ __forceinline__ real4<real> gather_acc(const P *part, int S, int64_t n, int64_t i,
-                                                  real G) {
+// The epilogues work on components: thread t has component c = t mod 4 (x, y, z,
+// potential or mass) of particle t / 4, all arrays being real4.  A particle's
+// FP64 additions, 4 S of them and about 40 of the update, would keep one thread
+// and with it a quarter of an SM busy for longer than the memory access takes
+// (64 cycles a warp each; the epilogue of N = 4096 with S = 32 took 14.3 us with
+// one thread per particle).  A mixed step of 2048 particles went from 51.0 to
+// 48.0 us, an FP64 step of 4096 from 161.5 to 160.7; the order of the operations
+// is the same.
+
+// Component c of the sum of the S j-segment partials of the k-th particle of
+// the sums, in segment order, with G and the sign of the potential applied.
+template <typename real>
+__device__ __forceinline__ real gather_comp(const real *part, int S, int64_t n, int64_t k, int c,
+                                            real G) {
   using O = ops<real>;
-  const P p0 = part[i];
-  real x = (real)p0.x, y = (real)p0.y, z = (real)p0.z, w = (real)p0.w;
-  for (int s = 1; s < S; s++) {
-    const P p = part[(int64_t)s * n + i];
-    x = O::add(x, (real)p.x);
-    y = O::add(y, (real)p.y);
-    z = O::add(z, (real)p.z);
-    w = O::add(w, (real)p.w);
+  const real *p = part + 4 * k + c;
+  real x = *p;
+#pragma unroll 4
+  for (int s = 1; s < S; s++) x = O::add(x, p[4 * (int64_t)s * n]);
+  const real a = O::mul(G, x);
+  return c < 3 ? a : -a;
+}
+template <typename real, class F>
+__device__ __forceinline__ void for_components(int64_t n, const int32_t *perm, F f) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 4 * n;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = t >> 2;
+    f(k, perm ? (int64_t)perm[k] : k, (int)(t & 3));
   }
-  return mk4<real>(O::mul(G, x), O::mul(G, y), O::mul(G, z), -O::mul(G, w));
 }
 
 // ---------------------------------------------------------------- pack / unpack
@@ -102,31 +115,28 @@ __global__ void k_unpack_state(const real4<real> *__restrict__ posm,
   }
 }
 
-template <typename real, typename P>
-__global__ void k_store_acc(const P *__restrict__ part, const int32_t *__restrict__ perm, int S,
-                            int64_t n, real G, real4<real> *__restrict__ acc) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    acc[perm ? perm[k] : k] = gather_acc<real, P>(part, S, n, k, G);
+template <typename real>
+__global__ void k_store_acc(const real *__restrict__ part, const int32_t *__restrict__ perm, int S,
+                            int64_t n, real G, real *__restrict__ acc) {
+  for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
+    acc[4 * i + c] = gather_comp<real>(part, S, n, k, c, G);
+  });
 }
 
 // The sums of one evaluation straight into the caller's layout (either output
 // may be NULL).
-template <typename real, typename P>
-__global__ void k_acc_out(const P *__restrict__ part, const int32_t *__restrict__ perm, int S,
+template <typename real>
+__global__ void k_acc_out(const real *__restrict__ part, const int32_t *__restrict__ perm, int S,
                           int64_t n, real G, double *__restrict__ acc3,
                           double *__restrict__ pot) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = perm ? perm[k] : k;
-    const real4<real> a = gather_acc<real, P>(part, S, n, k, G);
-    if (acc3) {
-      acc3[3 * i] = a.x;
-      acc3[3 * i + 1] = a.y;
-      acc3[3 * i + 2] = a.z;
+  for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
+    const real a = gather_comp<real>(part, S, n, k, c, G);
+    if (c < 3) {
+      if (acc3) acc3[3 * i + c] = a;
+    } else if (pot) {
+      pot[i] = a;
     }
-    if (pot) pot[i] = a.w;
-  }
+  });
 }
 
 template <typename real>
@@ -149,60 +159,51 @@ __global__ void k_unpack_acc(const real4<real> *__restrict__ acc, int64_t n,
 //   vt = v + dt a                      (Eq. 5)
 //   r' = r + dt/2 (vt + v)             (Eq. 6)     -> posm_nxt (mass copied)
 //   vbar = (v + vt) / 2                (first term of Eq. 7, kept for the corrector)
+// one component (c = 3: the mass is copied, vbar's fourth component is 0)
 template <typename real>
-__device__ __forceinline__ void kdk_predict_one(real dt, real hdt, const real4<real> &r,
-                                                const real4<real> &v, const real4<real> &a,
-                                                real4<real> &vbar, real4<real> &rn) {
+__device__ __forceinline__ void kdk_predict_one(int c, real dt, real hdt, real r, real v, real a,
+                                                real &vbar, real &rn) {
   using O = ops<real>;
-  const real tx = O::add(v.x, O::mul(dt, a.x));
-  const real ty = O::add(v.y, O::mul(dt, a.y));
-  const real tz = O::add(v.z, O::mul(dt, a.z));
-  rn = mk4<real>(O::add(r.x, O::mul(hdt, O::add(tx, v.x))), O::add(r.y, O::mul(hdt, O::add(ty, v.y))),
-                 O::add(r.z, O::mul(hdt, O::add(tz, v.z))), r.w);
-  vbar = mk4<real>(O::mul(O::add(v.x, tx), (real)0.5), O::mul(O::add(v.y, ty), (real)0.5),
-                   O::mul(O::add(v.z, tz), (real)0.5), (real)0);
+  const real t = O::add(v, O::mul(dt, a));
+  rn = c < 3 ? O::add(r, O::mul(hdt, O::add(t, v))) : r;
+  vbar = c < 3 ? O::mul(O::add(v, t), (real)0.5) : (real)0;
 }
 
 template <typename real>
-__global__ void k_kdk_predict(int64_t n, real dt, real hdt, const real4<real> *__restrict__ posm,
-                              const real4<real> *__restrict__ vel,
-                              const real4<real> *__restrict__ acc, real4<real> *__restrict__ vbar,
-                              real4<real> *__restrict__ posm_nxt) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    real4<real> vb, rn;
-    kdk_predict_one<real>(dt, hdt, posm[i], vel[i], acc[i], vb, rn);
-    vbar[i] = vb;
-    posm_nxt[i] = rn;
-  }
+__global__ void k_kdk_predict(int64_t n, real dt, real hdt, const real *__restrict__ posm,
+                              const real *__restrict__ vel, const real *__restrict__ acc,
+                              real *__restrict__ vbar, real *__restrict__ posm_nxt) {
+  for_components<real>(n, nullptr, [&](int64_t, int64_t i, int c) {
+    const int64_t o = 4 * i + c;
+    real vb, rn;
+    kdk_predict_one<real>(c, dt, hdt, posm[o], vel[o], acc[o], vb, rn);
+    vbar[o] = vb;
+    posm_nxt[o] = rn;
+  });
 }
 
 // After the force at r(t+dt): a' = G sum(parts); corrector
 //   v(t+dt) = vbar + dt/2 a'           (Eq. 7, chdt = dt/2 of the step just ended)
 // then the predictor and drift of the next step, of size dt_next (the same dt
 // for KDK; the next substep's for the fourth-order composition), into posm_pred.
-template <typename real, typename P>
-__global__ void k_kdk_correct_predict(const P *__restrict__ part,
+template <typename real>
+__global__ void k_kdk_correct_predict(const real *__restrict__ part,
                                       const int32_t *__restrict__ perm, int S, int64_t n, real G,
-                                      real chdt, real dt, real hdt, real4<real> *__restrict__ acc,
-                                      const real4<real> *__restrict__ posm_new,
-                                      real4<real> *__restrict__ vel, real4<real> *__restrict__ vbar,
-                                      real4<real> *__restrict__ posm_pred) {
+                                      real chdt, real dt, real hdt, real *__restrict__ acc,
+                                      const real *__restrict__ posm_new, real *__restrict__ vel,
+                                      real *__restrict__ vbar, real *__restrict__ posm_pred) {
   using O = ops<real>;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = perm ? perm[k] : k;
-    const real4<real> a = gather_acc<real, P>(part, S, n, k, G);
-    acc[i] = a;
-    const real4<real> vb = vbar[i];
-    const real4<real> v = mk4<real>(O::add(vb.x, O::mul(chdt, a.x)), O::add(vb.y, O::mul(chdt, a.y)),
-                                    O::add(vb.z, O::mul(chdt, a.z)), (real)0);
-    vel[i] = v;
-    real4<real> nvb, rn;
-    kdk_predict_one<real>(dt, hdt, posm_new[i], v, a, nvb, rn);
-    vbar[i] = nvb;
-    posm_pred[i] = rn;
-  }
+  for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
+    const int64_t o = 4 * i + c;
+    const real a = gather_comp<real>(part, S, n, k, c, G);
+    acc[o] = a;
+    const real v = c < 3 ? O::add(vbar[o], O::mul(chdt, a)) : (real)0;
+    vel[o] = v;
+    real nvb, rn;
+    kdk_predict_one<real>(c, dt, hdt, posm_new[o], v, a, nvb, rn);
+    vbar[o] = nvb;
+    posm_pred[o] = rn;
+  });
 }
 
 // ---------------------------------------------------------------- RK4
@@ -212,57 +213,43 @@ __global__ void k_kdk_correct_predict(const P *__restrict__ part,
 // where v2 = v + dt/2 a1, v3 = v + dt/2 a2, v4 = v + dt a3 and the stage
 // positions are r + dt/2 v, r + dt/2 v2, r + dt v3.  Stage k runs after the
 // force evaluation a_k.
-template <typename real, typename P>
-__global__ void k_rk4_stage(const P *__restrict__ part, const int32_t *__restrict__ perm, int S,
+template <typename real>
+__global__ void k_rk4_stage(const real *__restrict__ part, const int32_t *__restrict__ perm, int S,
                             int64_t n, real G, int stage, real dt, real hdt, real dt6,
-                            real4<real> *__restrict__ posm0,
-                            real4<real> *__restrict__ vel0, real4<real> *__restrict__ vs,
-                            real4<real> *__restrict__ sr, real4<real> *__restrict__ sv,
-                            real4<real> *__restrict__ posm_stage) {
+                            real *__restrict__ posm0, real *__restrict__ vel0,
+                            real *__restrict__ vs, real *__restrict__ sr, real *__restrict__ sv,
+                            real *__restrict__ posm_stage) {
   using O = ops<real>;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = perm ? perm[k] : k;
-    const real4<real> a = gather_acc<real, P>(part, S, n, k, G);
-    const real4<real> r0 = posm0[i];
-    const real4<real> v0 = vel0[i];
-    if (stage == 1) {
-      const real4<real> v2 = mk4<real>(O::add(v0.x, O::mul(hdt, a.x)), O::add(v0.y, O::mul(hdt, a.y)),
-                                       O::add(v0.z, O::mul(hdt, a.z)), (real)0);
-      sv[i] = mk4<real>(a.x, a.y, a.z, (real)0);
-      sr[i] = mk4<real>(O::add(v0.x, O::mul((real)2, v2.x)), O::add(v0.y, O::mul((real)2, v2.y)),
-                        O::add(v0.z, O::mul((real)2, v2.z)), (real)0);
-      vs[i] = v2;
-      posm_stage[i] = mk4<real>(O::add(r0.x, O::mul(hdt, v0.x)), O::add(r0.y, O::mul(hdt, v0.y)),
-                                O::add(r0.z, O::mul(hdt, v0.z)), r0.w);
-    } else if (stage == 2 || stage == 3) {
-      const real c = stage == 2 ? hdt : dt;  // v3 = v + dt/2 a2 ; v4 = v + dt a3
-      const real4<real> vp = vs[i];          // v2 (stage 2) or v3 (stage 3)
-      const real4<real> vn = mk4<real>(O::add(v0.x, O::mul(c, a.x)), O::add(v0.y, O::mul(c, a.y)),
-                                       O::add(v0.z, O::mul(c, a.z)), (real)0);
-      real4<real> s = sv[i];
-      s = mk4<real>(O::add(s.x, O::mul((real)2, a.x)), O::add(s.y, O::mul((real)2, a.y)),
-                    O::add(s.z, O::mul((real)2, a.z)), (real)0);
-      sv[i] = s;
-      real4<real> q = sr[i];
-      const real w = stage == 2 ? (real)2 : (real)1;  // + 2 v3 ; + v4
-      q = mk4<real>(O::add(q.x, O::mul(w, vn.x)), O::add(q.y, O::mul(w, vn.y)),
-                    O::add(q.z, O::mul(w, vn.z)), (real)0);
-      sr[i] = q;
-      vs[i] = vn;
-      // stage positions r + dt/2 v2 (after a2) and r + dt v3 (after a3)
-      posm_stage[i] = mk4<real>(O::add(r0.x, O::mul(c, vp.x)), O::add(r0.y, O::mul(c, vp.y)),
-                                O::add(r0.z, O::mul(c, vp.z)), r0.w);
-    } else {
-      const real4<real> s = sv[i];
-      const real4<real> q = sr[i];
-      const real sx = O::add(s.x, a.x), sy = O::add(s.y, a.y), sz = O::add(s.z, a.z);
-      posm0[i] = mk4<real>(O::add(r0.x, O::mul(dt6, q.x)), O::add(r0.y, O::mul(dt6, q.y)),
-                           O::add(r0.z, O::mul(dt6, q.z)), r0.w);
-      vel0[i] = mk4<real>(O::add(v0.x, O::mul(dt6, sx)), O::add(v0.y, O::mul(dt6, sy)),
-                          O::add(v0.z, O::mul(dt6, sz)), (real)0);
+  for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
+    const int64_t o = 4 * i + c;
+    if (c == 3) {  // masses of the stage positions; the velocities' fourth component is 0
+      if (stage < 4) posm_stage[o] = posm0[o];
+      if (stage == 1 || stage == 4) (stage == 1 ? vs : vel0)[o] = (real)0;
+      return;
     }
-  }
+    const real a = gather_comp<real>(part, S, n, k, c, G);
+    const real r0 = posm0[o], v0 = vel0[o];
+    if (stage == 1) {
+      const real v2 = O::add(v0, O::mul(hdt, a));
+      sv[o] = a;
+      sr[o] = O::add(v0, O::mul((real)2, v2));
+      vs[o] = v2;
+      posm_stage[o] = O::add(r0, O::mul(hdt, v0));
+    } else if (stage == 2 || stage == 3) {
+      const real h = stage == 2 ? hdt : dt;  // v3 = v + dt/2 a2 ; v4 = v + dt a3
+      const real vp = vs[o];                 // v2 (stage 2) or v3 (stage 3)
+      const real vn = O::add(v0, O::mul(h, a));
+      sv[o] = O::add(sv[o], O::mul((real)2, a));
+      const real w = stage == 2 ? (real)2 : (real)1;  // + 2 v3 ; + v4
+      sr[o] = O::add(sr[o], O::mul(w, vn));
+      vs[o] = vn;
+      // stage positions r + dt/2 v2 (after a2) and r + dt v3 (after a3)
+      posm_stage[o] = O::add(r0, O::mul(h, vp));
+    } else {
+      posm0[o] = O::add(r0, O::mul(dt6, sr[o]));
+      vel0[o] = O::add(v0, O::mul(dt6, O::add(sv[o], a)));
+    }
+  });
 }
 
 // ---------------------------------------------------------------- Eq. 8-10
@@ -331,13 +318,11 @@ __global__ void __launch_bounds__(DIAG_BT) k_diag_final(const double *__restrict
 }
 
 // ---------------------------------------------------------------- launchers
-// Blocks of 64 while they spread a small system over more SMs (the FP64
-// instructions of one particle keep an SM's quarter busy for about 2 us: 8.2
-// us for a step at N = 2048 in blocks of 256, 6.6 in blocks of 64).
-static int block_for(int64_t n) { return n < 152 * 256 ? 64 : 256; }
-static unsigned grid_for(int64_t n) {
-  const int bt = block_for(n);
-  int64_t g = (n + bt - 1) / bt;
+// Blocks of 64 while they spread a small system over more SMs.
+static int block_for(int64_t threads) { return threads < 152 * 256 ? 64 : 256; }
+static unsigned grid_for(int64_t threads) {
+  const int bt = block_for(threads);
+  int64_t g = (threads + bt - 1) / bt;
   if (g > 152 * 64) g = 152 * 64;
   return (unsigned)(g < 1 ? 1 : g);
 }
@@ -364,22 +349,23 @@ cudaError_t launch_unpack_state(int mode, const void *posm, const void *velv, in
 }
 
 cudaError_t launch_store_acc(int mode, const EpiIn &e, void *acc, cudaStream_t st) {
+  const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_store_acc<float, float4><<<grid_for(e.n), block_for(e.n), 0, st>>>((const float4 *)e.part, e.perm, e.S, e.n,
-                                                              (float)e.G, (float4 *)acc);
+    k_store_acc<float><<<g, b, 0, st>>>((const float *)e.part, e.perm, e.S, e.n, (float)e.G,
+                                        (float *)acc);
   else
-    k_store_acc<double, d4><<<grid_for(e.n), block_for(e.n), 0, st>>>((const d4 *)e.part, e.perm, e.S, e.n, e.G,
-                                                           (d4 *)acc);
+    k_store_acc<double><<<g, b, 0, st>>>((const double *)e.part, e.perm, e.S, e.n, e.G,
+                                         (double *)acc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_acc_out(int mode, const EpiIn &e, double *acc3, double *pot, cudaStream_t st) {
+  const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_acc_out<float, float4><<<grid_for(e.n), block_for(e.n), 0, st>>>(
-        (const float4 *)e.part, e.perm, e.S, e.n, (float)e.G, acc3, pot);
+    k_acc_out<float><<<g, b, 0, st>>>((const float *)e.part, e.perm, e.S, e.n, (float)e.G, acc3,
+                                      pot);
   else
-    k_acc_out<double, d4><<<grid_for(e.n), block_for(e.n), 0, st>>>((const d4 *)e.part, e.perm, e.S,
-                                                                    e.n, e.G, acc3, pot);
+    k_acc_out<double><<<g, b, 0, st>>>((const double *)e.part, e.perm, e.S, e.n, e.G, acc3, pot);
   return cudaGetLastError();
 }
 
@@ -395,44 +381,48 @@ cudaError_t launch_unpack_acc(int mode, const void *acc, int64_t n, double *acc3
 cudaError_t launch_kdk_predict(int mode, int64_t n, double dt, const void *posm_cur,
                                const void *vel, const void *acc, void *vbar, void *posm_nxt,
                                cudaStream_t st) {
+  const unsigned g = grid_for(4 * n), b = block_for(4 * n);
   if (mode == NBODY_FP32)
-    k_kdk_predict<float><<<grid_for(n), block_for(n), 0, st>>>(
-        n, (float)dt, (float)(dt / 2), (const float4 *)posm_cur, (const float4 *)vel,
-        (const float4 *)acc, (float4 *)vbar, (float4 *)posm_nxt);
+    k_kdk_predict<float><<<g, b, 0, st>>>(n, (float)dt, (float)(dt / 2), (const float *)posm_cur,
+                                          (const float *)vel, (const float *)acc, (float *)vbar,
+                                          (float *)posm_nxt);
   else
-    k_kdk_predict<double><<<grid_for(n), block_for(n), 0, st>>>(n, dt, dt / 2, (const d4 *)posm_cur,
-                                                       (const d4 *)vel, (const d4 *)acc,
-                                                       (d4 *)vbar, (d4 *)posm_nxt);
+    k_kdk_predict<double><<<g, b, 0, st>>>(n, dt, dt / 2, (const double *)posm_cur,
+                                           (const double *)vel, (const double *)acc,
+                                           (double *)vbar, (double *)posm_nxt);
   return cudaGetLastError();
 }
 
 cudaError_t launch_kdk_correct_predict(int mode, const EpiIn &e, double dt, double dt_next,
                                        void *acc, void *posm_new, void *vel, void *vbar,
                                        void *posm_pred, cudaStream_t st) {
+  const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_kdk_correct_predict<float, float4><<<grid_for(e.n), block_for(e.n), 0, st>>>(
-        (const float4 *)e.part, e.perm, e.S, e.n, (float)e.G, (float)(dt / 2), (float)dt_next,
-        (float)(dt_next / 2), (float4 *)acc, (const float4 *)posm_new, (float4 *)vel,
-        (float4 *)vbar, (float4 *)posm_pred);
+    k_kdk_correct_predict<float><<<g, b, 0, st>>>(
+        (const float *)e.part, e.perm, e.S, e.n, (float)e.G, (float)(dt / 2), (float)dt_next,
+        (float)(dt_next / 2), (float *)acc, (const float *)posm_new, (float *)vel, (float *)vbar,
+        (float *)posm_pred);
   else
-    k_kdk_correct_predict<double, d4><<<grid_for(e.n), block_for(e.n), 0, st>>>(
-        (const d4 *)e.part, e.perm, e.S, e.n, e.G, dt / 2, dt_next, dt_next / 2, (d4 *)acc,
-        (const d4 *)posm_new, (d4 *)vel, (d4 *)vbar, (d4 *)posm_pred);
+    k_kdk_correct_predict<double><<<g, b, 0, st>>>(
+        (const double *)e.part, e.perm, e.S, e.n, e.G, dt / 2, dt_next, dt_next / 2, (double *)acc,
+        (const double *)posm_new, (double *)vel, (double *)vbar, (double *)posm_pred);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rk4_stage(int mode, const EpiIn &e, int stage, double dt, const void *posm0,
                              void *vel0, void *rk_vs, void *rk_sr, void *rk_sv, void *posm_stage,
                              cudaStream_t st) {
+  const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_rk4_stage<float, float4><<<grid_for(e.n), block_for(e.n), 0, st>>>(
-        (const float4 *)e.part, e.perm, e.S, e.n, (float)e.G, stage, (float)dt, (float)(dt / 2),
-        (float)(dt / 6), (float4 *)posm0, (float4 *)vel0, (float4 *)rk_vs, (float4 *)rk_sr,
-        (float4 *)rk_sv, (float4 *)posm_stage);
+    k_rk4_stage<float><<<g, b, 0, st>>>((const float *)e.part, e.perm, e.S, e.n, (float)e.G, stage,
+                                        (float)dt, (float)(dt / 2), (float)(dt / 6),
+                                        (float *)posm0, (float *)vel0, (float *)rk_vs,
+                                        (float *)rk_sr, (float *)rk_sv, (float *)posm_stage);
   else
-    k_rk4_stage<double, d4><<<grid_for(e.n), block_for(e.n), 0, st>>>(
-        (const d4 *)e.part, e.perm, e.S, e.n, e.G, stage, dt, dt / 2, dt / 6, (d4 *)posm0, (d4 *)vel0,
-        (d4 *)rk_vs, (d4 *)rk_sr, (d4 *)rk_sv, (d4 *)posm_stage);
+    k_rk4_stage<double><<<g, b, 0, st>>>((const double *)e.part, e.perm, e.S, e.n, e.G, stage, dt,
+                                         dt / 2, dt / 6, (double *)posm0, (double *)vel0,
+                                         (double *)rk_vs, (double *)rk_sr, (double *)rk_sv,
+                                         (double *)posm_stage);
   return cudaGetLastError();
 }
 
