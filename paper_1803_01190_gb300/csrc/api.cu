@@ -115,9 +115,10 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
   sh.t = nb::force_tile(c->mode);
   // measured on GB300 (Gint/s): FP64 R = 1, 2 at N = 65536 131, 127; MIXED R = 1,
   // 2 at 12000 2067, 1919, at 32768 2485, 2474, at 65536 2548, 2601, at 131072
-  // 2605, 2735 (unequal masses at 16387: 5 % slower at R = 2); FP32 R = 1, 2, 4 at 8192 1806, 1632, 1577, at 16384 2348, 2381,
-  // 2390, at 131072 2656, 2733, 2856; F64E keeps enough warps resident only at
-  // R = 2 and below one block per SM at R = 1
+  // 2605, 2735 (unequal masses at 16387: 5 % slower at R = 2); FP32 R = 1, 2, 4
+  // at 8192 1806, 1632, 1577, at 16384 2348, 2381, 2390, at 131072 2656, 2733,
+  // 2856; F64E keeps enough warps resident only at R = 2 and below one block per
+  // SM at R = 1
   int r = r_req;
   if (!r) switch (c->mode) {
       case NBODY_FP64: r = 1; break;

@@ -7,10 +7,11 @@
 // A simulation occupies a contiguous range of it; ranges are handed out first
 // fit and returned on eviction, so admission is decided by free device memory
 // (a free range of n particles) and a free slot.  One tick advances every
-// resident simulation by one step with at most three force launches (MIXED
-// prep, MIXED force, FP64 force) over work-unit tables that never let a tile
-// cross from one simulation into another, plus one epilogue launch that sums
-// each simulation's j-segments in a fixed order and applies its KDK update.
+// resident simulation by one step with at most five launches for the forces
+// (MIXED and F64E prep and force, FP64 force) over work-unit tables that never
+// let a tile cross from one simulation into another, plus one epilogue launch
+// that sums each simulation's j-segments in a fixed order and applies its KDK
+// update.
 //
 // Per simulation (pool range [off, off+n)):
 //   R  (x, y, z, m) state positions at the step boundary

@@ -28,9 +28,10 @@
 //         FP32 pipes: 1/r and 1/r^2 within 0.52 ulp (SFU seed, exact integer
 //         residual), the products m/r and (m/r)/r^2 by a correctly rounded
 //         integer binary64 multiply, and the potential sum by a correctly
-//         rounded integer binary64 add.  From 64 blocks of 384 particles the FP64 path
-//         evaluates each pair once for both particles (k_force_f64_sym:
-//         12 FP64 instructions per pair, 6 per interaction).
+//         rounded integer binary64 add.  At large N the FP64 path evaluates each
+//         pair once for both particles: softened ones in the same fixed point
+//         (k_force_fx_sym), eps = 0 in binary64 (k_force_f64_sym: 12 FP64
+//         instructions per pair, 6 per interaction).
 //   mixed binary32 pair arithmetic (packed: two j per instruction, SFU
 //         reciprocal square root) on coordinates re-centred on an anchor (the
 //         per-coordinate median) per j-tile, with the i coordinates held as
