@@ -524,6 +524,7 @@ __device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, cons
 template <int BT, int R, int T, int IW, class W>
 __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W work,
                                                   d4 *__restrict__ part) {
+  chain_begin();
   static_assert(T == BT, "one j per thread");
   constexpr int NW = BT / 32, RI = R < 2 ? R : 2, NG = R / RI, IT = BT / IW;
   __shared__ d4 tile[T];
@@ -1440,6 +1441,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
                                                    const float4 *__restrict__ jff,
                                                    const float4 *__restrict__ anchor, W work,
                                                    d4 *__restrict__ part) {
+  chain_begin();
   constexpr int IT = BT / IW;
   __shared__ float4 tH[T / 2], tH2[T / 2], tL[T / 2], tL2[T / 2];
   __shared__ d4 red[IW > 1 ? BT : 1];
@@ -1717,6 +1719,7 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
                                                     const float4 *__restrict__ fpos,
                                                     const float4 *__restrict__ anchor, W work,
                                                     d4 *__restrict__ part) {
+  chain_begin();
   __shared__ float4 tA[T / 2], tB[T / 2];
   for (int64_t uk = work.first(); uk < work.count(); uk += work.stride()) {
     const Unit u = work.get(uk);
@@ -1847,6 +1850,7 @@ template <int BT, class W, bool FF>
 __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, W work,
                                                    float4 *__restrict__ fpos,
                                                    float4 *__restrict__ anchor) {
+  chain_begin();
   static_assert((BT & (BT - 1)) == 0, "bitonic sort needs a power-of-two block");
   __shared__ int v[2][3][BT];
   __shared__ int mid[3], first[3], same[3];
@@ -1949,6 +1953,7 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
 template <int BT, int R, int T, int IW, class W>
 __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ posm, W work,
                                                   float4 *__restrict__ part) {
+  chain_begin();
   constexpr int IT = BT / IW;
   __shared__ float4 tA[T / 2], tB[T / 2];
   __shared__ float4 red[IW > 1 ? BT : 1];
@@ -2091,23 +2096,34 @@ int force_max_blocks_per_sm(int mode, const Shape &sh) {
   return nb;
 }
 
+// One system's launches are links of a chain; those over a table of units (a
+// pool's, or each pair once) follow copies and larger kernels and are plain.
+template <class... P, class... A>
+static cudaError_t launch_k(const DenseWork &, void (*k)(P...), dim3 grid, int bt, cudaStream_t st,
+                            A... args) {
+  return launch_chained(k, grid, bt, st, args...);
+}
+template <class... P, class... A>
+static cudaError_t launch_k(const TableWork &, void (*k)(P...), dim3 grid, int bt, cudaStream_t st,
+                            A... args) {
+  k<<<grid, bt, 0, st>>>(args...);
+  return cudaGetLastError();
+}
+
 template <int R, bool SPLIT, class W>
-static void launch_rw(int mode, const void *posm, const float4 *fpos, const float4 *anchor,
-                      const W &w, dim3 grid, void *part, cudaStream_t st) {
-  if (mode == NBODY_FP64) {
-    k_force_f64<BT_F64, R, T_F64, SPLIT ? IW_F64 : 1, W>
-        <<<grid, BT_F64, 0, st>>>((const d4 *)posm, w, (d4 *)part);
-  } else if (mode == NBODY_MIXED) {
-    k_force_mixed<BT_F32, R, T_F32, W>
-        <<<grid, BT_F32, 0, st>>>((const d4 *)posm, fpos, anchor, w, (d4 *)part);
-  } else if (mode == NBODY_F64E) {
-    constexpr int RF = R < 4 ? R : 4;
-    k_force_f64e<BT_FF, RF, T_FF, SPLIT ? IW_FF : 1, W>
-        <<<grid, BT_FF, 0, st>>>((const d4 *)posm, fpos, anchor, w, (d4 *)part);
-  } else {
-    k_force_f32<BT_F32, R, T_F32, SPLIT ? IW_F32 : 1, W>
-        <<<grid, BT_F32, 0, st>>>((const float4 *)posm, w, (float4 *)part);
-  }
+static cudaError_t launch_rw(int mode, const void *posm, const float4 *fpos, const float4 *anchor,
+                             const W &w, dim3 grid, void *part, cudaStream_t st) {
+  if (mode == NBODY_FP64)
+    return launch_k(w, k_force_f64<BT_F64, R, T_F64, SPLIT ? IW_F64 : 1, W>, grid, BT_F64, st,
+                    (const d4 *)posm, w, (d4 *)part);
+  if (mode == NBODY_MIXED)
+    return launch_k(w, k_force_mixed<BT_F32, R, T_F32, W>, grid, BT_F32, st, (const d4 *)posm, fpos,
+                    anchor, w, (d4 *)part);
+  if (mode == NBODY_F64E)
+    return launch_k(w, k_force_f64e<BT_FF, (R < 4 ? R : 4), T_FF, SPLIT ? IW_FF : 1, W>, grid,
+                    BT_FF, st, (const d4 *)posm, fpos, anchor, w, (d4 *)part);
+  return launch_k(w, k_force_f32<BT_F32, R, T_F32, SPLIT ? IW_F32 : 1, W>, grid, BT_F32, st,
+                  (const float4 *)posm, w, (float4 *)part);
 }
 
 template <class W>
@@ -2115,13 +2131,12 @@ static cudaError_t launch_w(int mode, int r, const void *posm, const float4 *fpo
                             const float4 *anchor, const W &w, dim3 grid, void *part,
                             cudaStream_t st) {
   switch (r) {
-    case 1: launch_rw<1, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
-    case 2: launch_rw<2, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
-    case 4: launch_rw<4, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
-    case 8: launch_rw<8, false>(mode, posm, fpos, anchor, w, grid, part, st); break;
+    case 1: return launch_rw<1, false>(mode, posm, fpos, anchor, w, grid, part, st);
+    case 2: return launch_rw<2, false>(mode, posm, fpos, anchor, w, grid, part, st);
+    case 4: return launch_rw<4, false>(mode, posm, fpos, anchor, w, grid, part, st);
+    case 8: return launch_rw<8, false>(mode, posm, fpos, anchor, w, grid, part, st);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- binary64, each pair once: launches
@@ -2208,10 +2223,8 @@ cudaError_t launch_force(int mode, const ForceIn &in, const Shape &sh, cudaStrea
   w.per_block = (int)per_block;
   w.tile = sh.t;
   const dim3 grid((unsigned)gx, (unsigned)sh.s);
-  if (sh.iw > 1) {
-    launch_rw<1, true>(mode, in.posm, in.fpos, in.anchor, w, grid, in.part, st);
-    return cudaGetLastError();
-  }
+  if (sh.iw > 1)
+    return launch_rw<1, true>(mode, in.posm, in.fpos, in.anchor, w, grid, in.part, st);
   return launch_w(mode, sh.r, in.posm, in.fpos, in.anchor, w, grid, in.part, st);
 }
 
@@ -2235,11 +2248,8 @@ cudaError_t launch_mixed_prep(const d4 *posm, int64_t n, int tile, float4 *fpos,
   DensePrep w;
   w.n = n;
   w.tile = tile;
-  if (ff)
-    k_mixed_prep<256, DensePrep, true><<<(unsigned)nt, 256, 0, st>>>(posm, w, fpos, anchor);
-  else
-    k_mixed_prep<256, DensePrep, false><<<(unsigned)nt, 256, 0, st>>>(posm, w, fpos, anchor);
-  return cudaGetLastError();
+  return launch_chained(ff ? k_mixed_prep<256, DensePrep, true> : k_mixed_prep<256, DensePrep, false>,
+                        dim3((unsigned)nt), 256, st, posm, w, fpos, anchor);
 }
 
 cudaError_t launch_mixed_prep_units(const d4 *posm, const PrepUnit *units, int64_t nunits,

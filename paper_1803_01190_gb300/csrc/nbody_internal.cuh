@@ -20,6 +20,38 @@
 
 namespace nb {
 
+// A kernel of the chains that a force evaluation or a step is made of (order,
+// prep, force, epilogue): launched with launch_chained() it may be set up while
+// the kernel before it in the stream runs its last blocks.  It calls
+// chain_begin() first, which waits until that kernel has completed and its writes
+// are visible (at once after a plain launch), then lets the next kernel of the
+// chain be set up as soon as all blocks of this one have started.  Every thread
+// calls it before anything else, so "the kernel before has completed" holds for
+// all earlier ones too, whatever buffers they share.  At small N a step is a
+// chain of 2 to 6 kernels of a few us each and the gaps between them count:
+// a MIXED step of 2048 particles took 48.0 us with plain launches, 35.7 so; an
+// FP64 evaluation of 1000 48.8 and 43.5, an FP64 step of 4096 160.7 and 155.5.
+__device__ __forceinline__ void chain_begin() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st,
+                           A... args) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3((unsigned)threads);
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // returned here, not left for the next call
+  return e;
+}
+
 struct __align__(32) d4 {
   double x, y, z, w;
 };

@@ -74,6 +74,7 @@ __device__ __forceinline__ uint64_t warp_extreme(uint64_t k) {
 // part[3..5] maxima, as ordered integers.  NaNs are left out.
 __global__ void __launch_bounds__(kBT) k_bbox_partial(const d4 *__restrict__ posm, int64_t n,
                                                       uint64_t *__restrict__ part) {
+  chain_begin();
   __shared__ uint64_t s[6][kBT / 32];
   uint64_t v[6];
 #pragma unroll
@@ -173,6 +174,7 @@ __global__ void __launch_bounds__(kChunk) k_sort_chunk(const d4 *__restrict__ po
                                                        const uint64_t *__restrict__ part, int nparts,
                                                        uint64_t *__restrict__ keys,
                                                        int32_t *__restrict__ idx) {
+  chain_begin();
   __shared__ uint64_t sk[2][kChunk];
   __shared__ int si[2][kChunk];
   const Cells q = reduce_box(part, nparts);
@@ -214,6 +216,7 @@ __global__ void __launch_bounds__(32 * kRankWarps) k_rank_gather(
     const d4 *__restrict__ posm, int64_t n, const uint64_t *__restrict__ keys,
     const int32_t *__restrict__ idx, int chunks, int32_t *__restrict__ perm,
     d4 *__restrict__ sposm) {
+  chain_begin();
   __shared__ int count[kRankWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t g = blockIdx.x * (int64_t)32 + lane;
@@ -287,16 +290,14 @@ cudaError_t launch_spatial_order(const d4 *posm, int64_t n, void *scratch, int32
   int32_t *idx = (int32_t *)p;
   p += align256(sizeof(int32_t) * n);
   const int nb = (int)std::min<int64_t>(kBboxBlocks, (n + kBT - 1) / kBT);
-  k_bbox_partial<<<nb, kBT, 0, st>>>(posm, n, bb);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_chained(k_bbox_partial, dim3(nb), kBT, st, posm, n, bb);
   if (e != cudaSuccess) return e;
   if (n <= kRankMax) {
     const int chunks = (int)(padded(n) / kChunk);
-    k_sort_chunk<<<chunks, kChunk, 0, st>>>(posm, n, bb, nb, kin, idx);
-    e = cudaGetLastError();
+    e = launch_chained(k_sort_chunk, dim3(chunks), kChunk, st, posm, n, bb, nb, kin, idx);
     if (e != cudaSuccess) return e;
-    k_rank_gather<<<(unsigned)((n + 31) / 32), 32 * kRankWarps, 0, st>>>(posm, n, kin, idx, chunks, perm, sposm);
-    return cudaGetLastError();
+    return launch_chained(k_rank_gather, dim3((unsigned)((n + 31) / 32)), 32 * kRankWarps, st, posm,
+                          n, kin, idx, chunks, perm, sposm);
   }
   k_morton_keys<<<grid(n), kBT, 0, st>>>(posm, n, bb, nb, kin, idx);
   e = cudaGetLastError();

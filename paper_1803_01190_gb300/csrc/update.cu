@@ -118,6 +118,7 @@ __global__ void k_unpack_state(const real4<real> *__restrict__ posm,
 template <typename real>
 __global__ void k_store_acc(const real *__restrict__ part, const int32_t *__restrict__ perm, int S,
                             int64_t n, real G, real *__restrict__ acc) {
+  chain_begin();
   for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
     acc[4 * i + c] = gather_comp<real>(part, S, n, k, c, G);
   });
@@ -129,6 +130,7 @@ template <typename real>
 __global__ void k_acc_out(const real *__restrict__ part, const int32_t *__restrict__ perm, int S,
                           int64_t n, real G, double *__restrict__ acc3,
                           double *__restrict__ pot) {
+  chain_begin();
   for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
     const real a = gather_comp<real>(part, S, n, k, c, G);
     if (c < 3) {
@@ -173,6 +175,7 @@ template <typename real>
 __global__ void k_kdk_predict(int64_t n, real dt, real hdt, const real *__restrict__ posm,
                               const real *__restrict__ vel, const real *__restrict__ acc,
                               real *__restrict__ vbar, real *__restrict__ posm_nxt) {
+  chain_begin();
   for_components<real>(n, nullptr, [&](int64_t, int64_t i, int c) {
     const int64_t o = 4 * i + c;
     real vb, rn;
@@ -192,6 +195,7 @@ __global__ void k_kdk_correct_predict(const real *__restrict__ part,
                                       real chdt, real dt, real hdt, real *__restrict__ acc,
                                       const real *__restrict__ posm_new, real *__restrict__ vel,
                                       real *__restrict__ vbar, real *__restrict__ posm_pred) {
+  chain_begin();
   using O = ops<real>;
   for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
     const int64_t o = 4 * i + c;
@@ -219,6 +223,7 @@ __global__ void k_rk4_stage(const real *__restrict__ part, const int32_t *__rest
                             real *__restrict__ posm0, real *__restrict__ vel0,
                             real *__restrict__ vs, real *__restrict__ sr, real *__restrict__ sv,
                             real *__restrict__ posm_stage) {
+  chain_begin();
   using O = ops<real>;
   for_components<real>(n, perm, [&](int64_t k, int64_t i, int c) {
     const int64_t o = 4 * i + c;
@@ -351,22 +356,19 @@ cudaError_t launch_unpack_state(int mode, const void *posm, const void *velv, in
 cudaError_t launch_store_acc(int mode, const EpiIn &e, void *acc, cudaStream_t st) {
   const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_store_acc<float><<<g, b, 0, st>>>((const float *)e.part, e.perm, e.S, e.n, (float)e.G,
-                                        (float *)acc);
-  else
-    k_store_acc<double><<<g, b, 0, st>>>((const double *)e.part, e.perm, e.S, e.n, e.G,
-                                         (double *)acc);
-  return cudaGetLastError();
+    return launch_chained(k_store_acc<float>, g, b, st, (const float *)e.part, e.perm, e.S, e.n,
+                          (float)e.G, (float *)acc);
+  return launch_chained(k_store_acc<double>, g, b, st, (const double *)e.part, e.perm, e.S, e.n,
+                        e.G, (double *)acc);
 }
 
 cudaError_t launch_acc_out(int mode, const EpiIn &e, double *acc3, double *pot, cudaStream_t st) {
   const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_acc_out<float><<<g, b, 0, st>>>((const float *)e.part, e.perm, e.S, e.n, (float)e.G, acc3,
-                                      pot);
-  else
-    k_acc_out<double><<<g, b, 0, st>>>((const double *)e.part, e.perm, e.S, e.n, e.G, acc3, pot);
-  return cudaGetLastError();
+    return launch_chained(k_acc_out<float>, g, b, st, (const float *)e.part, e.perm, e.S, e.n,
+                          (float)e.G, acc3, pot);
+  return launch_chained(k_acc_out<double>, g, b, st, (const double *)e.part, e.perm, e.S, e.n, e.G,
+                        acc3, pot);
 }
 
 cudaError_t launch_unpack_acc(int mode, const void *acc, int64_t n, double *acc3, double *pot,
@@ -383,14 +385,12 @@ cudaError_t launch_kdk_predict(int mode, int64_t n, double dt, const void *posm_
                                cudaStream_t st) {
   const unsigned g = grid_for(4 * n), b = block_for(4 * n);
   if (mode == NBODY_FP32)
-    k_kdk_predict<float><<<g, b, 0, st>>>(n, (float)dt, (float)(dt / 2), (const float *)posm_cur,
-                                          (const float *)vel, (const float *)acc, (float *)vbar,
-                                          (float *)posm_nxt);
-  else
-    k_kdk_predict<double><<<g, b, 0, st>>>(n, dt, dt / 2, (const double *)posm_cur,
-                                           (const double *)vel, (const double *)acc,
-                                           (double *)vbar, (double *)posm_nxt);
-  return cudaGetLastError();
+    return launch_chained(k_kdk_predict<float>, g, b, st, n, (float)dt, (float)(dt / 2),
+                          (const float *)posm_cur, (const float *)vel, (const float *)acc,
+                          (float *)vbar, (float *)posm_nxt);
+  return launch_chained(k_kdk_predict<double>, g, b, st, n, dt, dt / 2, (const double *)posm_cur,
+                        (const double *)vel, (const double *)acc, (double *)vbar,
+                        (double *)posm_nxt);
 }
 
 cudaError_t launch_kdk_correct_predict(int mode, const EpiIn &e, double dt, double dt_next,
@@ -398,15 +398,14 @@ cudaError_t launch_kdk_correct_predict(int mode, const EpiIn &e, double dt, doub
                                        void *posm_pred, cudaStream_t st) {
   const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_kdk_correct_predict<float><<<g, b, 0, st>>>(
-        (const float *)e.part, e.perm, e.S, e.n, (float)e.G, (float)(dt / 2), (float)dt_next,
-        (float)(dt_next / 2), (float *)acc, (const float *)posm_new, (float *)vel, (float *)vbar,
-        (float *)posm_pred);
-  else
-    k_kdk_correct_predict<double><<<g, b, 0, st>>>(
-        (const double *)e.part, e.perm, e.S, e.n, e.G, dt / 2, dt_next, dt_next / 2, (double *)acc,
-        (const double *)posm_new, (double *)vel, (double *)vbar, (double *)posm_pred);
-  return cudaGetLastError();
+    return launch_chained(k_kdk_correct_predict<float>, g, b, st, (const float *)e.part, e.perm,
+                          e.S, e.n, (float)e.G, (float)(dt / 2), (float)dt_next,
+                          (float)(dt_next / 2), (float *)acc, (const float *)posm_new,
+                          (float *)vel, (float *)vbar, (float *)posm_pred);
+  return launch_chained(k_kdk_correct_predict<double>, g, b, st, (const double *)e.part, e.perm,
+                        e.S, e.n, e.G, dt / 2, dt_next, dt_next / 2, (double *)acc,
+                        (const double *)posm_new, (double *)vel, (double *)vbar,
+                        (double *)posm_pred);
 }
 
 cudaError_t launch_rk4_stage(int mode, const EpiIn &e, int stage, double dt, const void *posm0,
@@ -414,16 +413,13 @@ cudaError_t launch_rk4_stage(int mode, const EpiIn &e, int stage, double dt, con
                              cudaStream_t st) {
   const unsigned g = grid_for(4 * e.n), b = block_for(4 * e.n);
   if (mode == NBODY_FP32)
-    k_rk4_stage<float><<<g, b, 0, st>>>((const float *)e.part, e.perm, e.S, e.n, (float)e.G, stage,
-                                        (float)dt, (float)(dt / 2), (float)(dt / 6),
-                                        (float *)posm0, (float *)vel0, (float *)rk_vs,
-                                        (float *)rk_sr, (float *)rk_sv, (float *)posm_stage);
-  else
-    k_rk4_stage<double><<<g, b, 0, st>>>((const double *)e.part, e.perm, e.S, e.n, e.G, stage, dt,
-                                         dt / 2, dt / 6, (double *)posm0, (double *)vel0,
-                                         (double *)rk_vs, (double *)rk_sr, (double *)rk_sv,
-                                         (double *)posm_stage);
-  return cudaGetLastError();
+    return launch_chained(k_rk4_stage<float>, g, b, st, (const float *)e.part, e.perm, e.S, e.n,
+                          (float)e.G, stage, (float)dt, (float)(dt / 2), (float)(dt / 6),
+                          (float *)posm0, (float *)vel0, (float *)rk_vs, (float *)rk_sr,
+                          (float *)rk_sv, (float *)posm_stage);
+  return launch_chained(k_rk4_stage<double>, g, b, st, (const double *)e.part, e.perm, e.S, e.n,
+                        e.G, stage, dt, dt / 2, dt / 6, (double *)posm0, (double *)vel0,
+                        (double *)rk_vs, (double *)rk_sr, (double *)rk_sv, (double *)posm_stage);
 }
 
 cudaError_t launch_diag(int mode, const void *posm, const void *vel, const void *acc, int64_t n,
