@@ -366,7 +366,7 @@ __device__ __forceinline__ void fx_box_add(FxBox &b, const d4 &p) {
     b.lo[c] = min(b.lo[c], fx_key(h[c]));
     b.hi[c] = max(b.hi[c], fx_key(h[c]));
   }
-  bool bad = h[3] < 0 || (h[3] < 0x00100000 && p.w > 0.0);
+  bool bad = h[3] < 0 || (h[3] < 0x00100000 && (h[3] | __double2loint(p.w)) != 0);
 #pragma unroll
   for (int c = 0; c < 4; c++) bad |= (h[c] & 0x7FF00000) == 0x7FF00000;
   b.mmax = max(b.mmax, h[3]);
