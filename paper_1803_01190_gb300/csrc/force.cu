@@ -1276,6 +1276,24 @@ __device__ __forceinline__ double join_ff(float h, float l) {
   return finite ? f2d_exact(h) + f2d_exact(l) : (double)h + (double)l;
 }
 
+// -(x - c) of an i-particle against a tile's anchor c, exact but for the split:
+// the difference is taken in binary64, as the j side's is by the prep kernel, so
+// both are off by 2^-49 of their distance from the anchor.  From float-floats of
+// x and c each it would be off by 2^-49 of |x|, which is what bounded the
+// accelerations: their relative error at N = 65539 (disk and halo) 9.4e-15 so,
+// 5.1e-15 here, at the same time (32.5 ms for three evaluations: the FP64 pipe
+// is idle otherwise).
+__device__ __forceinline__ void ff_shift(const double (&x)[3], const double (&c)[3],
+                                         float2 (&nh)[3], float2 (&nl)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    float h, l;
+    split_ff(c[k] - x[k], h, l);
+    nh[k] = f2(h, h);
+    nl[k] = f2(l, l);
+  }
+}
+
 // A pair's geometry: d, y = 1/r and q = 1/r^2 as float-float, for one tile entry
 // (j = 2k, 2k+1 as H = (xh0, xh1, yh0, yh1), H2 = (zh0, zh1, mh0, mh1), L, L2 the
 // matching low parts) and the negated float-float i coordinates (nxh, ...) in
@@ -1454,17 +1472,14 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
     const float e2hs = (float)u.eps2;
     const float e2ls = (float)(u.eps2 - (double)e2hs);
     const float2 e2h = f2(e2hs, e2hs), e2l = f2(e2ls, e2ls);
-    float xh[R][3], xl[R][3];
-    double acc[R][4];
+    double x[R][3], acc[R][4];
 #pragma unroll
     for (int r = 0; r < R; r++) {
       const int li = r * IT + it;
       const d4 p = posm[u.i0 + (li < u.ni ? li : 0)];
-      const double c3[3] = {p.x, p.y, p.z};
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        split_ff(c3[c], xh[r][c], xl[r][c]);
-      }
+      x[r][0] = p.x;
+      x[r][1] = p.y;
+      x[r][2] = p.z;
 #pragma unroll
       for (int c = 0; c < 4; c++) acc[r][c] = 0.0;
     }
@@ -1475,20 +1490,11 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
       __syncthreads();
       const int64_t tt = u.anchor + (jt - u.j0) / T;
       const float4 ch = anchor[2 * tt], cl = anchor[2 * tt + 1];
-      const float chv[3] = {ch.x, ch.y, ch.z}, clv[3] = {cl.x, cl.y, cl.z};
+      const double ct[3] = {join_ff(ch.x, cl.x), join_ff(ch.y, cl.y), join_ff(ch.z, cl.z)};
       float2 nh[R][3], nl[R][3], ah[R][4], al[R][4];
 #pragma unroll
       for (int r = 0; r < R; r++) {
-#pragma unroll
-        for (int c = 0; c < 3; c++) {  // -(x_i - c_t) as float-float
-          float s, e;
-          two_sum1(xh[r][c], -chv[c], s, e);
-          const float t = __fadd_rn(__fsub_rn(xl[r][c], clv[c]), e);
-          float h, l;
-          two_sum1(s, t, h, l);
-          nh[r][c] = f2(-h, -h);
-          nl[r][c] = f2(-l, -l);
-        }
+        ff_shift(x[r], ct, nh[r], nl[r]);
 #pragma unroll
         for (int c = 0; c < 4; c++) ah[r][c] = al[r][c] = f2(0.0f, 0.0f);
       }
@@ -1648,27 +1654,18 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
     tL2[tid] = make_float4(alo.z, blo.z, alo.w, blo.w);
   }
   const float4 ch = anchor[2 * J], cl = anchor[2 * J + 1];
-  const float chv[3] = {ch.x, ch.y, ch.z}, clv[3] = {cl.x, cl.y, cl.z};
+  const double ct[3] = {join_ff(ch.x, cl.x), join_ff(ch.y, cl.y), join_ff(ch.z, cl.z)};
   float2 nh[R][3], nl[R][3], ah[R][4], al[R][4], mh[R], ml[R];
 #pragma unroll
   for (int r = 0; r < R; r++) {
     const int64_t i = i0 + r * BT + tid;
     // beyond n: massless, 1e18 from the anchor (finite r^2, zero contribution)
     const d4 pi = i < n ? posm[i] : d4{0.0, 0.0, 0.0, 0.0};
-    const double c3[3] = {pi.x, pi.y, pi.z};
+    const double x[3] = {pi.x, pi.y, pi.z};
+    ff_shift(x, ct, nh[r], nl[r]);
+    if (i >= n)
 #pragma unroll
-    for (int c = 0; c < 3; c++) {  // -(x_i - c_J) as float-float
-      float xh, xl;
-      split_ff(c3[c], xh, xl);
-      float s, e;
-      two_sum1(xh, -chv[c], s, e);
-      const float t = __fadd_rn(__fsub_rn(xl, clv[c]), e);
-      float h, l;
-      two_sum1(s, t, h, l);
-      if (i >= n) h = 1e18f, l = 0.0f;
-      nh[r][c] = f2(-h, -h);
-      nl[r][c] = f2(-l, -l);
-    }
+      for (int c = 0; c < 3; c++) nh[r][c] = f2(-1e18f, -1e18f), nl[r][c] = f2(0.0f, 0.0f);
     float m_h, m_l;
     split_ff(pi.w, m_h, m_l);
     mh[r] = f2(m_h, m_h);
@@ -1923,7 +1920,14 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
     }
   }
   __syncthreads();
-  const double c[3] = {med[0], med[1], med[2]};
+  double c[3] = {med[0], med[1], med[2]};
+  if (FF)  // as the force kernels will read it back, to the last bit
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      float h, l;
+      split_ff(c[q], h, l);
+      c[q] = join_ff(h, l);
+    }
   if (tid < cnt) {
     const double dx = p.x - c[0], dy = p.y - c[1], dz = p.z - c[2];
     const float hx = __double2float_rn(dx), hy = __double2float_rn(dy), hz = __double2float_rn(dz),

@@ -1,0 +1,46 @@
+"""F64E: both sides of a pair are taken from the tile's anchor in binary64.
+
+A system far from the origin keeps the accuracy of one at it: coordinates are
+off by 2^-49 of their distance from the anchor, not of their magnitude.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nb():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    import paper_1803_01190_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("n", [2, 257, 700, 2049])
+@pytest.mark.parametrize("sym", [0, 1])
+@pytest.mark.parametrize("equal", [True, False])
+def test_far_from_the_origin(nb, n, sym, equal):
+    rng = np.random.default_rng(n)
+    pos = np.array([4096.0, -3000.0, 1.0e4]) + rng.random((n, 3))
+    mass = np.full(n, 1.0 / n) if equal else rng.uniform(0.5, 2.0, n) / n
+    eps = 0.05
+    with nb.Simulation(n, "f64e", eps=eps) as sim:
+        sim.set_symmetric(sym if n > 256 else 0)
+        acc, pot = sim.accel(pos, mass)
+    oa, op, _ = oracle.accel(pos, mass, eps)
+    # |x - c| < 1: each coordinate of a difference is off by at most 2^-49 from
+    # either split and 2^-47 from adding the low parts, 2.5e-14 in all three; a
+    # term m d / r^3 changes by at most 4 m / r^3 of that, m / r by m / r^2, and
+    # the float-float arithmetic adds 2^-43 of a term
+    r2 = ((pos[:, None] - pos[None]) ** 2).sum(2) + eps * eps
+    np.fill_diagonal(r2, np.inf)
+    bound = (mass / r2 ** 1.5).sum(1) * 1e-13 + (mass / r2).sum(1) * 2.0 ** -43
+    assert (np.linalg.norm(acc - oa, axis=1) <= bound).all()
+    bound = (mass / r2).sum(1) * 2.5e-14 + (mass / r2 ** 0.5).sum(1) * 2.0 ** -43
+    assert (np.abs(pot - op) <= bound).all()
