@@ -44,9 +44,9 @@ EPS, DT = 0.02, 5e-4
 # the pipe that binds is the FMA-heavy one.
 FP64_INSTR_PER_INTERACTION = {False: 9, True: 6}
 # FMA-heavy pipe cycles per warp and interaction of the fixed-point kernels,
-# equal masses, by ncu (sm__pipe_fmaheavy_cycles_active at N = 16384): each
-# pair once, 273 per pair.
-FX_HEAVY_CYCLES_PER_INTERACTION = {True: 136.5}
+# equal masses, by ncu (sm__pipe_fmaheavy_cycles_active): 263 one-sided (N =
+# 16384); each pair once 268 per pair (N = 32768).
+FX_HEAVY_CYCLES_PER_INTERACTION = {False: 263, True: 134}
 # FP32 FMA-pipe lane operations: mixed 13 (3 differences, 3 FMAs for
 # |d|^2 + eps^2, m y, y^2, m y^3, 3 FMAs and 1 add into the sums; two j per
 # packed instruction; 12 in tiles of equal masses, this workload's); F64E
@@ -466,17 +466,19 @@ def roofline_fp64(n, sym, force_ms, step_ms, pipes):
     ipi = FP64_INSTR_PER_INTERACTION[sym]
     achieved = inter * ipi / (force_ms * 1e-3) / 1e9
     conv = inter * FLOP_PER_INTERACTION / (force_ms * 1e-3) / 1e12
-    heavy = FX_HEAVY_CYCLES_PER_INTERACTION.get(sym)
+    heavy = FX_HEAVY_CYCLES_PER_INTERACTION[sym]
     heavy_peak = 4 * pipes["sms"] * pipes["sm_mhz"] / 1e3
-    heavy_achieved = heavy and inter / 32 * heavy / (force_ms * 1e-3) / 1e9
+    heavy_achieved = inter / 32 * heavy / (force_ms * 1e-3) / 1e9
     return {"bound": "alu", "pipe": "fp64", "kernel": "k_force_fx_sym" if sym else "k_force_f64",
-            "integer_pipe": heavy and {
+            "integer_pipe": {
                 "pipe": "fma heavy", "cycles_per_warp_interaction": heavy, "achieved": heavy_achieved,
                 "peak": heavy_peak, "unit": "G pipe cycles/s", "frac": heavy_achieved / heavy_peak,
                 "note": "fixed-point pair sums: 32 x 32 -> 64 products of 4 cycles a warp; peak = "
                         "4 sub-partitions x SMs x the SM clock of this run"},
             "achieved": achieved, "peak": pipes["dfma_ginstr_s"], "unit": "G FP64-pipe instr/s",
             "frac": achieved / pipes["dfma_ginstr_s"],
+            "frac_note": "FP64 instructions that the binary64 pair body would issue; the fixed-point "
+                         "kernels do not issue them and are bound by the pipe of integer_pipe",
             "peak_source": (f"measured in this run: nbody_measure_pipes DFMA issue rate "
                             f"({pipes['dfma_per_clk_sm']:.3f}/clk/SM x {pipes['sms']:.0f} SMs at "
                             f"{pipes['sm_mhz']:.0f} MHz)"),
