@@ -146,9 +146,18 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
     // N = 131072 at 8, 16 and 24 segments 2449, 2549, 2557; 300000 at 4, 8, 32:
     // 2462, 2543, 2568; 2^20 at 2, 4, 16: 2550, 2556, 2562; one-sided FP64 65536
     // at 8, 16, 32: 128, 131, 132)
+    // (MIXED, whose sums are compensated, and the binary64 modes; FP32's segment
+    // count is part of its rounding and stays a function of n alone: eight waves
+    // of R = 1 or, from a full wave of them, 2)
     const int64_t slots = (int64_t)c->num_sms * occ;
     s = std::max<int64_t>((8 * slots + bx - 1) / bx,
                           std::min<int64_t>((32 * slots + bx - 1) / bx, smax / 16));
+    if (c->mode == NBODY_FP32) {
+      const int rs = r_req ? r_req : (int64_t)sh.bt * 2 * c->num_sms > c->n ? 1 : 2;
+      const int64_t rows = (int64_t)sh.bt * rs, b = (c->n + rows - 1) / rows;
+      const int resident = rs == 1 ? 5 : rs == 2 ? 4 : rs == 4 ? 2 : 1;
+      s = (8LL * c->num_sms * resident + b - 1) / b;
+    }
   }
   if (s > smax) s = smax;
   if (s > 64) s = 64;

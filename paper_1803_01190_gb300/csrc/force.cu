@@ -1159,7 +1159,11 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 // EQUAL leaves the mass out: the sums are those of 1/r^3 and 1/r, multiplied by
 // the tile's one mass when they are folded: 12 lane operations instead of 13.
 // Measured at N = 131072: MIXED 2735 Gint/s against 2545, FP32 (R = 2) 2731
-// against 2620.
+// against 2620 (there for masses that are powers of two, in the binary32 kernel).
+// Masses up to 1 alone, so that no term is smaller than with the mass, and from
+// eps = 2^-40, so that 1/r^3 is finite: systems in other units (masses in kg at
+// distances in m) keep the mass in the body, where it brings 1/r^3 into range.
+__device__ __forceinline__ bool leave_mass_out(float eps2) { return eps2 >= 0x1p-80f; }
 template <bool MASK, bool REFINE, bool EQUAL = false>
 __device__ __forceinline__ void body_pair(const float4 &A, const float4 &B, float2 nx, float2 ny,
                                           float2 nz, float2 e2, float2 &ax, float2 &ay,
@@ -1472,6 +1476,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
     const float e2hs = (float)u.eps2;
     const float e2ls = (float)(u.eps2 - (double)e2hs);
     const float2 e2h = f2(e2hs, e2hs), e2l = f2(e2ls, e2ls);
+    const bool no_mass = leave_mass_out(e2hs);
     double x[R][3], acc[R][4];
 #pragma unroll
     for (int r = 0; r < R; r++) {
@@ -1501,7 +1506,8 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
       const int np = (cnt + 1) / 2;
       const int k0 = np * jw / IW, k1 = np * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      const bool full = cnt == T && !diag, equal = full && ch.w != 0.0f;
+      const bool full = cnt == T && !diag;
+      const bool equal = full && ch.w != 0.0f && no_mass;
       if (full) {  // k1 - k0 is a multiple of FF_STEPS
         if (equal)
           ff_tile<R, true>(tH, tH2, tL, tL2, k0, k1, nh, nl, e2h, e2l, ah, al);
@@ -1674,7 +1680,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
     for (int c = 0; c < 4; c++) ah[r][c] = al[r][c] = f2(0.0f, 0.0f);
   }
   __syncthreads();
-  const bool equal = ch.w != 0.0f && anchor[2 * I].w != 0.0f;
+  const bool equal = ch.w != 0.0f && anchor[2 * I].w != 0.0f && leave_mass_out(e2hs);
   if (equal)
     ff_sym_tile<R, NE, T, true>(tH, tH2, tL, tL2, nh, nl, mh, ml, e2h, e2l, ah, al, colw[warp]);
   else
@@ -1710,7 +1716,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e_sym(const d4 *__restrict__ po
 // ---------------------------------------------------------------- mixed
 // fpos[j] = (x_j - c_t, y_j - c_t, z_j - c_t, m_j) in binary32, c_t the anchor of
 // j's tile; anchor[2t] = float hi part of c_t, anchor[2t+1] = float lo part;
-// anchor[2t].w = the mass of a full tile of equal masses, or 0.
+// anchor[2t].w = the mass of a full tile of equal masses up to 1, or 0.
 template <int BT, int R, int T, class W>
 __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
                                                     const float4 *__restrict__ fpos,
@@ -1723,6 +1729,7 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
     const int tid = threadIdx.x;
     const int64_t j1 = u.j0 + u.nj;
     const float2 e2 = f2((float)u.eps2, (float)u.eps2);
+    const bool no_mass = leave_mass_out(e2.x);
     float xh[R], yh[R], zh[R], xl[R], yl[R], zl[R];
     float axh[R], axl[R], ayh[R], ayl[R], azh[R], azl[R], pth[R], ptl[R];
 #pragma unroll
@@ -1759,7 +1766,7 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
       }
       const int np = (cnt + 1) / 2;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      const bool equal = ch.w != 0.0f;
+      const bool equal = ch.w != 0.0f && no_mass;
       if (cnt == T && !diag && equal) {
 #pragma unroll(R == 1 ? 2 : 4)
         for (int k = 0; k < T / 2; k++) {
@@ -1946,7 +1953,7 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
   if (tid == 0) {
     const float hx = __double2float_rn(c[0]), hy = __double2float_rn(c[1]),
                 hz = __double2float_rn(c[2]);
-    anchor[2 * t] = make_float4(hx, hy, hz, equal ? __double2float_rn(p.w) : 0.0f);
+    anchor[2 * t] = make_float4(hx, hy, hz, equal && p.w <= 1.0 ? __double2float_rn(p.w) : 0.0f);
     anchor[2 * t + 1] = make_float4(__double2float_rn(c[0] - (double)hx),
                                     __double2float_rn(c[1] - (double)hy),
                                     __double2float_rn(c[2] - (double)hz), 0.0f);
@@ -1954,24 +1961,44 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
 }
 
 // ---------------------------------------------------------------- binary32 (paper's SP)
-template <int BT, int R, int T, int IW, class W>
+// Tiles of equal masses run without the mass when it is a power of two (masses
+// 1 / 2^k, as of equal-mass systems of 2^k particles): the sums are then held in
+// units of it, which changes no bit of them.  Other masses keep the product in
+// the body: sums in another rounding would move single precision positions, and
+// with them close pairs at a small softening, by as much as its whole error.
+// The range of masses and the softening keep 1/r^3 and the sums in units of the
+// mass finite (1/r <= 2^20) and not smaller than with it (m <= 1).
+__device__ __forceinline__ bool f32_unit_mass(float m, float eps2) {
+  return (__float_as_uint(m) & 0x807FFFFFu) == 0 && m <= 1.0f && m >= 0x1p-40f && eps2 >= 0x1p-40f;
+}
+template <int BT, int R, int T, class W>
 __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ posm, W work,
                                                   float4 *__restrict__ part) {
   chain_begin();
-  constexpr int IT = BT / IW;
   __shared__ float4 tA[T / 2], tB[T / 2];
-  __shared__ float4 red[IW > 1 ? BT : 1];
   for (int64_t uk = work.first(); uk < work.count(); uk += work.stride()) {
     const Unit u = work.get(uk);
     const int tid = threadIdx.x;
-    // i-thread, share of the j-tile
-  const int it = IW == 1 ? tid : tid % IT, jw = IW == 1 ? 0 : tid / IT;
     const int64_t j1 = u.j0 + u.nj;
     const float2 e2 = f2((float)u.eps2, (float)u.eps2);
     float2 nx[R], ny[R], nz[R], ax[R], ay[R], az[R], pt[R];
+    float unit = 1.0f;  // of the sums
+    auto in_units_of = [&](float m) {
+      if (m == unit) return;
+      const float f = unit / m;  // of powers of two: exact
+      const float2 f_2 = f2(f, f);
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        ax[r] = __fmul2_rn(ax[r], f_2);
+        ay[r] = __fmul2_rn(ay[r], f_2);
+        az[r] = __fmul2_rn(az[r], f_2);
+        pt[r] = __fmul2_rn(pt[r], f_2);
+      }
+      unit = m;
+    };
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int li = r * IT + it;
+      const int li = r * BT + tid;
       const float4 p = posm[u.i0 + (li < u.ni ? li : 0)];
       nx[r] = f2(-p.x, -p.x);
       ny[r] = f2(-p.y, -p.y);
@@ -1983,35 +2010,26 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
       __syncthreads();
       load_pairs<BT, T>(posm, jt, cnt, tA, tB);
       const float m = posm[jt].w;
-      const bool equal = __syncthreads_and(tid < cnt && posm[jt + min(tid, cnt - 1)].w == m);
+      const bool equal = __syncthreads_and(tid < cnt && posm[jt + min(tid, cnt - 1)].w == m) &&
+                         f32_unit_mass(m, e2.x);
       const int np = (cnt + 1) / 2;
-      const int k0 = np * jw / IW, k1 = np * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
       if (cnt == T && !diag && equal) {
-        float2 sx[R], sy[R], sz[R], sp[R];
-#pragma unroll
-        for (int r = 0; r < R; r++) sx[r] = sy[r] = sz[r] = sp[r] = f2(0.0f, 0.0f);
+        in_units_of(m);
 #pragma unroll 2
-        for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
+        for (int k = 0; k < T / 2; k++) {
           const float4 A = tA[k], B = tB[k];
 #pragma unroll
           for (int r = 0; r < R; r++)
-            body_pair<false, false, true>(A, B, nx[r], ny[r], nz[r], e2, sx[r], sy[r], sz[r],
-                                         sp[r], false, false);
-        }
-        const float2 m2 = f2(m, m);
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-          ax[r] = __ffma2_rn(sx[r], m2, ax[r]);
-          ay[r] = __ffma2_rn(sy[r], m2, ay[r]);
-          az[r] = __ffma2_rn(sz[r], m2, az[r]);
-          pt[r] = __ffma2_rn(sp[r], m2, pt[r]);
+            body_pair<false, false, true>(A, B, nx[r], ny[r], nz[r], e2, ax[r], ay[r], az[r],
+                                         pt[r], false, false);
         }
         continue;
       }
+      in_units_of(1.0f);
       if (cnt == T && !diag) {
 #pragma unroll 2
-        for (int k = IW == 1 ? 0 : k0; k < (IW == 1 ? T / 2 : k1); k++) {
+        for (int k = 0; k < T / 2; k++) {
           const float4 A = tA[k], B = tB[k];
 #pragma unroll
           for (int r = 0; r < R; r++)
@@ -2019,24 +2037,26 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
                                     false, false);
         }
       } else {
-        for (int k = k0; k < k1; k++) {
+        for (int k = 0; k < np; k++) {
           const float4 A = tA[k], B = tB[k];
           const int64_t j = jt + 2 * k;
 #pragma unroll
           for (int r = 0; r < R; r++) {
-            const int64_t i = u.i0 + r * IT + it;
+            const int64_t i = u.i0 + r * BT + tid;
             body_pair<true, false>(A, B, nx[r], ny[r], nz[r], e2, ax[r], ay[r], az[r], pt[r],
                                    j == i, j + 1 == i);
           }
         }
       }
     }
+    in_units_of(1.0f);
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const int li = r * IT + it;
-      const float4 v = make_float4(__fadd_rn(ax[r].x, ax[r].y), __fadd_rn(ay[r].x, ay[r].y),
-                                   __fadd_rn(az[r].x, az[r].y), __fadd_rn(pt[r].x, pt[r].y));
-      store_shares<IW>(part, work.get(uk), li, v, red, it, IT, jw);
+      const int li = r * BT + tid;
+      const Unit w = work.get(uk);  // again: not kept in registers over the pair loop
+      if (li >= w.w0 && li < min(w.ni, w.w1))
+        part[w.out + li] = make_float4(__fadd_rn(ax[r].x, ax[r].y), __fadd_rn(ay[r].x, ay[r].y),
+                                       __fadd_rn(az[r].x, az[r].y), __fadd_rn(pt[r].x, pt[r].y));
     }
   }
 }
@@ -2051,17 +2071,17 @@ int force_block_threads(int mode) {
   return mode == NBODY_FP64 ? BT_F64 : mode == NBODY_F64E ? BT_FF : BT_F32;
 }
 // Warps of a block that share i-particles at small n: all of them.
-constexpr int IW_F64 = BT_F64 / 32, IW_F32 = BT_F32 / 32, IW_FF = BT_FF / 32;
+constexpr int IW_F64 = BT_F64 / 32, IW_FF = BT_FF / 32;
 int force_split(int mode) {
-  return mode == NBODY_FP64 ? IW_F64 : mode == NBODY_F64E ? IW_FF : mode == NBODY_FP32 ? IW_F32 : 1;
+  return mode == NBODY_FP64 ? IW_F64 : mode == NBODY_F64E ? IW_FF : 1;
 }
 // Measured on GB300 (force kernel, split against one i-particle per thread, us):
 // FP64 N = 1000 23 / 57, 3000 88 / 111, 4096 147 / 162, 6000 299 / 308; F64E 1000
-// 14 / 35, 4096 88 / 100, 6000 174 / 187; FP32 3000 12.0 / 14.9, 5000 20.9 / 22.5,
-// 6000 26.5 / 26.6.  MIXED is not split: a pair costs it so little that what a
-// thread does once per i-particle weighs more (4096: 39 / 18).
+// 14 / 35, 4096 88 / 100, 6000 174 / 187.  MIXED is not split: a pair costs it so
+// little that what a thread does once per i-particle weighs more (4096: 39 / 18);
+// FP32 neither: its sums keep their order (see above).
 int64_t force_split_max_n(int mode) {
-  return mode == NBODY_MIXED ? 0 : mode == NBODY_FP32 ? 6144 : 8192;
+  return mode == NBODY_FP64 || mode == NBODY_F64E ? 8192 : 0;
 }
 int force_tile(int mode) { return mode == NBODY_FP64 ? T_F64 : mode == NBODY_F64E ? T_FF : T_F32; }
 
@@ -2079,7 +2099,7 @@ static const void *kernel_for(int mode) {
     case NBODY_FP64: return (const void *)k_force_f64<BT_F64, R, T_F64, 1, DenseWork>;
     case NBODY_MIXED: return (const void *)k_force_mixed<BT_F32, R, T_F32, DenseWork>;
     case NBODY_F64E: return (const void *)k_force_f64e<BT_FF, (R < 4 ? R : 4), T_FF, 1, DenseWork>;
-    default: return (const void *)k_force_f32<BT_F32, R, T_F32, 1, DenseWork>;
+    default: return (const void *)k_force_f32<BT_F32, R, T_F32, DenseWork>;
   }
 }
 
@@ -2126,7 +2146,7 @@ static cudaError_t launch_rw(int mode, const void *posm, const float4 *fpos, con
   if (mode == NBODY_F64E)
     return launch_k(w, k_force_f64e<BT_FF, (R < 4 ? R : 4), T_FF, SPLIT ? IW_FF : 1, W>, grid,
                     BT_FF, st, (const d4 *)posm, fpos, anchor, w, (d4 *)part);
-  return launch_k(w, k_force_f32<BT_F32, R, T_F32, SPLIT ? IW_F32 : 1, W>, grid, BT_F32, st,
+  return launch_k(w, k_force_f32<BT_F32, R, T_F32, W>, grid, BT_F32, st,
                   (const float4 *)posm, w, (float4 *)part);
 }
 
