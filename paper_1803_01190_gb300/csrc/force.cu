@@ -1767,8 +1767,12 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
       const int np = (cnt + 1) / 2;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
       const bool equal = ch.w != 0.0f && no_mass;
+      // R = 1 is the small-N shape, of few warps per SM: eight pair steps in flight.
+      // A KDK step at unroll 2, 4, 8 (us): N = 2048 28.2, 27.9, 26.3; 16387 153.0,
+      // 152.6, 143.9; 32768 471, 471, 463.  R = 2 at unroll 2, 4: 2500, 2517 Gint/s
+      // at N = 131072.
       if (cnt == T && !diag && equal) {
-#pragma unroll(R == 1 ? 2 : 4)
+#pragma unroll(R == 1 ? 8 : 4)
         for (int k = 0; k < T / 2; k++) {
           const float4 A = tA[k], B = tB[k];
 #pragma unroll
@@ -1777,8 +1781,7 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
                                          sp[r], false, false);
         }
       } else if (cnt == T && !diag) {
-// unroll 2 / 4 measured at N = 131072: R = 1 2446 / 2406 Gint/s, R = 2 2500 / 2517
-#pragma unroll(R == 1 ? 2 : 4)
+#pragma unroll(R == 1 ? 8 : 4)
         for (int k = 0; k < T / 2; k++) {
           const float4 A = tA[k], B = tB[k];
 #pragma unroll
@@ -1787,7 +1790,7 @@ __global__ void __launch_bounds__(BT) k_force_mixed(const d4 *__restrict__ posm,
                                    false, false);
         }
       } else {
-#pragma unroll(R == 1 ? 2 : 1)
+#pragma unroll(R == 1 ? 8 : 1)
         for (int k = 0; k < np; k++) {
           const float4 A = tA[k], B = tB[k];
           const int64_t j = jt + 2 * k;
