@@ -1471,7 +1471,7 @@ __global__ void __launch_bounds__(BT) k_force_f64e(const d4 *__restrict__ posm,
     const Unit u = work.get(uk);
     const int tid = threadIdx.x;
     // i-thread, share of the j-tile
-  const int it = IW == 1 ? tid : tid % IT, jw = IW == 1 ? 0 : tid / IT;
+    const int it = IW == 1 ? tid : tid % IT, jw = IW == 1 ? 0 : tid / IT;
     const int64_t j1 = u.j0 + u.nj;
     const float e2hs = (float)u.eps2;
     const float e2ls = (float)(u.eps2 - (double)e2hs);
