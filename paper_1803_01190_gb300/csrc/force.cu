@@ -1038,7 +1038,8 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
     for (int w = 0; w < NW; w++) fx_box_join(bj, sbox[w]);
     FxScale sc = fx_scale(bi, bj, eps2);
     const bool ok = sc.ok && oki, wide = sc.wide || widei;
-    if (!ok) sc.L = sc.em = emi = 0;  // the integer sums stay zero
+    const int emc = ok ? emi : 0;     // of the row block's masses, in this tile
+    if (!ok) sc.L = sc.em = 0;        // the integer sums stay zero
     {
       uint64_t X[3];
       fx_coords(pj, sc.L, X);
@@ -1056,9 +1057,9 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
         equali && tid < cnt && __double_as_longlong(pj.w) == __double_as_longlong(mj0));
     const FxMode mode = wide || !ok ? FX_WIDE : equal ? FX_EQUAL : FX_NARROW;
     const FxEps e2 = fx_eps2(eps2, sc.L);
-    const int emr = mode == FX_EQUAL ? FX_EQ_EM : sc.em, emc = mode == FX_EQUAL ? FX_EQ_EM : emi;
-    double fs = fx_exp2(fx_force_exp(sc.L, emr) + 32), ps = fx_exp2(fx_pot_exp(sc.L, emr) + 32);
-    double gs = fx_exp2(fx_force_exp(sc.L, emc) + 32), qs = fx_exp2(fx_pot_exp(sc.L, emc) + 32);
+    const int er = mode == FX_EQUAL ? FX_EQ_EM : sc.em, ec = mode == FX_EQUAL ? FX_EQ_EM : emc;
+    double fs = fx_exp2(fx_force_exp(sc.L, er) + 32), ps = fx_exp2(fx_pot_exp(sc.L, er) + 32);
+    double gs = fx_exp2(fx_force_exp(sc.L, ec) + 32), qs = fx_exp2(fx_pot_exp(sc.L, ec) + 32);
     if (mode == FX_EQUAL) {
       fs *= mj0;
       ps *= mj0;
@@ -1074,7 +1075,7 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
       fx_coords(p, sc.L, Xi[r]);
       const double m = i < n ? p.w : 0.0;
       const uint32_t mh = (uint32_t)__double2hiint(m), ml = (uint32_t)__double2loint(m);
-      Mi[r] = wide ? fx_mass<true>(mh, ml, emi) : fx_mass<false>(mh, ml, emi);
+      Mi[r] = wide ? fx_mass<true>(mh, ml, emc) : fx_mass<false>(mh, ml, emc);
     }
     if (mode == FX_WIDE)
       fx_sym_tile<BT, R, T, FX_WIDE>(posm, n, i0, eps2, ok, e2, tile, txy, tzm, tdm, cnt, Xi, Mi,

@@ -137,3 +137,28 @@ def test_negative_mass(nb):
     a2, p2, _ = oracle.accel(pos, np.maximum(-mass, 0.0), eps)
     assert np.abs(acc - (a1 - a2)).max() <= 1e-12 * np.abs(a1).max()
     assert np.abs(pot - (p1 - p2)).max() <= 1e-12 * np.abs(p1).max()
+
+
+# A tile that the fixed point does not take must leave the ones after it alone: the
+# first half of a column block holds a tracer far below the other masses, the second
+# half none
+@pytest.mark.parametrize("masses", ["light", "heavy", "one mass"])
+@pytest.mark.parametrize("tracer", [1e-25, 0.5, -1.0])
+@pytest.mark.parametrize("n", [512, 1000])
+def test_tile_after_a_refused_one(nb, masses, tracer, n):
+    pos, mass, eps = _case("plain", n)
+    rng = np.random.default_rng(n)
+    if masses == "light":
+        mass = 1e-5 * rng.uniform(1.0, 9.0, n)
+    elif masses == "heavy":
+        mass = np.exp2(rng.uniform(0.0, 6.0, n)) * 100
+    mass[256 + 10] = tracer * mass[0]
+    with nb.Simulation(n, "fp64", eps=eps) as sim:
+        sim.set_symmetric(1)
+        acc, pot = sim.accel(pos, mass)
+    if tracer > 0:
+        _check(pos, mass, eps, acc, pot)
+    else:  # the oracle takes no negative masses: the sum of both signs' parts
+        (a1, p1, s1), (a2, p2, s2) = (oracle.accel(pos, np.maximum(q, 0.0), eps) for q in (mass, -mass))
+        ok, err, _ = fp64_accel_gate(acc, a1 - a2, s1 + s2, n)
+        assert ok.all() and np.all(np.abs(pot - (p1 - p2)) <= 1e-12 * (np.abs(p1) + np.abs(p2)))
