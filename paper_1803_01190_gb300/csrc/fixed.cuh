@@ -298,6 +298,10 @@ struct FxTerm {
 FX_HD FxTerm fx_align(uint32_t w0, uint32_t w1, int32_t w2, int s) {
   return FxTerm{fx_shr(w0, w1, s), fx_shr(w1, (uint32_t)w2, s), w2 >> s};
 }
+// R, unsigned: 2^63 where x = 1/4 (r^2 a power of four)
+FX_HD FxTerm fx_align_r(const FxPair &p) {
+  return FxTerm{fx_shr(0, p.Rl, p.sp), fx_shr(p.Rl, p.Rh, p.sp), (int32_t)(p.Rh >> p.sp)};
+}
 // D_c F, unaligned
 template <bool ALU>
 FX_HD FxTerm fx_force(const FxPair &p, int c, int32_t fh, int32_t fl) {
@@ -336,7 +340,7 @@ FX_HD void fx_side(const FxPair &p, const FxMass &M, fx96 (&f)[3], fx96 &pot) {
 constexpr int FX_EQ_EM = -2;
 template <bool ALU>
 FX_HD void fx_both(const FxPair &p, fx96 (&f)[3], fx96 &pot, fx96 (*g)[3], fx96 *gpot) {
-  const FxTerm y = fx_align(0, p.Rl, (int32_t)p.Rh, p.sp);
+  const FxTerm y = fx_align_r(p);
   fx_add(pot, y.w0, y.w1, (uint32_t)y.w2);
   if (gpot) fx_add(*gpot, y.w0, y.w1, (uint32_t)y.w2);
   const uint64_t F = fx_mulhi64<ALU>(p.Rh, p.Rl, p.Qh, p.Ql);

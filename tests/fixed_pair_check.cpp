@@ -7,6 +7,8 @@
 // the 16-bit products of the low words: below 2^-52 r at r = 2^51 u).  With an
 // exponent of its own a mass is as exact as the largest, down to the last place
 // of the sums (2^-57 of the largest mass's force at the tile's extent).
+// Then pairs with r^2 exactly a power of four, where x = 1/4 and 1/r is at the
+// top of its range: prints the largest error of both terms in units of 2^-57.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -95,6 +97,38 @@ const ld ratio = equal ? 1 : (ld)mmax / m;
     if (!wide) bias += (double)rel, plain++;
     used++;
   }
-  printf("%ld %ld %ld %.4f %.4f %.3e\n", used, close, wrong, worst_f, worst_p, bias / plain);
+  double worst_4 = 0;
+  for (int k = -40; k <= 3; k++)  // r = 2^k at a unit of 2^(4 - FX_BITS)
+    for (int axis = 0; axis < 2; axis++)
+      for (int seed = -2; seed <= 2; seed++) {
+        const int L = 4 - FX_BITS;
+        const double r = std::exp2(k), d = axis ? r : r / 2, eps2 = axis ? 0.0 : r * r / 4;
+        if (std::exp2(51 + L) >= r) continue;
+        const uint64_t Xi[3] = {0, 0, 0}, q = fx_coord(hi(d), lo(d), L);
+        const uint64_t Xj[3] = {q, axis ? 0 : q, axis ? 0 : 0 - q};
+        FxPair p;
+        fx_geometry<false>(Xj, Xi, fx_eps2(eps2, L), [&](uint32_t x) {
+          const float y = (float)(1.0 / std::sqrt((double)(float)x)) * (1.0f + (float)seed * 0x1p-23f);
+          uint32_t b;
+          memcpy(&b, &y, 4);
+          return b;
+        }, p);
+        for (int form = 0; form < 3; form++) {  // equal, one exponent, an exponent each
+          fx96 f[3] = {}, pot = {};
+          const FxMass M = form == 1 ? fx_mass<false>(hi(1.0), 0, 0) : fx_mass<true>(hi(1.0), 0, 0);
+          if (form == 0)
+            fx_both<false>(p, f, pot, nullptr, nullptr);
+          else if (form == 1)
+            fx_side<false, false>(p, M, f, pot);
+          else
+            fx_side<false, true>(p, M, f, pot);
+          const int em = form ? 0 : FX_EQ_EM;
+          const ld ep = value(pot, fx_pot_exp(L, em)) * r - 1;
+          const ld ef = value(f[0], fx_force_exp(L, em)) * r * r * r / d - 1;
+          worst_4 = std::fmax(worst_4, (double)std::fmax(fabsl(ep), fabsl(ef)));
+        }
+      }
+  printf("%ld %ld %ld %.4f %.4f %.3e %.3f\n", used, close, wrong, worst_f, worst_p, bias / plain,
+         std::ldexp(worst_4, 57));
   return 0;
 }

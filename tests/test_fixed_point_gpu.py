@@ -162,3 +162,19 @@ def test_tile_after_a_refused_one(nb, masses, tracer, n):
         (a1, p1, s1), (a2, p2, s2) = (oracle.accel(pos, np.maximum(q, 0.0), eps) for q in (mass, -mass))
         ok, err, _ = fp64_accel_gate(acc, a1 - a2, s1 + s2, n)
         assert ok.all() and np.all(np.abs(pot - (p1 - p2)) <= 1e-12 * (np.abs(p1) + np.abs(p2)))
+
+
+# r^2 + eps^2 exactly a power of four, where 1/r is at the top of its range: lattices
+# whose (1,1,1) or (1,0,0) neighbours have it, particles at one place
+@pytest.mark.parametrize("kind,eps", [("lattice", 1.0), ("lattice", 1e-12), ("coincident", 0.25)])
+@pytest.mark.parametrize("sym", [0, 1])
+def test_distances_that_are_powers_of_two(nb, kind, eps, sym):
+    if kind == "lattice":
+        pos = np.stack(np.meshgrid(*[np.arange(12.0)] * 3), -1).reshape(-1, 3)
+    else:
+        pos = np.tile(np.random.default_rng(3).integers(-4, 5, (256, 3)) * 1.0, (4, 1))
+    mass = np.full(len(pos), 0.5)
+    with nb.Simulation(len(pos), "fp64", eps=eps) as sim:
+        sim.set_symmetric(sym)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, eps, acc, pot)
