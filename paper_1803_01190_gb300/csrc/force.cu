@@ -20,18 +20,18 @@
 //         rate, one FP64 instruction in the time of 32 integer ones, so the
 //         one-sided kernel sums softened pairs in 64-bit fixed point on the
 //         integer pipes (fixed.cuh), with less rounding than binary64 pair
-//         terms have.  Where that does not apply (eps = 0, masses of one tile
-//         over more than 2^6, close pairs in a wide tile) it takes the
-//         binary64 body, bound by the FP64 pipe with 9 FP64 instructions per
-//         pair (3 DADD for d, 3 DFMA for |d|^2 + eps^2, 3 DFMA for the
-//         acceleration sums); the rest of that body runs on the integer and
-//         FP32 pipes: 1/r and 1/r^2 within 0.52 ulp (SFU seed, exact integer
-//         residual), the products m/r and (m/r)/r^2 by a correctly rounded
-//         integer binary64 multiply, and the potential sum by a correctly
-//         rounded integer binary64 add.  At large N the FP64 path evaluates each
-//         pair once for both particles: softened ones in the same fixed point
-//         (k_force_fx_sym), eps = 0 in binary64 (k_force_f64_sym: 12 FP64
-//         instructions per pair, 6 per interaction).
+//         terms have.  Where that does not apply (eps = 0; masses of one tile
+//         over more than 2^8, negative or subnormal ones; single pairs too
+//         close for their tile's unit) it takes the binary64 body, bound by the
+//         FP64 pipe with 9 FP64 instructions per pair (3 DADD for d, 3 DFMA for
+//         |d|^2 + eps^2, 3 DFMA for the acceleration sums); the rest of that
+//         body runs on the integer and FP32 pipes: 1/r and 1/r^2 within 0.52 ulp
+//         (SFU seed, exact integer residual), the products m/r and (m/r)/r^2 by a
+//         correctly rounded integer binary64 multiply, and the potential sum by a
+//         correctly rounded integer binary64 add.  At large N the FP64 path
+//         evaluates each pair once for both particles: softened ones in the same
+//         fixed point (k_force_fx_sym), eps = 0 in binary64 (k_force_f64_sym: 12
+//         FP64 instructions per pair, 6 per interaction).
 //   mixed binary32 pair arithmetic (packed: two j per instruction, SFU
 //         reciprocal square root) on coordinates re-centred on an anchor (the
 //         per-coordinate median) per j-tile, with the i coordinates held as

@@ -6,9 +6,13 @@
 // where u is the unit of the coordinates (each rounded by at most u / 2, plus
 // the 16-bit products of the low words: below 2^-52 r at r = 2^51 u).  With an
 // exponent of its own a mass is as exact as the largest, down to the last place
-// of the sums (2^-57 of the largest mass's force at the tile's extent).
+// of the sums (2^-57 of the largest mass's force at the tile's extent, which is
+// what the mass rule bounds: see the sums around a heavy particle below).
 // Then pairs with r^2 exactly a power of four, where x = 1/4 and 1/r is at the
 // top of its range: prints the largest error of both terms in units of 2^-57.
+// Then the force on the heaviest particle of its tile, at the end of the mass
+// rule: 127 light ones on a sphere around it; prints the largest error in units
+// of 2^-53 of the sum of the terms' magnitudes.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -128,7 +132,42 @@ const ld ratio = equal ? 1 : (ld)mmax / m;
           worst_4 = std::fmax(worst_4, (double)std::fmax(fabsl(ep), fabsl(ef)));
         }
       }
-  printf("%ld %ld %ld %.4f %.4f %.3e %.3f\n", used, close, wrong, worst_f, worst_p, bias / plain,
-         std::ldexp(worst_4, 57));
+  double worst_heavy = 0;
+  std::normal_distribution<double> N;
+  for (int s = 0; s < 200; s++) {  // masses of 1 around one of 2^FX_MASS_RANGE, unit 2^(1 - FX_BITS)
+    const int L = 1 - FX_BITS;
+    const uint64_t Xi[3] = {0, 0, 0};
+    fx96 f[3] = {}, pot = {};
+    ld sum[3] = {0, 0, 0}, size = 0;
+    for (int k = 0; k < 127; k++) {
+      double x[3], n = 0;
+      uint64_t Xj[3];
+      for (double &c : x) c = N(g), n += c * c;
+      for (int c = 0; c < 3; c++) {
+        x[c] /= std::sqrt(n);
+        Xj[c] = fx_coord(hi(x[c]), lo(x[c]), L);
+      }
+      FxPair p;
+      fx_geometry<false>(Xj, Xi, fx_eps2(1e-4, L), [&](uint32_t v) {
+        const float y = (float)(1.0 / std::sqrt((double)(float)v));
+        uint32_t b;
+        memcpy(&b, &y, 4);
+        return b;
+      }, p);
+      fx_side<false, true>(p, fx_mass<true>(hi(1.0), 0, FX_MASS_RANGE), f, pot);
+      ld r2 = 1e-4L, d2 = 0;
+      for (double c : x) r2 += (ld)c * c, d2 += (ld)c * c;
+      for (int c = 0; c < 3; c++) sum[c] += x[c] / (r2 * sqrtl(r2));
+      size += sqrtl(d2) / (r2 * sqrtl(r2));
+    }
+    ld err = 0;
+    for (int c = 0; c < 3; c++) {
+      const ld v = value(f[c], fx_force_exp(L, FX_MASS_RANGE)) - sum[c];
+      err += v * v;
+    }
+    worst_heavy = std::fmax(worst_heavy, (double)(sqrtl(err) / size));
+  }
+  printf("%ld %ld %ld %.4f %.4f %.3e %.3f %.3f\n", used, close, wrong, worst_f, worst_p, bias / plain,
+         std::ldexp(worst_4, 57), std::ldexp(worst_heavy, 53));
   return 0;
 }

@@ -178,3 +178,24 @@ def test_distances_that_are_powers_of_two(nb, kind, eps, sym):
         sim.set_symmetric(sym)
         acc, pot = sim.accel(pos, mass)
     _check(pos, mass, eps, acc, pot)
+
+
+@pytest.mark.parametrize("bits", [9, 12, 20, 30, 40])
+@pytest.mark.parametrize("where", ["alone", "at a light one"])
+@pytest.mark.parametrize("sym", [0, 1])
+def test_heavy_particle(nb, bits, where, sym):
+    """The forces of the light particles alone: on the heavy one itself, and on a
+    light one at the heavy one's place, where its force vanishes."""
+    n = 1000
+    pos, mass, eps = _case("plain", n)
+    mass[:] = 2.0 ** -bits
+    mass[5] = 1.0
+    if where != "alone":
+        pos[700] = pos[5]
+    with nb.Simulation(n, "fp64", eps=eps) as sim:
+        sim.set_symmetric(sym)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, eps, acc, pot)
+    # no less exact than binary64 terms: 2^-53 of each, twice over, whatever their order
+    oa, _, smag = oracle.accel(pos, mass, eps)
+    assert np.linalg.norm(acc[5] - oa[5]) <= 2.0 ** -52 * smag[5]
