@@ -16,11 +16,16 @@
 //   Q  = y^2 2^61,  Y = m y,  F = Y y^2 (top 64 bits of the products with the
 //        63-bit mass; error of F < 2^-56),
 //   force sums += D F, potential sum += Y, aligned by h, in 96-bit integers,
-// converted to binary64 once per tile.  A pair closer than 2^51 u, where the
-// rounding of a coordinate (1/2 u) would exceed the rounding of a binary64
-// pair term, is left to the binary64 body by the caller; farther pairs carry a
-// smaller error than binary64 arithmetic gives them, and the sums are exact to
-// 2^-59 of a term.
+// converted to binary64 once per tile.  A pair with |d| below 2^51 u, where the
+// rounding of the coordinates (1/2 u each) and the last place of the sums
+// approach the rounding of a binary64 pair term, is left to the binary64 body by
+// the caller.  At that limit d is off by up to 2^-51 of itself and its term cut
+// off below 2^-52, both falling as 1/|d|; a binary64 difference may be off by
+// 2^-53 at any distance.  The limit is one of |d| and not of the softened r:
+// where eps is far above the separations, r says nothing of what the unit
+// leaves of them (two clumps 1e-6 eps across and 512 eps apart, the force in
+// the one at the origin, by host emulation: 1.1e-10 with a limit of r, 3e-16
+// with this one; a system of 1e-4 eps 1.1e-14 and 6e-16).
 //
 // What bounds it: the FMA-heavy pipe, where a 32 x 32 -> 64 multiply takes 4
 // cycles per warp (an addition on the ALU pipe takes 2).  So the products that
@@ -217,7 +222,7 @@ struct FxPair {
   int s, sp;             // right shifts of the force and potential terms
 };
 
-// false: the pair is closer than 2^51 units (EARLY: nothing else is set;
+// false: |d| is below 2^51 units (EARLY: nothing else is set;
 // otherwise 1/r and 1/r^2 are 0, so that its terms add nothing, and no branch
 // keeps the pairs of several calls from being interleaved).
 template <bool ALU, bool EARLY = true, class RSQRT>
@@ -240,7 +245,9 @@ FX_HD bool fx_geometry(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3], const F
   const int64_t Mid = S1 + (int64_t)(q >> 1);
   const uint64_t T = S2 + (uint64_t)(Mid >> 31);
   const uint32_t th = (uint32_t)(T >> 32), tl = (uint32_t)T, t0 = (uint32_t)Mid << 1;
-  const bool far = th >= 64u;
+  // |d| >= 2^51 units, from the upper words alone: the limit lies between
+  // sqrt(63/64) 2^51 and 2^51, by what eps^2 carries over from the word below
+  const bool far = th - (uint32_t)(e2.hi >> 32) >= 64u;
   if (EARLY && !far) return false;
 #ifdef __CUDA_ARCH__
   const int h = __clz(th) >> 1;

@@ -72,12 +72,14 @@ int main() {
       r2 += d[c] * d[c];
     }
     const ld r = sqrtl(r2), ur = ldexpl(1, L) / r;
+    // the limit: |d| between sqrt(63/64) 2^51 units and 2^51 units
+    const ld du = sqrtl(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) / ldexpl(1, L + 51);
     if (!ok) {
       close++;
-      if (ur < ldexpl(0.999L, -51)) wrong++;
+      if (du > 1.001L) wrong++;
       continue;
     }
-    if (ur > ldexpl(1.001L, -51)) wrong++;
+    if (du < 0.992L) wrong++;
     fx96 f[3] = {}, pot = {};
     if (equal)
       fx_both<false>(p, f, pot, nullptr, nullptr);

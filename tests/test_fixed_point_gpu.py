@@ -199,3 +199,19 @@ def test_heavy_particle(nb, bits, where, sym):
     # no less exact than binary64 terms: 2^-53 of each, twice over, whatever their order
     oa, _, smag = oracle.accel(pos, mass, eps)
     assert np.linalg.norm(acc[5] - oa[5]) <= 2.0 ** -52 * smag[5]
+
+
+# Separations far below the softening: of the whole system, or inside two clumps that
+# are far apart in units of it
+@pytest.mark.parametrize("size", [2.0 ** -7, 1e-3, 1e-4, 1e-6])
+@pytest.mark.parametrize("apart", [0.0, 32.0, 512.0, 1000.0])
+@pytest.mark.parametrize("sym", [0, 1])
+def test_separations_below_the_softening(nb, size, apart, sym):
+    n = 700
+    pos = size * np.random.default_rng(4).standard_normal((n, 3))
+    pos[1::2, 0] += apart
+    mass = np.full(n, 1.0 / n)
+    with nb.Simulation(n, "fp64", eps=1.0) as sim:
+        sim.set_symmetric(sym)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, 1.0, acc, pot)
