@@ -435,6 +435,29 @@ __device__ __forceinline__ void fx_coords(const d4 &p, int L, uint64_t (&X)[3]) 
   X[1] = fx_coord((uint32_t)__double2hiint(p.y), (uint32_t)__double2loint(p.y), L);
   X[2] = fx_coord((uint32_t)__double2hiint(p.z), (uint32_t)__double2loint(p.z), L);
 }
+// Too many of a tile's pairs too close for its unit?  One far particle makes all pairs
+// within 2^-10 of the distance to it such pairs; each costs its fixed-point geometry
+// and then a call for all lanes of the warp, so that from a small share of them on the
+// binary64 body is the cheaper one for the whole tile.  The share is estimated from
+// one pair a thread: its first i-particle against the tile entry 16 lanes off (never
+// itself: blocks and tiles start at multiples of 32), differences taken from the
+// upper words; FX_NEAR of a block's 128 such pairs send the tile to binary64.
+// Measured (Gint/s, N = 65536, Plummer sphere of unit core, every 128th particle put
+// at 200, 400, 1000; one-sided): never 107, 78, 56; at 1 89, 71, 71; 2 100, 72, 71; 4 106,
+// 76, 71; 8 105, 84, 71; 16 104, 85, 71; each pair once (never: with every pair of a tile
+// out of line) 99, 50, 41; 1 105, 93, 93; 4 115, 93, 93; 8 118, 91, 93; 16 118, 90, 93.
+// The estimate costs a sphere without far particles 2 % one-sided (132.1 -> 129.4;
+// registers, not the work) and nothing each pair once.
+constexpr int FX_NEAR = 8;
+__device__ __forceinline__ bool fx_near(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3]) {
+  bool near = true;
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    const unsigned j = __shfl_xor_sync(0xFFFFFFFFu, (unsigned)(Xj[c] >> 32), 16);
+    near &= j - (unsigned)(Xi[c] >> 32) + 0x80000u < 0x100000u;
+  }
+  return near;
+}
 struct FxRsqrt {
   __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
     return __float_as_uint(rsqrt_approx(__uint2float_rn(x)));
@@ -518,8 +541,9 @@ __device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, cons
 // IW warps of a block share the same i-particles and split each j-tile (IW =
 // 1: BT * R i-particles per block; IW = 4, for small n: BT / 4 * R, four times
 // as many blocks and a quarter of the sequential pairs per thread).  Each tile
-// is summed in fixed point where fx_scale allows it and in binary64 otherwise;
-// pairs too close for the tile's unit go through pair_f64.  i-particles are
+// is summed in fixed point where fx_scale allows it and few of its pairs are
+// too close for its unit (FX_NEAR), and in binary64 otherwise; single pairs too
+// close for the unit go through pair_f64.  i-particles are
 // taken two at a time (RI), whatever R is.
 template <int BT, int R, int T, int IW, class W>
 __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W work,
@@ -573,20 +597,32 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
       const FxScale sc = fx_scale(bi, bj, eps2);
       const int k0 = cnt * jw / IW, k1 = cnt * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      if (sc.ok) {
-        {
-          uint64_t X[3];
-          fx_coords(pj, sc.L, X);
-          const uint32_t mh = (uint32_t)__double2hiint(pj.w), ml = (uint32_t)__double2loint(pj.w);
-          const FxMass M = sc.wide ? fx_mass<true>(mh, ml, sc.em) : fx_mass<false>(mh, ml, sc.em);
-          txy[tid] = make_uint4((uint32_t)X[0], (uint32_t)(X[0] >> 32), (uint32_t)X[1],
-                                (uint32_t)(X[1] >> 32));
-          tzm[tid] = make_uint4((uint32_t)X[2], (uint32_t)(X[2] >> 32), M.l, M.h);
-          tdm[tid] = M.dm;
+      bool fixed = sc.ok, equal = false;
+      const double m0 = tile[0].w;
+      uint64_t Xi[RI][3];
+      auto load_i = [&](int g) {
+#pragma unroll
+        for (int r = 0; r < RI; r++) {
+          const int li = (g * RI + r) * IT + it;
+          fx_coords(posm[u.i0 + (li < u.ni ? li : 0)], sc.L, Xi[r]);
         }
-        const double m0 = tile[0].w;
-        const bool equal = __syncthreads_and(
-            __double_as_longlong(pj.w) == __double_as_longlong(m0) || tid >= cnt);
+      };
+      if (sc.ok) {
+        uint64_t X[3];
+        fx_coords(pj, sc.L, X);
+        load_i(0);
+        const bool near = fx_near(X, Xi[0]) && (tid ^ 16) < cnt;
+        const uint32_t mh = (uint32_t)__double2hiint(pj.w), ml = (uint32_t)__double2loint(pj.w);
+        const FxMass M = sc.wide ? fx_mass<true>(mh, ml, sc.em) : fx_mass<false>(mh, ml, sc.em);
+        txy[tid] = make_uint4((uint32_t)X[0], (uint32_t)(X[0] >> 32), (uint32_t)X[1],
+                              (uint32_t)(X[1] >> 32));
+        tzm[tid] = make_uint4((uint32_t)X[2], (uint32_t)(X[2] >> 32), M.l, M.h);
+        tdm[tid] = M.dm;
+        equal = __syncthreads_and(__double_as_longlong(pj.w) == __double_as_longlong(m0) ||
+                                  tid >= cnt);
+        fixed = __syncthreads_count(near) < FX_NEAR;
+      }
+      if (fixed) {
         // FX_SELF in the split shape alone, where such tiles are a large share
         // (N = 4096: 139 us against 147); elsewhere one more form of the loop
         // made the others slower (N = 20011: 3.54 ms against 3.35)
@@ -602,13 +638,8 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
           ps *= m0;
         }
         for (int g = 0; g < NG; g++) {
-          uint64_t Xi[RI][3];
           fx96 f[RI][3] = {}, pt[RI] = {};
-#pragma unroll
-          for (int r = 0; r < RI; r++) {
-            const int li = (g * RI + r) * IT + it;
-            fx_coords(posm[u.i0 + (li < u.ni ? li : 0)], sc.L, Xi[r]);
-          }
+          if (g > 0) load_i(g);
           const int ii = (int)(u.i0 - jt) + g * RI * IT + it;  // tile entry of particle 0
           auto self = [&](int r, int k) { return diag && k == ii + r * IT; };
           auto close = [&](int r, int k) {
@@ -798,6 +829,50 @@ __device__ __forceinline__ d4 pad_or_load(const d4 *posm, int64_t k, int64_t n) 
   return k < n ? posm[k] : d4{1e30, 1e30, 1e30, 0.0};
 }
 
+// One column tile (the first cnt entries, in chunks of 32) against R i-particles of
+// each thread: row sums into acc, the warp's column sums into colw (ADD: onto it).
+template <int R, int T, bool ADD>
+__device__ __forceinline__ void f64_sym_tile(const d4 *tile, int cnt, const d4 (&p)[R],
+                                             const MassSig (&ms)[R], double eps2, d4 (&acc)[R],
+                                             d4 *colw) {
+  const int lane = threadIdx.x & 31;
+  uint64_t pt[R];
+#pragma unroll
+  for (int r = 0; r < R; r++) pt[r] = (uint64_t)__double_as_longlong(acc[r].w);
+#pragma unroll 1
+  for (int c = 0; c < T; c += 32) {
+    if (c >= cnt) break;
+    double gx = 0.0, gy = 0.0, gz = 0.0;
+    uint64_t gp = 0;  // bit pattern of the column potential sum, as pt
+    // not unrolled: measured on GB300 at N = 2^18, unroll 2 ran 4 % slower
+#pragma unroll 1
+    for (int k = 0; k < 32; k++) {
+      const d4 pj = tile[c + ((lane + k) & 31)];
+      const MassSig mj = mass_sig(pj.w);
+#pragma unroll
+      for (int r = 0; r < R; r++)
+        body_f64_sym(pj, mj, p[r].x, p[r].y, p[r].z, p[r].w, ms[r], eps2, acc[r].x, acc[r].y,
+                     acc[r].z, pt[r], gx, gy, gz, gp);
+      const int src = (lane + 1) & 31;
+      gx = __shfl_sync(0xFFFFFFFFu, gx, src);
+      gy = __shfl_sync(0xFFFFFFFFu, gy, src);
+      gz = __shfl_sync(0xFFFFFFFFu, gz, src);
+      gp = __shfl_sync(0xFFFFFFFFu, gp, src);
+    }
+    d4 g = d4{gx, gy, gz, __longlong_as_double((long long)gp)};
+    if (ADD) {
+      const d4 s = colw[c + lane];
+      g.x += s.x;
+      g.y += s.y;
+      g.z += s.z;
+      g.w += s.w;
+    }
+    colw[c + lane] = g;
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++) acc[r].w = __longlong_as_double((long long)pt[r]);
+}
+
 template <int BT, int R, int T>
 __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ posm, int64_t n,
                                                       double eps2, int M, int d0,
@@ -807,7 +882,7 @@ __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ pos
   static_assert(T == BT && B % T == 0, "one column sum per thread per tile");
   __shared__ d4 tile[T];
   __shared__ d4 colw[NW][T];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5;
   const int dl = blockIdx.x / M, I = blockIdx.x % M, d = d0 + dl;
   const int J = (I + d) % M;
   const int64_t i0 = (int64_t)I * B, j0 = (int64_t)J * B;
@@ -820,46 +895,20 @@ __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ pos
     }
     return;
   }
-  double xi[R], yi[R], zi[R], mi[R], ax[R], ay[R], az[R];
-  uint64_t pt[R];  // bit patterns of the row potential sums
-  MassSig msi[R];
+  d4 p[R], acc[R];
+  MassSig ms[R];
 #pragma unroll
   for (int r = 0; r < R; r++) {
-    const d4 p = pad_or_load(posm, i0 + r * BT + tid, n);
-    xi[r] = p.x;
-    yi[r] = p.y;
-    zi[r] = p.z;
-    mi[r] = p.w;
-    msi[r] = mass_sig(p.w);
-    ax[r] = ay[r] = az[r] = 0.0;
-    pt[r] = 0;
+    p[r] = pad_or_load(posm, i0 + r * BT + tid, n);
+    ms[r] = mass_sig(p[r].w);
+    acc[r] = d4{0.0, 0.0, 0.0, 0.0};
   }
   for (int t0 = 0; t0 < B; t0 += T) {
     const int64_t jt = j0 + t0;
     __syncthreads();
     for (int k = tid; k < T; k += BT) tile[k] = pad_or_load(posm, jt + k, n);
     __syncthreads();
-#pragma unroll 1
-    for (int c = 0; c < T; c += 32) {
-      double gx = 0.0, gy = 0.0, gz = 0.0;
-      uint64_t gp = 0;  // bit pattern of the column potential sum
-      // not unrolled: measured on GB300 at N = 2^18, unroll 2 ran 4 % slower
-#pragma unroll 1
-      for (int k = 0; k < 32; k++) {
-        const d4 pj = tile[c + ((lane + k) & 31)];
-        const MassSig mj = mass_sig(pj.w);
-#pragma unroll
-        for (int r = 0; r < R; r++)
-          body_f64_sym(pj, mj, xi[r], yi[r], zi[r], mi[r], msi[r], eps2, ax[r], ay[r], az[r],
-                       pt[r], gx, gy, gz, gp);
-        const int src = (lane + 1) & 31;
-        gx = __shfl_sync(0xFFFFFFFFu, gx, src);
-        gy = __shfl_sync(0xFFFFFFFFu, gy, src);
-        gz = __shfl_sync(0xFFFFFFFFu, gz, src);
-        gp = __shfl_sync(0xFFFFFFFFu, gp, src);
-      }
-      colw[warp][c + lane] = d4{gx, gy, gz, __longlong_as_double((long long)gp)};
-    }
+    f64_sym_tile<R, T, false>(tile, T, p, ms, eps2, acc, colw[warp]);
     __syncthreads();
     {
       d4 s = colw[0][tid];
@@ -877,8 +926,23 @@ __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ pos
 #pragma unroll
   for (int r = 0; r < R; r++) {
     const int64_t i = i0 + r * BT + tid;
-    if (i < n) rowo[i] = d4{ax[r], ay[r], az[r], __longlong_as_double((long long)pt[r])};
+    if (i < n) rowo[i] = acc[r];
   }
+}
+
+// One pair out of line: what it adds to i's sums and to j's.
+struct F64Both {
+  d4 i, j;
+};
+__device__ __noinline__ F64Both pair_f64_both(double dx, double dy, double dz, double mj,
+                                              double mi, double eps2) {
+  F64Both v = {};
+  uint64_t pi = 0, pj = 0;
+  body_f64_sym(d4{dx, dy, dz, mj}, mass_sig(mj), 0.0, 0.0, 0.0, mi, mass_sig(mi), eps2, v.i.x,
+               v.i.y, v.i.z, pi, v.j.x, v.j.y, v.j.z, pj);
+  v.i.w = __longlong_as_double((long long)pi);
+  v.j.w = __longlong_as_double((long long)pj);
+  return v;
 }
 
 // ---------------------------------------------------------------- fixed point, each pair once
@@ -886,10 +950,11 @@ __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ pos
 // arithmetic of fixed.cuh: the geometry of a pair (d, 1/r, 1/r^2: 20 of the 38
 // wide multiplies of one side) serves both particles.  Sums of a tile are
 // 96-bit integers in registers; the column sums of a chunk of 32 j travel
-// around the lanes (12 words per step).  Pairs too close for the unit, and
-// every pair of an item that fx_scale does not take, are evaluated in
-// binary64 out of line and added in binary64 (rows in registers, columns in
-// the warp's slots of colw, where a lane owns its j at each step).  Measured
+// around the lanes (12 words per step).  Single pairs too close for the unit
+// are evaluated in binary64 out of line and added in binary64 (rows in
+// registers, columns in the warp's slots of colw, where a lane owns its j at
+// each step); tiles that fx_scale does not take, or with many such pairs
+// (FX_NEAR), go through the tile loop of k_force_f64_sym.  Measured
 // (whole force evaluation, N = 65536): 215-219 Gint/s for equal masses, where
 // the two sides share their terms, 147 for lognormal masses, against 93 for
 // k_force_f64_sym; relative error of the accelerations 1.6e-16 against 2.6e-16.
@@ -897,7 +962,7 @@ __global__ void __launch_bounds__(BT) k_force_f64_sym(const d4 *__restrict__ pos
 // three blocks, 214 at R = 1, 175 at R = 3.
 template <int BT, int R, int T, FxMode MODE>
 __device__ __forceinline__ void fx_sym_tile(const d4 *__restrict__ posm, int64_t n, int64_t i0,
-                                            double eps2, bool ok, const FxEps &e2,
+                                            double eps2, const FxEps &e2,
                                             const d4 *tile, const uint4 *txy, const uint4 *tzm,
                                             const int *tdm, int cnt, const uint64_t (&Xi)[R][3],
                                             const FxMass (&Mi)[R], d4 (&acc)[R], double fs,
@@ -918,7 +983,7 @@ __device__ __forceinline__ void fx_sym_tile(const d4 *__restrict__ posm, int64_t
 #pragma unroll
       for (int r = 0; r < R; r++) {
         FxPair p;
-        if (ok && fx_geometry<true>(Xj, Xi[r], e2, FxRsqrt(), p)) {
+        if (fx_geometry<true>(Xj, Xi[r], e2, FxRsqrt(), p)) {
           if (MODE == FX_EQUAL) {
             fx_both<true>(p, f[r], pt[r], &g, &gp);
           } else {
@@ -929,17 +994,16 @@ __device__ __forceinline__ void fx_sym_tile(const d4 *__restrict__ posm, int64_t
           const int64_t i = i0 + r * BT + tid;
           if (jj < cnt && i < n) {
             const d4 pi = posm[i], q = tile[jj];
-            const double dx = q.x - pi.x, dy = q.y - pi.y, dz = q.z - pi.z;
-            const d4 v = pair_f64(dx, dy, dz, q.w, eps2);
-            acc[r].x += v.x;
-            acc[r].y += v.y;
-            acc[r].z += v.z;
-            acc[r].w += v.w;
-            const d4 w = pair_f64(-dx, -dy, -dz, pi.w, eps2);
-            colw[jj].x += w.x;
-            colw[jj].y += w.y;
-            colw[jj].z += w.z;
-            colw[jj].w += w.w;
+            const F64Both v =
+                pair_f64_both(q.x - pi.x, q.y - pi.y, q.z - pi.z, q.w, pi.w, eps2);
+            acc[r].x += v.i.x;
+            acc[r].y += v.i.y;
+            acc[r].z += v.i.z;
+            acc[r].w += v.i.w;
+            colw[jj].x += v.j.x;
+            colw[jj].y += v.j.y;
+            colw[jj].z += v.j.z;
+            colw[jj].w += v.j.w;
           }
         }
       }
@@ -980,7 +1044,7 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
   static_assert(T == BT && B % T == 0, "one column sum per thread per tile");
   __shared__ d4 tile[T];
   __shared__ uint4 txy[T], tzm[T];
-  __shared__ int tdm[T];
+  __shared__ int tdm[T], snear[NW];
   __shared__ d4 colw[NW][T];
   __shared__ FxBox sbox[NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1029,18 +1093,22 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
     FxBox bj;
     fx_box_init(bj);
     fx_box_add(bj, pj);
-    tile[tid] = pj;
     if (tid >= cnt) pj.w = 0.0;
+    tile[tid] = pj;
     fx_box_warp(bj);
     if (lane == 0) sbox[warp] = bj;
+#pragma unroll
+    for (int w = 0; w < NW; w++) colw[w][tid] = d4{0.0, 0.0, 0.0, 0.0};
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < NW; w++) fx_box_join(bj, sbox[w]);
-    FxScale sc = fx_scale(bi, bj, eps2);
-    const bool ok = sc.ok && oki, wide = sc.wide || widei;
-    const int emc = ok ? emi : 0;     // of the row block's masses, in this tile
-    if (!ok) sc.L = sc.em = 0;        // the integer sums stay zero
-    {
+    const FxScale sc = fx_scale(bi, bj, eps2);
+    const bool wide = sc.wide || widei;
+    const double mj0 = tile[0].w;
+    bool fixed = sc.ok && oki, equal = false;
+    uint64_t Xi[R][3];
+    FxMass Mi[R];
+    if (fixed) {
       uint64_t X[3];
       fx_coords(pj, sc.L, X);
       const uint32_t mh = (uint32_t)__double2hiint(pj.w), ml = (uint32_t)__double2loint(pj.w);
@@ -1049,43 +1117,56 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
                             (uint32_t)(X[1] >> 32));
       tzm[tid] = make_uint4((uint32_t)X[2], (uint32_t)(X[2] >> 32), m.l, m.h);
       tdm[tid] = m.dm;
-    }
 #pragma unroll
-    for (int w = 0; w < NW; w++) colw[w][tid] = d4{0.0, 0.0, 0.0, 0.0};
-    const double mj0 = tile[0].w;
-    const bool equal = __syncthreads_and(
-        equali && tid < cnt && __double_as_longlong(pj.w) == __double_as_longlong(mj0));
-    const FxMode mode = wide || !ok ? FX_WIDE : equal ? FX_EQUAL : FX_NARROW;
-    const FxEps e2 = fx_eps2(eps2, sc.L);
-    const int er = mode == FX_EQUAL ? FX_EQ_EM : sc.em, ec = mode == FX_EQUAL ? FX_EQ_EM : emc;
-    double fs = fx_exp2(fx_force_exp(sc.L, er) + 32), ps = fx_exp2(fx_pot_exp(sc.L, er) + 32);
-    double gs = fx_exp2(fx_force_exp(sc.L, ec) + 32), qs = fx_exp2(fx_pot_exp(sc.L, ec) + 32);
-    if (mode == FX_EQUAL) {
-      fs *= mj0;
-      ps *= mj0;
-      gs *= mi0;
-      qs *= mi0;
-    }
-    uint64_t Xi[R][3];
-    FxMass Mi[R];
+      for (int r = 0; r < R; r++) {
+        const int64_t i = i0 + r * BT + tid;
+        const d4 p = posm[i < n ? i : i0];
+        fx_coords(p, sc.L, Xi[r]);
+        const double mi = i < n ? p.w : 0.0;
+        const uint32_t ih = (uint32_t)__double2hiint(mi), il = (uint32_t)__double2loint(mi);
+        Mi[r] = wide ? fx_mass<true>(ih, il, emi) : fx_mass<false>(ih, il, emi);
+      }
+      const unsigned near = __ballot_sync(0xFFFFFFFFu, fx_near(X, Xi[0]) && (tid ^ 16) < cnt);
+      if (lane == 0) snear[warp] = __popc(near);
+      equal = __syncthreads_and(equali && tid < cnt &&
+                                __double_as_longlong(pj.w) == __double_as_longlong(mj0));
+      int n_near = 0;
 #pragma unroll
-    for (int r = 0; r < R; r++) {
-      const int64_t i = i0 + r * BT + tid;
-      const d4 p = posm[i < n ? i : i0];
-      fx_coords(p, sc.L, Xi[r]);
-      const double m = i < n ? p.w : 0.0;
-      const uint32_t mh = (uint32_t)__double2hiint(m), ml = (uint32_t)__double2loint(m);
-      Mi[r] = wide ? fx_mass<true>(mh, ml, emc) : fx_mass<false>(mh, ml, emc);
+      for (int w = 0; w < NW; w++) n_near += snear[w];
+      fixed = n_near < FX_NEAR;
     }
-    if (mode == FX_WIDE)
-      fx_sym_tile<BT, R, T, FX_WIDE>(posm, n, i0, eps2, ok, e2, tile, txy, tzm, tdm, cnt, Xi, Mi,
-                                     acc, fs, ps, gs, qs, colw[warp]);
-    else if (mode == FX_EQUAL)
-      fx_sym_tile<BT, R, T, FX_EQUAL>(posm, n, i0, eps2, true, e2, tile, txy, tzm, tdm, cnt, Xi,
-                                      Mi, acc, fs, ps, gs, qs, colw[warp]);
-    else
-      fx_sym_tile<BT, R, T, FX_NARROW>(posm, n, i0, eps2, true, e2, tile, txy, tzm, tdm, cnt, Xi,
-                                       Mi, acc, fs, ps, gs, qs, colw[warp]);
+    if (fixed) {
+      const FxMode mode = wide ? FX_WIDE : equal ? FX_EQUAL : FX_NARROW;
+      const FxEps e2 = fx_eps2(eps2, sc.L);
+      const int er = mode == FX_EQUAL ? FX_EQ_EM : sc.em, ec = mode == FX_EQUAL ? FX_EQ_EM : emi;
+      double fs = fx_exp2(fx_force_exp(sc.L, er) + 32), ps = fx_exp2(fx_pot_exp(sc.L, er) + 32);
+      double gs = fx_exp2(fx_force_exp(sc.L, ec) + 32), qs = fx_exp2(fx_pot_exp(sc.L, ec) + 32);
+      if (mode == FX_EQUAL) {
+        fs *= mj0;
+        ps *= mj0;
+        gs *= mi0;
+        qs *= mi0;
+      }
+      if (mode == FX_WIDE)
+        fx_sym_tile<BT, R, T, FX_WIDE>(posm, n, i0, eps2, e2, tile, txy, tzm, tdm, cnt, Xi, Mi, acc,
+                                       fs, ps, gs, qs, colw[warp]);
+      else if (mode == FX_EQUAL)
+        fx_sym_tile<BT, R, T, FX_EQUAL>(posm, n, i0, eps2, e2, tile, txy, tzm, tdm, cnt, Xi, Mi, acc,
+                                        fs, ps, gs, qs, colw[warp]);
+      else
+        fx_sym_tile<BT, R, T, FX_NARROW>(posm, n, i0, eps2, e2, tile, txy, tzm, tdm, cnt, Xi, Mi,
+                                         acc, fs, ps, gs, qs, colw[warp]);
+    } else {  // one i-particle at a time: 92 Gint/s against 85 for both at once (N = 65536)
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const int64_t i = i0 + r * BT + tid;
+        d4 p[1] = {posm[i < n ? i : i0]}, a[1] = {acc[r]};
+        if (i >= n) p[0].w = 0.0;
+        const MassSig ms[1] = {mass_sig(p[0].w)};
+        f64_sym_tile<1, T, true>(tile, cnt, p, ms, eps2, a, colw[warp]);
+        acc[r] = a[0];
+      }
+    }
     __syncthreads();
     {
       d4 s = colw[0][tid];

@@ -215,3 +215,22 @@ def test_separations_below_the_softening(nb, size, apart, sym):
         sim.set_symmetric(sym)
         acc, pot = sim.accel(pos, mass)
     _check(pos, mass, 1.0, acc, pot)
+
+
+# Far particles in every tile, so that most, some or few of the other pairs are too close for
+# the tiles' units (within 2^-10 of the extent)
+@pytest.mark.parametrize("extent", [30.0, 300.0, 1e3, 1e4, 1e8])
+@pytest.mark.parametrize("equal", [True, False])
+@pytest.mark.parametrize("n,sym", [(129, 0), (1000, 0), (9001, 0), (257, 1), (1000, 1), (2305, 1)])
+def test_far_particles(nb, extent, equal, n, sym):
+    pos, mass, eps = _case("plain", n)
+    rng = np.random.default_rng(n)
+    v = rng.standard_normal((len(pos[7::50]), 3))
+    pos[7::50] = extent * v / np.linalg.norm(v, axis=1)[:, None]
+    if not equal:
+        mass = mass * rng.uniform(0.5, 1.0, n)
+        mass[n // 3] *= 2.0 ** -30  # one tile outside the mass rule as well
+    with nb.Simulation(n, "fp64", eps=eps) as sim:
+        sim.set_symmetric(sym)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, eps, acc, pot)
