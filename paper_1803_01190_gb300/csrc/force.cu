@@ -2051,8 +2051,12 @@ __global__ void __launch_bounds__(BT) k_mixed_prep(const d4 *__restrict__ posm, 
 // units of it, which changes no bit of them.  Other masses keep the product in
 // the body: sums in another rounding would move single precision positions, and
 // with them close pairs at a small softening, by as much as its whole error.
-// The range of masses and the softening keep 1/r^3 and the sums in units of the
-// mass finite (1/r <= 2^20) and not smaller than with it (m <= 1).
+// The range of masses and the softening keep the terms in units of the mass
+// finite (1/r <= 2^20) and not smaller than with it (m <= 1).  The sums so far,
+// which tiles of other masses may have made large, are taken into those units
+// only where that leaves every one of the warp's below 2^100; a tile's own terms
+// add less than 2^50.  Otherwise the tile keeps its mass in the body, which gives
+// the same bits.
 __device__ __forceinline__ bool f32_unit_mass(float m, float eps2) {
   return (__float_as_uint(m) & 0x807FFFFFu) == 0 && m <= 1.0f && m >= 0x1p-40f && eps2 >= 0x1p-40f;
 }
@@ -2067,7 +2071,18 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
     const int64_t j1 = u.j0 + u.nj;
     const float2 e2 = f2((float)u.eps2, (float)u.eps2);
     float2 nx[R], ny[R], nz[R], ax[R], ay[R], az[R], pt[R];
-    float unit = 1.0f;  // of the sums
+    float unit = 1.0f;  // of the sums, the same for a warp
+    auto fit_units_of = [&](float m) {
+      if (m >= unit) return true;
+      float top = 0.0f;
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const float2 v[4] = {ax[r], ay[r], az[r], pt[r]};
+#pragma unroll
+        for (int c = 0; c < 4; c++) top = fmaxf(top, fmaxf(fabsf(v[c].x), fabsf(v[c].y)));
+      }
+      return __all_sync(0xFFFFFFFFu, top * (unit / m) < 0x1p100f) != 0;
+    };
     auto in_units_of = [&](float m) {
       if (m == unit) return;
       const float f = unit / m;  // of powers of two: exact
@@ -2099,7 +2114,7 @@ __global__ void __launch_bounds__(BT) k_force_f32(const float4 *__restrict__ pos
                          f32_unit_mass(m, e2.x);
       const int np = (cnt + 1) / 2;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
-      if (cnt == T && !diag && equal) {
+      if (cnt == T && !diag && equal && fit_units_of(m)) {
         in_units_of(m);
 #pragma unroll 2
         for (int k = 0; k < T / 2; k++) {

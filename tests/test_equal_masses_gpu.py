@@ -64,3 +64,15 @@ def test_fp32_units_do_not_change_the_sums(nb, n):
         a, p = sim.accel(pos, mass)
         b, q = sim.accel(pos, mass * 2.0 ** 13)
     assert (a * 2.0 ** 13 == b).all() and (p * 2.0 ** 13 == q).all()
+
+
+@pytest.mark.parametrize("heavy", [1.0, 1e20, 1e32])
+@pytest.mark.parametrize("n", [1024, 20000])
+def test_fp32_heavy_particle_before_light_tiles(nb, heavy, n):
+    """Sums that a heavy particle has made large stay finite in units of a small mass."""
+    rng = np.random.default_rng(n)
+    pos = rng.standard_normal((n, 3))
+    mass = np.full(n, 2.0 ** -40)
+    mass[3] = heavy
+    ea, ep = _errors(nb, "fp32", pos, mass, 0.05)
+    assert ea <= TOL["fp32"] and ep <= TOL["fp32"]
