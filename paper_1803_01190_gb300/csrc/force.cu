@@ -1356,10 +1356,14 @@ __device__ __forceinline__ void split_ff(double x, float &h, float &l) {
     l = __double2float_rn(x - (double)h);
   }
 }
-// h + l in binary64 (non-finite halves by conversion, which keeps them so)
+// h + l in binary64 (non-finite and subnormal halves by conversion, which keeps
+// them; a half of zero is exact either way)
+__device__ __forceinline__ bool is_normal_or_0(float x) {
+  return (__float_as_uint(x) & 0x7FFFFFFFu) - 0x00800000u < 0x7F000000u || x == 0.0f;
+}
 __device__ __forceinline__ double join_ff(float h, float l) {
-  const bool finite = fabsf(h) < INFINITY && fabsf(l) < INFINITY;
-  return finite ? f2d_exact(h) + f2d_exact(l) : (double)h + (double)l;
+  return is_normal_or_0(h) && is_normal_or_0(l) ? f2d_exact(h) + f2d_exact(l)
+                                                : (double)h + (double)l;
 }
 
 // -(x - c) of an i-particle against a tile's anchor c, exact but for the split:

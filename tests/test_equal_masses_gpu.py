@@ -76,3 +76,20 @@ def test_fp32_heavy_particle_before_light_tiles(nb, heavy, n):
     mass[3] = heavy
     ea, ep = _errors(nb, "fp32", pos, mass, 0.05)
     assert ea <= TOL["fp32"] and ep <= TOL["fp32"]
+
+
+@pytest.mark.parametrize("n", [300, 1200])
+@pytest.mark.parametrize("equal", [True, False])
+def test_mixed_subnormal_forces(nb, n, equal):
+    """Sums below binary32's normal numbers keep what its subnormal ones hold: m y, m y^3
+    and d m y^3 of a term and its additions are each off by up to 2^-150, with y <= 2 and
+    d y^2 <= 1."""
+    rng = np.random.default_rng(n)
+    pos = rng.standard_normal((n, 3))
+    mass = 2.0 ** -136 * (np.ones(n) if equal else rng.integers(1, 3, n))
+    with nb.Simulation(n, "mixed", eps=0.5) as sim:
+        acc, pot = sim.accel(pos, mass)
+    oa, op, _ = oracle.accel(pos, mass, 0.5)
+    assert 1e-40 < np.abs(oa).max() < 2.0 ** -126
+    assert (np.abs(acc - oa) <= 4 * n * 2.0 ** -150 + 1e-5 * np.abs(oa).max()).all()
+    assert (np.abs(pot - op) <= 4 * n * 2.0 ** -150 + 1e-5 * np.abs(op)).all()
