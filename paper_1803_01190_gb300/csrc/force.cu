@@ -42,7 +42,7 @@
 //   f64e  binary64-class accuracy on the binary32 pipes: float-float (about 48
 //         significant bits) pair arithmetic on coordinates re-centred per
 //         j-tile, float-float tile partials folded into binary64 per tile.
-//         About 134 to 146 binary32 operations per pair (84 to 96 per
+//         About 136 to 148 binary32 operations per pair (86 to 98 per
 //         interaction when each pair is evaluated once), but on pipes 64 times
 //         faster than GB300's FP64 pipe.  From 64 blocks of 256 particles it
 //         evaluates each pair once for both particles (k_force_f64e_sym).
@@ -1464,28 +1464,32 @@ __device__ __forceinline__ void ff_terms(const FfPair &g, float2 mh, float2 ml, 
   t.l[3] = al;
 }
 
-// (h, l) += t: the high parts by TwoSum, the rest into the low part.  The sums
-// are renormalised (ff_renorm) every few terms, not after each, which saves 3
-// of 11 operations a term: the low part then grows to a few ulps of the high
-// one.  Every 4 terms for the accelerations, whose error is that of the
-// coordinates; every 2 for the potentials, whose error is that of the sum.
-// Measured each pair once, N = 65536, equal masses (Gint/s, relative error of
-// the potentials): every term 375, 7.0e-16; all every 2: 400, 7.1e-16; all every
-// 4: 411, 7.4e-16; every 8: 410, 8.0e-16; 303, 6.9e-16 before this and the shared
-// terms; unequal masses 355 every 4.
+// (h, l) += t: the high parts by TwoSum, the rest into the low part.  The
+// potentials, whose error is that of the sum, are renormalised with every term;
+// the accelerations, whose error is that of the coordinates, every FF_STEPS steps
+// (ff_renorm), which saves 3 of 11 operations a term: their low part grows to a few
+// ulps of the high one.  Measured each pair once (48 systems of 1500 to 65539
+// particles; largest RMS error over that with every sum renormalised with every
+// term): accelerations 1.08, potentials 1.00; potentials every second step 1.08, for
+// an FR4 step of 65539 in 32.3 ms against 32.9.  Every sum with every term takes 9 %
+// longer than every fourth step.
 __device__ __forceinline__ void ff_add(const FfTerms &t, float2 (&h)[4], float2 (&l)[4]) {
 #pragma unroll
   for (int c = 0; c < 4; c++) {
     float2 s, es;
     two_sum2(h[c], t.h[c], s, es);
-    h[c] = s;
-    l[c] = __fadd2_rn(l[c], __fadd2_rn(es, t.l[c]));
+    const float2 lo = __fadd2_rn(l[c], __fadd2_rn(es, t.l[c]));
+    if (c < 3) {
+      h[c] = s;
+      l[c] = lo;
+    } else {
+      fast_two_sum2(s, lo, h[c], l[c]);
+    }
   }
 }
-template <int C0 = 0>
 __device__ __forceinline__ void ff_renorm(float2 (&h)[4], float2 (&l)[4]) {
 #pragma unroll
-  for (int c = C0; c < 4; c++) {
+  for (int c = 0; c < 3; c++) {
     float2 s, e;
     fast_two_sum2(h[c], l[c], s, e);
     h[c] = s;
@@ -1511,7 +1515,7 @@ __device__ __forceinline__ void load_pairs_ff(const float4 *__restrict__ src, in
   }
 }
 
-// Terms between renormalisations of the acceleration sums.
+// Steps between renormalisations of the acceleration sums.
 constexpr int FF_STEPS = 4;
 
 template <int R, bool EQUAL>
@@ -1532,10 +1536,7 @@ __device__ __forceinline__ void ff_tile(const float4 *tH, const float4 *tH2, con
         ff_geometry<false>(H, H2, L, L2, nh[r], nl[r], e2h, e2l, false, false, g);
         ff_terms<EQUAL>(g, f2(H2.z, H2.w), f2(L2.z, L2.w), t);
         ff_add(t, ah[r], al[r]);
-        if (q == FF_STEPS - 1)
-          ff_renorm(ah[r], al[r]);
-        else if (q % 2 == 1)
-          ff_renorm<3>(ah[r], al[r]);
+        if (q == FF_STEPS - 1) ff_renorm(ah[r], al[r]);
       }
     }
   }
@@ -1683,10 +1684,6 @@ __device__ __forceinline__ void ff_sym_tile(const float4 *tH, const float4 *tH2,
           ff_renorm(gh, gl);
 #pragma unroll
           for (int r = 0; r < R; r++) ff_renorm(ah[r], al[r]);
-        } else if (s % 2 == 1) {
-          ff_renorm<3>(gh, gl);
-#pragma unroll
-          for (int r = 0; r < R; r++) ff_renorm<3>(ah[r], al[r]);
         }
         const int src = (lane + 1) & 31;
 #pragma unroll
