@@ -44,3 +44,21 @@ def test_far_from_the_origin(nb, n, sym, equal):
     assert (np.linalg.norm(acc - oa, axis=1) <= bound).all()
     bound = (mass / r2).sum(1) * 2.5e-14 + (mass / r2 ** 0.5).sum(1) * 2.0 ** -43
     assert (np.abs(pot - op) <= bound).all()
+
+
+@pytest.mark.parametrize("equal", [True, False])
+def test_potential_sums_each_pair_once(nb, equal):
+    """Coordinates that float-floats hold exactly leave the error of the sums.  With the
+    sums renormalised at every term its RMS over these draws is 1.66e-15 (1.64e-15 for
+    uneven masses), at every second step 1.82e-15 (1.81e-15)."""
+    err = []
+    for s in range(5):
+        rng = np.random.default_rng(s)
+        pos = rng.integers(-64, 65, (1500, 3)) * 1.0
+        mass = np.ones(1500) if equal else rng.integers(1, 2 ** 20, 1500) * 2.0 ** -20
+        with nb.Simulation(1500, "f64e", eps=64.0) as sim:
+            sim.set_symmetric(1)
+            _, pot = sim.accel(pos, mass)
+        _, op, _ = oracle.accel(pos, mass, 64.0)
+        err.append(np.sqrt((((pot - op) / op) ** 2).mean()))
+    assert np.mean(err) <= 1.74e-15
