@@ -590,9 +590,10 @@ static int batch_step_impl(nbody_batch *b, int64_t nticks) {
       // One block per unit by default: the fixed-point pair sums need the warps
       // of a full SM to hide their latency, and blocks of one unit end soon
       // enough for another pool's ticks on a stream of higher priority to get
-      // their SMs.  Measured with the serving mix (12 s, FP64 and MIXED pools):
-      // 967 Gint/s, FP64 tick p50 106 ms, MIXED 21 ms; a persistent grid of 2
-      // blocks per SM 824, 109, 14; of 4, 721, 86, 27.
+      // their SMs, as long as units are short (R = 1, segments of 2048).  Measured
+      // so with the serving mix (15 s, FP64 and MIXED pools): 1265 Gint/s, FP64
+      // ticks 103 ms (p50), MIXED 14 ms (p50) and 20 ms (p99); a persistent grid of
+      // 2 blocks per SM 1066, 230, 16 and 31; of 3, 913, 154, 23 and 60.
       BCK(nb::launch_force_units(NBODY_FP64, b->F, nullptr, nullptr, b->d_units[tb], b->n64,
                                  b->r_mode[0], b->part, (int64_t)b->fp64_per_sm * b->sms, b->st));
       if (b->prof) BCK(cudaEventRecord(e[3], b->st));

@@ -159,10 +159,18 @@ class Batch:
 
 
 class Autotuner:
-    """Chooses (ipt, seg) per (mode, load bucket) from measured ns per interaction."""
+    """Chooses (ipt, seg) per (mode, load bucket) from measured ns per interaction.
+
+    Without `candidates`, FP64 is offered short units alone.  Its pair sums keep the
+    multiply pipe that MIXED needs as well, and a MIXED tick's kernels wait for FP64
+    blocks to end whatever their stream's priority: with units of up to 4 x 8192 pairs
+    a thread among the candidates, the serving mix (16 FP64 and 64 MIXED simulations)
+    ran at 924 Gint/s with MIXED ticks of 22 ms (p50) and 55 ms (p99); with 1 x 2048
+    alone 1265 Gint/s, 14 and 20 ms, with 2 x 2048 1212, 16 and 21."""
 
     def __init__(self, candidates=None, trials=1, recheck_every=64):
         self.candidates = candidates or [(ipt, seg) for ipt in (2, 1, 4) for seg in (8192, 2048)]
+        self._fp64 = candidates or [(1, 2048), (2, 2048)]
         self.trials = trials
         self.recheck_every = recheck_every
         self.stats = collections.defaultdict(lambda: collections.defaultdict(list))
@@ -173,22 +181,25 @@ class Autotuner:
         """Load bucket: the mode and the tick's interactions to within a factor of 8."""
         return (mode, int(math.log2(max(interactions, 1.0)) // 3))
 
+    def _offered(self, key):
+        return self._fp64 if key[0] == "fp64" else self.candidates
+
     def choose(self, key):
         st = self.stats[key]
-        for c in self.candidates:                 # explore: every candidate `trials` times
+        for c in self._offered(key):              # explore: every candidate `trials` times
             if len(st[c]) < self.trials:
                 return c
         self.picks[key] += 1
         best = self.best(key)
         if self.recheck_every and self.picks[key] % self.recheck_every == 0:
-            ranked = sorted(self.candidates, key=lambda c: np.median(st[c]))
+            ranked = sorted(self._offered(key), key=lambda c: np.median(st[c]))
             return ranked[1] if len(ranked) > 1 else best   # re-measure the runner-up
         return best
 
     def best(self, key):
         st = self.stats[key]
-        tried = [c for c in self.candidates if st[c]]
-        return min(tried, key=lambda c: np.median(st[c])) if tried else self.candidates[0]
+        tried = [c for c in self._offered(key) if st[c]]
+        return min(tried, key=lambda c: np.median(st[c])) if tried else self._offered(key)[0]
 
     def record(self, key, cand, ns_per_interaction):
         lst = self.stats[key][cand]
@@ -219,7 +230,7 @@ class _Pool:
         self.mode = mode
         self.kernel = kernel or mode       # the batch mode the pool's simulations run in
         # MIXED ticks are short: give their stream priority so that their blocks are
-        # scheduled as soon as an SM has room next to the long FP64 blocks
+        # scheduled as soon as an SM has room next to the FP64 blocks
         self.stream = torch.cuda.Stream(priority=-1 if mode == "mixed" else 0)
         self.batch = Batch(capacity, max_sims, stream=self.stream)
         self.batch.profile(True)
@@ -236,9 +247,9 @@ class Server:
     """Admit / tick / retire loop with one resident pool per precision mode.
 
     FP64 and MIXED simulations live in separate pools, each ticking on its own
-    CUDA stream: an FP64 tick is bound by the FP64 pipe and a MIXED tick by
-    FP32 issue, so the two run side by side on the same SMs, and the fast
-    MIXED ticks do not wait for the slow FP64 ones.  Each pool admits queued
+    CUDA stream, the MIXED one at the higher priority: the two run side by side
+    on the same SMs, and a fast MIXED tick waits for the FP64 blocks that hold
+    its SMs, not for the slow FP64 ticks.  Each pool admits queued
     requests of its mode between its own ticks (first fit by free range and
     slot, with a look-ahead past requests that do not fit yet).
 
@@ -254,7 +265,7 @@ class Server:
         max_sims: resident simulations per pool, an int or {mode: int}; fp64_kernel:
         "fp64" (binary64 FP64 pipe) or "f64e" (binary64-class float-float on the FP32
         pipes, within the same parity gate) for requests asking for FP64."""
-        launch = launch or {"fp64": (2, 4096), "mixed": (2, 8192), "f64e": (2, 4096)}
+        launch = launch or {"fp64": (1, 2048), "mixed": (2, 8192), "f64e": (2, 4096)}
         split = split or {m: 1.0 / len(modes) for m in modes}
         cap = capacity if isinstance(capacity, dict) else {m: max(1, int(capacity * split[m])) for m in modes}
         ms = max_sims if isinstance(max_sims, dict) else {m: max_sims for m in modes}

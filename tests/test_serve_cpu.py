@@ -62,3 +62,19 @@ def test_poisson_requests(serve):
     assert 0.45 < np.mean([r.eps == 0.02 for r in reqs]) < 0.55   # disk + halo half of the time
     p, v, m = reqs[0].make()
     assert p.shape == (reqs[0].n, 3) and m.shape == (reqs[0].n,)
+
+
+def test_autotuner_offers_fp64_short_units(serve):
+    """Long FP64 units hold the SMs that another pool's ticks wait for; candidates given
+    by the caller hold for every mode."""
+    t = serve.Autotuner()
+    for mode, want in (("fp64", {(1, 2048), (2, 2048)}),
+                       ("mixed", {(i, s) for i in (1, 2, 4) for s in (2048, 8192)})):
+        key, seen = serve.Autotuner.bucket(mode, 1e12), set()
+        for k in range(200):
+            c = t.choose(key)
+            seen.add(c)
+            t.record(key, c, 1.0 + c[0] + c[1] * 1e-4)
+        assert seen == want and t.best(key) == (1, 2048)
+    given = serve.Autotuner(candidates=[(4, 8192)])
+    assert given.choose(serve.Autotuner.bucket("fp64", 1e12)) == (4, 8192)
