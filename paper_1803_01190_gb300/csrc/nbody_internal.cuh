@@ -193,7 +193,8 @@ int diag_blocks(int64_t n);
 
 // Spatial (Morton) order of the particles (order.cu).  launch_spatial_order
 // writes perm (sorted position -> input index) and sposm[s] = posm[perm[s]],
-// using `scratch` of order_scratch_bytes(n).  Its kernel launches: at most 4.
+// using `scratch` of order_scratch_bytes(n).  Three kernels of its own (box, keys
+// or sorted chunks, gather), above 65536 particles those of a radix sort between.
 size_t order_scratch_bytes(int64_t n);
 cudaError_t launch_spatial_order(const d4 *posm, int64_t n, void *scratch, int32_t *perm,
                                  d4 *sposm, cudaStream_t st);

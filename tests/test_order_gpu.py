@@ -62,3 +62,13 @@ def test_tied_coordinates(nb, mode, tol, kind):
     assert err.max() <= 80 * (2.0 ** -24 if mode == "mixed" else 2.0 ** -48)
     assert np.sqrt(np.mean(err ** 2)) <= tol
     assert np.abs(pot / op - 1).max() <= 10 * tol
+
+
+@pytest.mark.parametrize("n", [300, 65536, 65537])
+def test_launches_counted(nb, n):
+    """One evaluation: pack, the order's own three kernels, prep, force, sums out."""
+    pos, _, mass = nbody_ics.plummer(n, 3)
+    with nb.Simulation(n, "mixed", eps=0.05) as sim:
+        before = sim.launch_count
+        sim.accel(pos, mass)
+        assert sim.launch_count - before == 7
