@@ -290,15 +290,25 @@ static int force_sym(nbody_ctx *c, const void *posm_in, int &S) {
   return NBODY_OK;
 }
 
-static int ensure_order(nbody_ctx *c) {
-  if (c->perm) return NBODY_OK;
-  if (cudaMalloc(&c->ord_scratch, nb::order_scratch_bytes(c->n)) != cudaSuccess ||
-      cudaMalloc(&c->perm, sizeof(int32_t) * c->n) != cudaSuccess ||
-      cudaMalloc(&c->sposm, sizeof(d4) * c->n) != cudaSuccess) {
+// Allocates *p unless an earlier call has: a set of buffers whose allocation
+// failed half-way is completed by the next call instead of being taken for whole.
+template <class T>
+static bool ensure_buffer(T *&p, size_t bytes) {
+  if (p) return true;
+  void *q = nullptr;
+  if (cudaMalloc(&q, bytes) != cudaSuccess) {
     cudaGetLastError();
-    return fail(NBODY_ENOMEM, "spatial order buffers");
+    return false;
   }
-  return NBODY_OK;
+  p = (T *)q;
+  return true;
+}
+
+static int ensure_order(nbody_ctx *c) {
+  if (ensure_buffer(c->ord_scratch, nb::order_scratch_bytes(c->n)) &&
+      ensure_buffer(c->perm, sizeof(int32_t) * c->n) && ensure_buffer(c->sposm, sizeof(d4) * c->n))
+    return NBODY_OK;
+  return fail(NBODY_ENOMEM, "spatial order buffers");
 }
 
 static int force_sums(nbody_ctx *c, const void *posm_in, int &S);
@@ -711,12 +721,9 @@ static int step_fr4(nbody_ctx *c, double dt, int64_t nsteps) {
 }
 
 static int step_rk4(nbody_ctx *c, double dt, int64_t nsteps) {
-  if (!c->rk_vs) {
-    const size_t b4 = (size_t)c->n * r4(c);
-    if (cudaMalloc(&c->rk_vs, b4) != cudaSuccess || cudaMalloc(&c->rk_sr, b4) != cudaSuccess ||
-        cudaMalloc(&c->rk_sv, b4) != cudaSuccess)
-      return fail(NBODY_ENOMEM, "RK4 stage buffers");
-  }
+  const size_t b4 = (size_t)c->n * r4(c);
+  if (!ensure_buffer(c->rk_vs, b4) || !ensure_buffer(c->rk_sr, b4) || !ensure_buffer(c->rk_sv, b4))
+    return fail(NBODY_ENOMEM, "RK4 stage buffers");
   const int stg = 1 - c->cur;
   for (int64_t k = 0; k < nsteps; k++) {
     for (int stage = 1; stage <= 4; stage++) {
