@@ -44,9 +44,9 @@ EPS, DT = 0.02, 5e-4
 # the pipe that binds is the FMA-heavy one.
 FP64_INSTR_PER_INTERACTION = {False: 9, True: 6}
 # FMA-heavy pipe cycles per warp and interaction of the fixed-point kernels,
-# equal masses, by ncu (sm__pipe_fmaheavy_cycles_active): 263 one-sided (N =
-# 16384); each pair once 268 per pair (N = 32768).
-FX_HEAVY_CYCLES_PER_INTERACTION = {False: 263, True: 134}
+# equal masses, by ncu (sm__pipe_fmaheavy_cycles_active): 266 one-sided (N =
+# 16384); each pair once 265 per pair (N = 32768).
+FX_HEAVY_CYCLES_PER_INTERACTION = {False: 266, True: 133}
 # FP32 FMA-pipe lane operations: mixed 13 (3 differences, 3 FMAs for
 # |d|^2 + eps^2, m y, y^2, m y^3, 3 FMAs and 1 add into the sums; two j per
 # packed instruction; 12 in tiles of equal masses, this workload's); F64E
@@ -66,8 +66,8 @@ TRAFFIC = {"k_force_f64": {"bytes": 47.05e6 + 62.96e6, "n": 2 ** 20, "src_sha": 
            # launch on the 4096 diagonal blocks + 2048 block diagonals in launches of 5 (pair
            # kernel and combine); bytes of the first launch of each kernel in one full-size
            # capture, the pair and combine launches scaled by 2048 / 5
-           "k_force_f64_sym": {"bytes": 34.01e6 + 2048 / 5 * (433.28e6 + 384.12e6), "n": 2 ** 20,
-                               "src_sha": "29bfce536ae80db9"}}
+           "k_force_f64_sym": {"bytes": 34.19e6 + 2048 / 5 * (427.33e6 + 384.13e6), "n": 2 ** 20,
+                               "src_sha": "e75974de50ed64c7"}}
 
 
 def _kernel_src_sha(names):
@@ -401,7 +401,7 @@ def run_gpu(args):
                    "parallelism": "replicas" if world > 1 else "single GPU",
                    "launch": {**fp64["sim"].get_launch(), "each_pair_once": sym}},
         "p50_step_ms": float(np.percentile(per, 50)), "p99_step_ms": float(np.percentile(per, 99)),
-        "roofline": roofline_fp64(n, sym, fms, ms64, pipes),
+        "roofline": roofline_fixed(n, sym, fms, ms64, pipes),
         "gpu_launches": fp64["launches"] * world,
         "clocks": fp64["clocks"],
         "e2e": {"value": world * inter / e2e64["sec"] / 1e9, "unit": UNIT,
@@ -457,32 +457,45 @@ def run_gpu(args):
 
 
 def roofline_fp64(n, sym, force_ms, step_ms, pipes):
-    """The binary64 force path against the FP64 pipe: achieved = the FP64
-    instructions per interaction of the binary64 pair body x N^2 / the force
-    evaluation's CUDA-event time; peak = the DFMA issue rate measured in the
-    same run.  The fixed-point kernels do not issue them, so the fraction may
-    exceed 1: `integer_pipe` is the pipe that binds those."""
+    """The binary64 pair body against the FP64 pipe, its bound: achieved = its FP64
+    instructions per interaction x N^2 / the force evaluation's CUDA-event time;
+    peak = the DFMA issue rate measured in the same run.  For the softened
+    workload, summed in fixed point (roofline_fixed), this is the rate in terms
+    of the binary64 body and may exceed the peak."""
     inter = float(n) * n
     ipi = FP64_INSTR_PER_INTERACTION[sym]
     achieved = inter * ipi / (force_ms * 1e-3) / 1e9
     conv = inter * FLOP_PER_INTERACTION / (force_ms * 1e-3) / 1e12
-    heavy = FX_HEAVY_CYCLES_PER_INTERACTION[sym]
-    heavy_peak = 4 * pipes["sms"] * pipes["sm_mhz"] / 1e3
-    heavy_achieved = inter / 32 * heavy / (force_ms * 1e-3) / 1e9
-    return {"bound": "alu", "pipe": "fp64", "kernel": "k_force_fx_sym" if sym else "k_force_f64",
-            "integer_pipe": {
-                "pipe": "fma heavy", "cycles_per_warp_interaction": heavy, "achieved": heavy_achieved,
-                "peak": heavy_peak, "unit": "G pipe cycles/s", "frac": heavy_achieved / heavy_peak,
-                "note": "fixed-point pair sums: 32 x 32 -> 64 products of 4 cycles a warp; peak = "
-                        "4 sub-partitions x SMs x the SM clock of this run"},
+    return {"bound": "alu", "pipe": "fp64", "kernel": "k_force_f64_sym" if sym else "k_force_f64",
             "achieved": achieved, "peak": pipes["dfma_ginstr_s"], "unit": "G FP64-pipe instr/s",
             "frac": achieved / pipes["dfma_ginstr_s"],
-            "frac_note": "FP64 instructions that the binary64 pair body would issue; the fixed-point "
-                         "kernels do not issue them and are bound by the pipe of integer_pipe",
             "peak_source": (f"measured in this run: nbody_measure_pipes DFMA issue rate "
                             f"({pipes['dfma_per_clk_sm']:.3f}/clk/SM x {pipes['sms']:.0f} SMs at "
                             f"{pipes['sm_mhz']:.0f} MHz)"),
             "instr_per_interaction": ipi,
+            "convention_20flop": {"achieved": conv, "peak": 2 * pipes["dfma_ginstr_s"] / 1e3,
+                                  "unit": "TFLOP/s", "frac": conv / (2 * pipes["dfma_ginstr_s"] / 1e3),
+                                  "note": "20 flop/interaction x N^2 against 2 flop per measured DFMA; "
+                                          + ("each pair is evaluated once for both particles, so this "
+                                             "can exceed 1" if sym else "")},
+            "force_ms_per_launch": force_ms, "force_ms_note": "one force evaluation (all its launches)",
+            "force_share_of_step": force_ms / step_ms}
+
+
+def roofline_fixed(n, sym, force_ms, step_ms, pipes):
+    """The fixed-point pair sums of the softened binary64 mode against the pipe that
+    binds them: achieved = FMA-heavy pipe cycles per warp and interaction x N^2 / 32 /
+    force time; peak = one cycle per sub-partition and clock at this run's SM clock."""
+    inter = float(n) * n
+    heavy = FX_HEAVY_CYCLES_PER_INTERACTION[sym]
+    achieved = inter / 32 * heavy / (force_ms * 1e-3) / 1e9
+    peak = 4 * pipes["sms"] * pipes["sm_mhz"] / 1e3
+    return {"bound": "alu", "pipe": "fma heavy", "kernel": "k_force_fx_sym" if sym else "k_force_f64",
+            "achieved": achieved, "peak": peak, "unit": "G FMA-heavy cycles/s", "frac": achieved / peak,
+            "peak_source": (f"4 sub-partitions x {pipes['sms']:.0f} SMs x {pipes['sm_mhz']:.0f} MHz, "
+                            f"measured in this run (nbody_measure_pipes)"),
+            "cycles_per_warp_interaction": heavy,
+            "cycles_note": "by ncu, equal masses: 32 x 32 -> 64 products take 4 cycles a warp",
             "traffic": traffic_f64(n, sym),
             "traffic_note": ("DRAM bytes per force evaluation from one full-size ncu capture: mostly the "
                              "per-diagonal row/column slices of the each-pair-once schedule, O(N^2/256), far "
@@ -490,11 +503,7 @@ def roofline_fp64(n, sym, force_ms, step_ms, pipes):
                              if sym else
                              "DRAM bytes per force evaluation from one full-size ncu capture; the O(N) "
                              "algorithmic bytes (32 B in + partial sums out per particle) mostly stay in L2"),
-            "convention_20flop": {"achieved": conv, "peak": 2 * pipes["dfma_ginstr_s"] / 1e3,
-                                  "unit": "TFLOP/s", "frac": conv / (2 * pipes["dfma_ginstr_s"] / 1e3),
-                                  "note": "20 flop/interaction x N^2 against 2 flop per measured DFMA; "
-                                          + ("each pair is evaluated once for both particles, so this "
-                                             "can exceed 1" if sym else "")},
+            "binary64_body": roofline_fp64(n, sym, force_ms, step_ms, pipes),
             "force_ms_per_launch": force_ms, "force_ms_note": "one force evaluation (all its launches)",
             "force_share_of_step": force_ms / step_ms}
 

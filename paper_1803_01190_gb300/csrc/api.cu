@@ -146,9 +146,10 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
     // N = 131072 at 8, 16 and 24 segments 2449, 2549, 2557; 300000 at 4, 8, 32:
     // 2462, 2543, 2568; 2^20 at 2, 4, 16: 2550, 2556, 2562; one-sided FP64 65536
     // at 8, 16, 32: 128, 131, 132)
-    // (MIXED, whose sums are compensated, and the binary64 modes; FP32's segment
-    // count is part of its rounding and stays a function of n alone: eight waves
-    // of R = 1 or, from a full wave of them, 2)
+    // (MIXED, whose sums are compensated, and the binary64 modes.  FP32's segment
+    // count is part of its rounding, so it does not follow the kernel's registers:
+    // eight waves of a fixed 5, 4, 2 or 1 resident blocks at R = 1, 2, 4, 8, for R =
+    // 1 or, from a full wave of them, 2 by default, whatever R then runs)
     const int64_t slots = (int64_t)c->num_sms * occ;
     s = std::max<int64_t>((8 * slots + bx - 1) / bx,
                           std::min<int64_t>((32 * slots + bx - 1) / bx, smax / 16));
@@ -187,9 +188,13 @@ static int ensure_part(nbody_ctx *c, int S) {
 
 // Smallest n at which the automatic choice evaluates each pair once: 64 blocks
 // of 256 (F64E), and 64 blocks of 384 in FP64 whatever its block size.  With
-// few blocks the diagonals hold too few work items to fill the GPU (measured
-// on GB300 with blocks of 512: 43.6 against 55.9 Gint/s at 32 blocks, N = 2^14;
-// 68.5 against 56.6 at 64 blocks, N = 2^15).
+// few blocks the diagonals hold too few work items to fill the GPU.  The line was
+// drawn for binary64 bodies (blocks of 512: 43.6 against 55.9 Gint/s at N = 2^14,
+// 68.5 against 56.6 at 2^15); for the present kernels it lies high: one-sided
+// against each pair once (ms, equal masses; unequal) FP64 8192 0.61 / 0.60; 0.64 /
+// 0.75, 12000 1.23 / 0.96; 1.29 / 1.28, 20011 3.25 / 2.07; 3.44 / 2.87, 24193 4.66 / 2.85;
+// 4.94 / 4.02, F64E 8192 0.34 / 0.31; 0.35 / 0.34, 16129 1.10 / 0.92; 1.11 / 0.92.
+// nbody_set_symmetric(1) takes each pair once below it.
 static int64_t sym_auto_min_n(int mode) { return mode == NBODY_F64E ? 63 * 256 + 1 : 63 * 384 + 1; }
 
 static int sym_block(const nbody_ctx *c) {

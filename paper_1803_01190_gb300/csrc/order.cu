@@ -13,8 +13,9 @@
 // The order is a deterministic function of the positions alone: the bounding
 // box is an exact min/max (order independent), the key of a particle is the
 // bit interleave of its three 21-bit cell indices in that box, and the sort is
-// stable on (key, input index), so equal keys keep input order.  Results therefore stay bit-reproducible (a resumed run recomputes
-// the same order from the same positions).
+// stable on (key, input index), so equal keys keep input order.  Results
+// therefore stay bit-reproducible (a resumed run recomputes the same order from
+// the same positions).
 //
 // Steps (one force evaluation): bbox partials -> keys -> sort -> gather of the
 // positions into sorted order; the epilogue kernels read the sorted partial
@@ -27,8 +28,7 @@
 // 5.5) where the dozen launches of the radix sort took about 45; a whole mixed
 // evaluation with its copies falls from 202 to 84 us at N = 4096, 336 to 204 at
 // 16387, 2088 to 1905 at 65536.  Chunks of 512 measure the same within 3 %.
-// Above, the radix sort moves fewer bytes than
-// n / 256 searches per particle.
+// Above, the radix sort moves fewer bytes than n / 256 searches per particle.
 #include <cuda_runtime.h>
 
 #include <algorithm>
