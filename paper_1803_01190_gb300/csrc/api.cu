@@ -113,17 +113,17 @@ static void default_shape(nbody_ctx *c, nb::Shape &sh, int r_req, int s_req) {
   sh = nb::Shape();
   sh.bt = nb::force_block_threads(c->mode);
   sh.t = nb::force_tile(c->mode);
-  // measured on GB300 (Gint/s): FP64 R = 1, 2 at N = 65536 131, 127; MIXED R = 1,
-  // 2 at 12000 2067, 1919, at 32768 2485, 2474, at 65536 2548, 2601, at 131072
-  // 2605, 2735 (unequal masses at 16387: 5 % slower at R = 2); FP32 (us, whole
+  // measured on GB300 (Gint/s): FP64 R = 1, 2 at N = 65536 131, 127; FP32 (us, whole
   // evaluation, R = 1, 2, 4) 15000 143, 145, -, 16384 164, 151, 165, 20000 221, 222, 249,
   // 32768 496, 445, 471, 65536 1790, 1606, 1645, 100000 4102, 3978, 4186 (R = 4 leaves
-  // half as many blocks to fill the last wave); F64E keeps enough warps resident
-  // only at R = 2 and below one block per SM at R = 1
+  // half as many blocks to fill the last wave).  MIXED and F64E take R = 2 where
+  // that leaves a block per SM: MIXED R = 1, 2 at 12000 2067, 1919, at 131072 2605,
+  // 2735; between 41000 and 77000 whole evaluations are within 3 % (unequal masses
+  // 1 to 5 % faster at R = 1), but an eighth of the rows takes up to a third longer
+  // at R = 2, for its last wave; F64E keeps enough warps resident only at R = 2
   int r = r_req;
   if (!r) switch (c->mode) {
       case NBODY_FP64: r = 1; break;
-      case NBODY_MIXED: r = c->n < 40000 ? 1 : 2; break;
       case NBODY_FP32: r = c->n < 16384 ? 1 : 2; break;
       default: r = (int64_t)sh.bt * 2 * c->num_sms > c->n ? 1 : 2;
     }
