@@ -531,9 +531,9 @@ __device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, cons
 
 // The binary64 force sum, bound by the FMA-heavy pipe (the wide integer
 // multiplies of fixed.cuh; 89 % busy by ncu at N = 16384), not by the FP64
-// pipe.  Measured on GB300 (force kernel alone, disk + halo of equal masses,
-// N = 65536): 131 Gint/s at R = 1, 127 at R = 2 (122 for unequal masses)
-// against 62 for the binary64 body with its 9 FP64 instructions; the relative
+// pipe.  Measured on GB300 (N = 65536, equal masses): 129 Gint/s at R = 1 (122
+// for unequal masses; before the estimate of close pairs 131, 127 at R = 2)
+// against 63 for the binary64 body with its 9 FP64 instructions; the relative
 // error of the accelerations against binary64 terms with pairwise sums falls
 // from 4.5e-16 to 1.9e-16 (it is the rounding of the tile sums).  R above 2
 // runs in groups of two.
@@ -955,8 +955,8 @@ __device__ __noinline__ F64Both pair_f64_both(double dx, double dy, double dz, d
 // registers, columns in the warp's slots of colw, where a lane owns its j at
 // each step); tiles that fx_scale does not take, or with many such pairs
 // (FX_NEAR), go through the tile loop of k_force_f64_sym.  Measured
-// (whole force evaluation, N = 65536): 215-219 Gint/s for equal masses, where
-// the two sides share their terms, 147 for lognormal masses, against 93 for
+// (whole force evaluation, N = 65536): 229 Gint/s for equal masses, where
+// the two sides share their terms, 155 for lognormal masses, against 92 for
 // k_force_f64_sym; relative error of the accelerations 1.6e-16 against 2.6e-16.
 // Four blocks of 128 per SM (128 registers, R = 2): 202 at 166 registers and
 // three blocks, 214 at R = 1, 175 at R = 3.
