@@ -393,35 +393,48 @@ __device__ __forceinline__ void fx_box_join(FxBox &b, const FxBox &o) {
 
 // Unit exponent L and mass exponent em for the i's of box bi against the j's
 // of box bj; ok = false: the fixed-point form does not apply (non-finite
-// values, negative masses, positive masses over a range above
-// 2^FX_MASS_RANGE, extreme exponents, or eps = 0).  eps = 0 stays in
-// binary64: there every pair term is specified to the ulp of the binary64
-// operations.  wide: the masses need exponents of their own.
+// values, negative masses, masses over too wide a range, extreme exponents, or
+// eps = 0).  eps = 0 stays in binary64: there every pair term is specified to
+// the ulp of the binary64 operations.  range: exponents that the positive masses
+// span; gap: exponents that the box lies below eps (an upper bound: where the
+// upper words of the coordinates do not tell, far from the origin, as many as
+// rule unequal masses out).  Both take digits from the terms of light masses, so
+// they share FX_MASS_RANGE (fx_masses_fit): with eps at 2^6 times the system's
+// size a force on the heaviest of masses over 2^8 was off by 1.3e-14 of its terms'
+// magnitudes without the gap.  Equal masses lose nothing by it that pairs too
+// close for the unit do not cover.
 struct FxScale {
-  int L, em;
-  bool ok, wide;
+  int L, em, range, gap;
+  bool ok;
 };
-// em of a box's masses; false: outside the rule above
-__device__ __forceinline__ bool fx_mass_scale(const FxBox &b, int &em, bool &wide) {
+__device__ __forceinline__ bool fx_masses_fit(int range, int gap) {
+  return range == 0 || range + gap <= FX_MASS_RANGE;
+}
+// em and range of a box's masses; false: outside the rule above whatever the gap
+__device__ __forceinline__ bool fx_mass_scale(const FxBox &b, int &em, int &range) {
   const int ex = b.mmax >> 20;
   em = b.mmax == 0 ? 0 : ex - 1023;
-  wide = b.mmax != 0 && (b.mmin >> 20) < ex - FX_MASS_NARROW;
-  return b.mmin >= 0 &&
-         (b.mmax == 0 || (ex > 623 && ex < 1423 && (b.mmin >> 20) >= ex - FX_MASS_RANGE));
+  range = b.mmax == 0 ? 0 : ex - (b.mmin >> 20);
+  return b.mmin >= 0 && (b.mmax == 0 || (ex > 623 && ex < 1423));
 }
 __device__ __forceinline__ FxScale fx_scale(const FxBox &bi, const FxBox &bj, double eps2) {
-  int top = ((__double2hiint(eps2) >> 20) - 1021) >> 1;  // eps < 2^top
+  const int te = ((__double2hiint(eps2) >> 20) - 1021) >> 1;  // eps < 2^te
+  int tb = -1023, far = 0;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     // bounds of the coordinate: the low words of the keys are unknown
     const int l = fx_key(min(bi.lo[c], bj.lo[c])), h = fx_key(max(bi.hi[c], bj.hi[c]));
     const double lo = __hiloint2double(l, l < 0 ? -1 : 0), hi = __hiloint2double(h, h < 0 ? 0 : -1);
-    top = max(top, (__double2hiint(hi - lo) >> 20) - 1022);  // hi - lo < 2^top
+    tb = max(tb, (__double2hiint(hi - lo) >> 20) - 1022);  // hi - lo < 2^tb
+    far = max(far, max(l & 0x7FFFFFFF, h & 0x7FFFFFFF));
   }
+  const int top = max(tb, te);
   FxScale f;
   f.L = top - FX_BITS;
-  const bool m = fx_mass_scale(bj, f.em, f.wide);
-  f.ok = m && eps2 > 0.0 && bi.mmin >= 0 && top > -200 && top < 200;
+  // an upper word is worth less than 2^(far's exponent - 1042)
+  f.gap = tb > (far >> 20) - 1040 ? max(te - tb + 1, 0) : FX_MASS_RANGE;
+  f.ok = fx_mass_scale(bj, f.em, f.range) && fx_masses_fit(f.range, f.gap) && eps2 > 0.0 &&
+         bi.mmin >= 0 && top > -200 && top < 200;
   return f;
 }
 __device__ __forceinline__ double fx_exp2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
@@ -597,6 +610,7 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
       const FxScale sc = fx_scale(bi, bj, eps2);
       const int k0 = cnt * jw / IW, k1 = cnt * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
+      const bool wide = sc.range > FX_MASS_NARROW;  // the masses need exponents of their own
       bool fixed = sc.ok, equal = false;
       const double m0 = tile[0].w;
       uint64_t Xi[RI][3];
@@ -613,7 +627,7 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
         load_i(0);
         const bool near = fx_near(X, Xi[0]) && (tid ^ 16) < cnt;
         const uint32_t mh = (uint32_t)__double2hiint(pj.w), ml = (uint32_t)__double2loint(pj.w);
-        const FxMass M = sc.wide ? fx_mass<true>(mh, ml, sc.em) : fx_mass<false>(mh, ml, sc.em);
+        const FxMass M = wide ? fx_mass<true>(mh, ml, sc.em) : fx_mass<false>(mh, ml, sc.em);
         txy[tid] = make_uint4((uint32_t)X[0], (uint32_t)(X[0] >> 32), (uint32_t)X[1],
                               (uint32_t)(X[1] >> 32));
         tzm[tid] = make_uint4((uint32_t)X[2], (uint32_t)(X[2] >> 32), M.l, M.h);
@@ -626,10 +640,10 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
         // FX_SELF in the split shape alone, where such tiles are a large share
         // (N = 4096: 139 us against 147); elsewhere one more form of the loop
         // made the others slower (N = 20011: 3.54 ms against 3.35)
-        const FxMode mode = sc.wide || (diag && IW == 1) ? FX_WIDE
-                            : diag                       ? FX_SELF
-                            : equal                      ? FX_EQUAL
-                                                         : FX_NARROW;
+        const FxMode mode = wide || (diag && IW == 1) ? FX_WIDE
+                            : diag                    ? FX_SELF
+                            : equal                   ? FX_EQUAL
+                                                      : FX_NARROW;
         const int em = mode == FX_EQUAL ? FX_EQ_EM : sc.em;
         const FxEps e2 = fx_eps2(eps2, sc.L);
         double fs = fx_exp2(fx_force_exp(sc.L, em) + 32), ps = fx_exp2(fx_pot_exp(sc.L, em) + 32);
@@ -1076,8 +1090,8 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
 #pragma unroll
   for (int w = 0; w < NW; w++) fx_box_join(bi, sbox[w]);
   int emi;
-  bool widei;
-  const bool oki = fx_mass_scale(bi, emi, widei);
+  int rangei;
+  const bool oki = fx_mass_scale(bi, emi, rangei);
   const double mi0 = posm[i0].w;
   bool equali = i0 + B <= n;
 #pragma unroll
@@ -1103,9 +1117,9 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
 #pragma unroll
     for (int w = 0; w < NW; w++) fx_box_join(bj, sbox[w]);
     const FxScale sc = fx_scale(bi, bj, eps2);
-    const bool wide = sc.wide || widei;
+    const bool wide = max(sc.range, rangei) > FX_MASS_NARROW;
     const double mj0 = tile[0].w;
-    bool fixed = sc.ok && oki, equal = false;
+    bool fixed = sc.ok && oki && fx_masses_fit(rangei, sc.gap), equal = false;
     uint64_t Xi[R][3];
     FxMass Mi[R];
     if (fixed) {

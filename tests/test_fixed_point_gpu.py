@@ -234,3 +234,23 @@ def test_far_particles(nb, extent, equal, n, sym):
         sim.set_symmetric(sym)
         acc, pot = sim.accel(pos, mass)
     _check(pos, mass, eps, acc, pot)
+
+
+# A softening above the system's size and a spread of masses take digits from the same
+# terms.  No more is lost than binary64 terms may lose: 2 of 3 roundings (2^-53 each) of a
+# term and as much again for the additions of a hundred of them
+@pytest.mark.parametrize("bits", [1, 3, 5, 8])
+@pytest.mark.parametrize("size", [2.0 ** -2, 2.0 ** -5, 2.0 ** -7, 2.0 ** -9])
+@pytest.mark.parametrize("offset", [0.0, 2.0 ** 20])
+@pytest.mark.parametrize("n,sym", [(100, 0), (300, 1)])
+def test_masses_below_a_large_softening(nb, bits, size, offset, n, sym):
+    rng = np.random.default_rng(bits)
+    pos = offset * size + size * rng.standard_normal((n, 3))
+    mass = np.full(n, 2.0 ** -bits)
+    mass[n // 2] = 1.0
+    with nb.Simulation(n, "fp64", eps=1.0) as sim:
+        sim.set_symmetric(sym)
+        acc, pot = sim.accel(pos, mass)
+    _check(pos, mass, 1.0, acc, pot)
+    oa, _, smag = oracle.accel(pos, mass, 1.0)
+    assert (np.linalg.norm(acc - oa, axis=1) <= 2.0 ** -50 * smag).all()
