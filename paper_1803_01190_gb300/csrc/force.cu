@@ -1340,13 +1340,16 @@ __device__ __forceinline__ void two_sum1(float a, float b, float &s, float &e) {
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// Exact binary32 -> binary64 by integer moves (zero and subnormal inputs give
-// 0, which is far below the precision of any value they are added to).
+// Exact binary32 -> binary64 by integer moves, for finite values (subnormal ones
+// are brought up by 2^24 first: the sums of small masses at large distances are
+// made of them).
 __device__ __forceinline__ double f2d_exact(float f) {
-  const unsigned b = __float_as_uint(f);
+  const bool sub = fabsf(f) < 0x1p-126f;
+  const unsigned b = __float_as_uint(sub ? __fmul_rn(f, 0x1p24f) : f);
   const unsigned mag = b & 0x7fffffffu;
-  if (mag < 0x00800000u) return 0.0;
-  return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
+  if (mag == 0) return 0.0;
+  const unsigned shift = sub ? 0x38000000u - 0x01800000u : 0x38000000u;
+  return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + shift)), (int)(b << 29));
 }
 
 // x = h + l in floats: h to nearest, l = the rest rounded to 24 bits.  The
@@ -1370,14 +1373,10 @@ __device__ __forceinline__ void split_ff(double x, float &h, float &l) {
     l = __double2float_rn(x - (double)h);
   }
 }
-// h + l in binary64 (non-finite and subnormal halves by conversion, which keeps
-// them; a half of zero is exact either way)
-__device__ __forceinline__ bool is_normal_or_0(float x) {
-  return (__float_as_uint(x) & 0x7FFFFFFFu) - 0x00800000u < 0x7F000000u || x == 0.0f;
-}
+// h + l in binary64 (non-finite halves by conversion, which keeps them so)
 __device__ __forceinline__ double join_ff(float h, float l) {
-  return is_normal_or_0(h) && is_normal_or_0(l) ? f2d_exact(h) + f2d_exact(l)
-                                                : (double)h + (double)l;
+  const bool finite = fabsf(h) < INFINITY && fabsf(l) < INFINITY;
+  return finite ? f2d_exact(h) + f2d_exact(l) : (double)h + (double)l;
 }
 
 // -(x - c) of an i-particle against a tile's anchor c, exact but for the split:

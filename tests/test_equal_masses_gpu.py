@@ -93,3 +93,19 @@ def test_mixed_subnormal_forces(nb, n, equal):
     assert 1e-40 < np.abs(oa).max() < 2.0 ** -126
     assert (np.abs(acc - oa) <= 4 * n * 2.0 ** -150 + 1e-5 * np.abs(oa).max()).all()
     assert (np.abs(pot - op) <= 4 * n * 2.0 ** -150 + 1e-5 * np.abs(op)).all()
+
+
+@pytest.mark.parametrize("n", [25, 300, 1200])
+@pytest.mark.parametrize("sym", [0, 1])
+def test_f64e_small_masses(nb, n, sym):
+    """Sums near and below binary32's normal numbers: m / r^3 >= 2.6e-38 is off by up to
+    2^-149 in each of its two products and its low part, which is what bounds the forces."""
+    rng = np.random.default_rng(n)
+    pos = 10.0 * rng.standard_normal((n, 3))
+    mass = np.full(n, 4e-32)
+    with nb.Simulation(n, "f64e", eps=100.0) as sim:
+        sim.set_symmetric(sym)
+        acc, pot = sim.accel(pos, mass)
+    oa, op, smag = oracle.accel(pos, mass, 100.0)
+    assert (np.linalg.norm(acc - oa, axis=1) <= 3 * 2.0 ** -149 / 2.6e-38 * smag).all()
+    assert (np.abs(pot - op) <= 1e-12 * np.abs(op)).all()
