@@ -66,8 +66,8 @@ TRAFFIC = {"k_force_f64": {"bytes": 47.05e6 + 62.96e6, "n": 2 ** 20, "src_sha": 
            # launch on the 4096 diagonal blocks + 2048 block diagonals in launches of 5 (pair
            # kernel and combine); bytes of the first launch of each kernel in one full-size
            # capture, the pair and combine launches scaled by 2048 / 5
-           "k_force_f64_sym": {"bytes": 34.19e6 + 2048 / 5 * (427.33e6 + 384.13e6), "n": 2 ** 20,
-                               "src_sha": "e75974de50ed64c7"}}
+           "k_force_f64_sym": {"bytes": 34.10e6 + 2048 / 5 * (427.26e6 + 383.90e6), "n": 2 ** 20,
+                               "src_sha": "d5f5921f48200450"}}
 
 
 def _kernel_src_sha(names):

@@ -395,47 +395,57 @@ __device__ __forceinline__ void fx_box_join(FxBox &b, const FxBox &o) {
 // of box bj; ok = false: the fixed-point form does not apply (non-finite
 // values, negative masses, masses over too wide a range, extreme exponents, or
 // eps = 0).  eps = 0 stays in binary64: there every pair term is specified to
-// the ulp of the binary64 operations.  range: exponents that the positive masses
-// span; gap: exponents that the box lies below eps (an upper bound: where the
-// upper words of the coordinates do not tell, far from the origin, as many as
-// rule unequal masses out).  Both take digits from the terms of light masses, so
-// they share FX_MASS_RANGE (fx_masses_fit): with eps at 2^6 times the system's
-// size a force on the heaviest of masses over 2^8 was off by 1.3e-14 of its terms'
-// magnitudes without the gap.  Equal masses lose nothing by it that pairs too
-// close for the unit do not cover.
+// the ulp of the binary64 operations.  range: exponents that the j's positive
+// masses span.  Box: largest extent below 2^box.
 struct FxScale {
-  int L, em, range, gap;
+  int L, em, range, box;
   bool ok;
 };
-__device__ __forceinline__ bool fx_masses_fit(int range, int gap) {
-  return range == 0 || range + gap <= FX_MASS_RANGE;
-}
-// em and range of a box's masses; false: outside the rule above whatever the gap
+// em and range of a box's masses; false: outside the rule whatever their range
 __device__ __forceinline__ bool fx_mass_scale(const FxBox &b, int &em, int &range) {
   const int ex = b.mmax >> 20;
   em = b.mmax == 0 ? 0 : ex - 1023;
   range = b.mmax == 0 ? 0 : ex - (b.mmin >> 20);
   return b.mmin >= 0 && (b.mmax == 0 || (ex > 623 && ex < 1423));
 }
+__device__ __forceinline__ int fx_eps_exp(double eps2) {  // eps < 2^it
+  return ((__double2hiint(eps2) >> 20) - 1021) >> 1;
+}
 __device__ __forceinline__ FxScale fx_scale(const FxBox &bi, const FxBox &bj, double eps2) {
-  const int te = ((__double2hiint(eps2) >> 20) - 1021) >> 1;  // eps < 2^te
-  int tb = -1023, far = 0;
+  FxScale f;
+  f.box = -1023;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     // bounds of the coordinate: the low words of the keys are unknown
     const int l = fx_key(min(bi.lo[c], bj.lo[c])), h = fx_key(max(bi.hi[c], bj.hi[c]));
     const double lo = __hiloint2double(l, l < 0 ? -1 : 0), hi = __hiloint2double(h, h < 0 ? 0 : -1);
-    tb = max(tb, (__double2hiint(hi - lo) >> 20) - 1022);  // hi - lo < 2^tb
-    far = max(far, max(l & 0x7FFFFFFF, h & 0x7FFFFFFF));
+    f.box = max(f.box, (__double2hiint(hi - lo) >> 20) - 1022);
   }
-  const int top = max(tb, te);
-  FxScale f;
+  const int top = max(f.box, fx_eps_exp(eps2));
   f.L = top - FX_BITS;
-  // an upper word is worth less than 2^(far's exponent - 1042)
-  f.gap = tb > (far >> 20) - 1040 ? max(te - tb + 1, 0) : FX_MASS_RANGE;
-  f.ok = fx_mass_scale(bj, f.em, f.range) && fx_masses_fit(f.range, f.gap) && eps2 > 0.0 &&
-         bi.mmin >= 0 && top > -200 && top < 200;
+  f.ok = fx_mass_scale(bj, f.em, f.range) && eps2 > 0.0 && bi.mmin >= 0 && top > -200 && top < 200;
   return f;
+}
+// Do masses over `range` exponents keep their digits in this tile?  Light ones lose
+// some to the heaviest, and all lose some where eps, not the extent, sets the unit
+// (the gap): both count towards FX_MASS_RANGE.  With eps at 2^6 times the system's
+// size a force on the heaviest of masses over 2^8 was off by 1.3e-14 of its terms'
+// magnitudes without the gap.  It is an upper bound; where the upper words of the
+// coordinates do not tell the box's size (far from the origin) it rules unequal
+// masses out.  Equal ones lose nothing by it that the pairs too close for the unit
+// do not cover.
+__device__ __forceinline__ bool fx_masses_fit(int range, const FxScale &f, const FxBox &bi,
+                                              const FxBox &bj, double eps2) {
+  if (range == 0) return true;
+  int far = 0;
+#pragma unroll
+  for (int c = 0; c < 3; c++)
+    far = max(far, max(fx_key(min(bi.lo[c], bj.lo[c])) & 0x7FFFFFFF,
+                       fx_key(max(bi.hi[c], bj.hi[c])) & 0x7FFFFFFF));
+  // an upper word is worth less than 2^(far's exponent - 1042)
+  const int gap =
+      f.box > (far >> 20) - 1040 ? max(fx_eps_exp(eps2) - f.box + 1, 0) : FX_MASS_RANGE;
+  return range + gap <= FX_MASS_RANGE;
 }
 __device__ __forceinline__ double fx_exp2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
 // acc + a 2^e, a the accumulator, scale = 2^(e + 32)
@@ -459,8 +469,8 @@ __device__ __forceinline__ void fx_coords(const d4 &p, int L, uint64_t (&X)[3]) 
 // at 200, 400, 1000; one-sided): never 107, 78, 56; at 1 89, 71, 71; 2 100, 72, 71; 4 106,
 // 76, 71; 8 105, 84, 71; 16 104, 85, 71; each pair once (never: with every pair of a tile
 // out of line) 99, 50, 41; 1 105, 93, 93; 4 115, 93, 93; 8 118, 91, 93; 16 118, 90, 93.
-// The estimate costs a sphere without far particles 2 % one-sided (132.1 -> 129.4;
-// registers, not the work) and nothing each pair once.
+// The estimate costs a sphere without far particles nothing that shows (one-sided
+// 132.1 -> 132.5, each pair once 228.1 -> 228.7).
 constexpr int FX_NEAR = 8;
 __device__ __forceinline__ bool fx_near(const uint64_t (&Xj)[3], const uint64_t (&Xi)[3]) {
   bool near = true;
@@ -544,9 +554,8 @@ __device__ __forceinline__ void fx_tile(const uint4 *txy, const uint4 *tzm, cons
 
 // The binary64 force sum, bound by the FMA-heavy pipe (the wide integer
 // multiplies of fixed.cuh; 89 % busy by ncu at N = 16384), not by the FP64
-// pipe.  Measured on GB300 (N = 65536, equal masses): 129 Gint/s at R = 1 (122
-// for unequal masses; before the estimate of close pairs 131, 127 at R = 2)
-// against 63 for the binary64 body with its 9 FP64 instructions; the relative
+// pipe.  Measured on GB300 (N = 65536, equal masses): 132 Gint/s at R = 1 (123
+// for unequal masses), 127 at R = 2, against 63 for the binary64 body with its 9 FP64 instructions; the relative
 // error of the accelerations against binary64 terms with pairwise sums falls
 // from 4.5e-16 to 1.9e-16 (it is the rounding of the tile sums).  R above 2
 // runs in groups of two.
@@ -611,7 +620,7 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
       const int k0 = cnt * jw / IW, k1 = cnt * (jw + 1) / IW;
       const bool diag = (jt < u.i0 + u.ni) && (jt + cnt > u.i0);
       const bool wide = sc.range > FX_MASS_NARROW;  // the masses need exponents of their own
-      bool fixed = sc.ok, equal = false;
+      bool fixed = sc.ok && fx_masses_fit(sc.range, sc, bi, bj, eps2), equal = false;
       const double m0 = tile[0].w;
       uint64_t Xi[RI][3];
       auto load_i = [&](int g) {
@@ -621,7 +630,7 @@ __global__ void __launch_bounds__(BT) k_force_f64(const d4 *__restrict__ posm, W
           fx_coords(posm[u.i0 + (li < u.ni ? li : 0)], sc.L, Xi[r]);
         }
       };
-      if (sc.ok) {
+      if (fixed) {
         uint64_t X[3];
         fx_coords(pj, sc.L, X);
         load_i(0);
@@ -1117,9 +1126,10 @@ __global__ void __launch_bounds__(BT, 4) k_force_fx_sym(const d4 *__restrict__ p
 #pragma unroll
     for (int w = 0; w < NW; w++) fx_box_join(bj, sbox[w]);
     const FxScale sc = fx_scale(bi, bj, eps2);
-    const bool wide = max(sc.range, rangei) > FX_MASS_NARROW;
     const double mj0 = tile[0].w;
-    bool fixed = sc.ok && oki && fx_masses_fit(rangei, sc.gap), equal = false;
+    const int range = max(sc.range, rangei);
+    const bool wide = range > FX_MASS_NARROW;
+    bool fixed = sc.ok && oki && fx_masses_fit(range, sc, bi, bj, eps2), equal = false;
     uint64_t Xi[R][3];
     FxMass Mi[R];
     if (fixed) {
